@@ -161,14 +161,20 @@ void sort_items_by_cost(const tfeti_ctx* c, std::vector<SolveItem>& items) {
 // Solve work items: elastic subdomains of one shape share the shape's template
 // factor and are grouped R to a CTA so that the items fit one wave of SMs;
 // subdomains with plastic points carry their own factor, one per CTA.
-void build_item_list(tfeti_ctx* c, const std::vector<int>& plastic_count, int R, std::vector<SolveItem>& items) {
+// skip_dg: leave out the elastic subdomains whose shape takes the tensor-core product.
+bool dg_shape(const tfeti_ctx* c, size_t sh) { return sh < c->dg_b_off.size() && c->dg_b_off[sh] >= 0; }
+
+void build_item_list(tfeti_ctx* c, const std::vector<int>& plastic_count, int R, std::vector<SolveItem>& items,
+                     bool skip_dg = false) {
   const int ns = (int)c->h_subs.size();
   items.clear();
+  std::vector<std::vector<int>> by(c->plan.shapes.size());
+  for (int p = 0; p < ns; ++p)
+    if (plastic_count[p] == 0 && !(skip_dg && dg_shape(c, c->h_subs[p].shape))) by[c->h_subs[p].shape].push_back(p);
   for (size_t sh = 0; sh < c->plan.shapes.size(); ++sh) {
     SolveItem it{};
     it.fac = c->tmpl_fac_off[sh];
-    for (int p = 0; p < ns; ++p) {
-      if (plastic_count[p] > 0 || c->h_subs[p].shape != (int)sh) continue;
+    for (int p : by[sh]) {
       it.sub[it.count++] = p;
       if (it.count == R) {
         items.push_back(it);
@@ -192,6 +198,85 @@ void build_item_list(tfeti_ctx* c, const std::vector<int>& plastic_count, int R,
   sort_items_by_cost(c, items);
   sort_items_by_cost(c, own);
   items.insert(items.end(), own.begin(), own.end());
+}
+
+// Rows, blocks and CTAs of the tensor-core FP64 product: the subdomains on their shape's elastic
+// factor, grouped by shape and padded to tiles of kDgM rows.  When the output tiles alone would leave
+// SMs idle, every block's K range is cut into the same number of splits (whole chunks), whose integer
+// results the scatter adds.  Wide shapes come first (the longest CTAs start first).
+void build_dg(tfeti_ctx* c, const std::vector<int>& plastic_count) {
+  c->dg_rows = c->dg_ctas = c->dg_ctas_bd = c->dg_max_n = 0;
+  if (!c->dg_B) return;
+  const Plan& P = c->plan;
+  const int ns = (int)c->h_subs.size();
+  std::vector<std::vector<int>> by(P.shapes.size());
+  for (int p = 0; p < ns; ++p)
+    if (plastic_count[p] == 0 && dg_shape(c, c->h_subs[p].shape)) by[c->h_subs[p].shape].push_back(p);
+  std::vector<int> order;
+  for (size_t sh = 0; sh < by.size(); ++sh)
+    if (!by[sh].empty()) order.push_back((int)sh);
+  std::stable_sort(order.begin(), order.end(), [&P](int a, int b) { return P.shapes[a].n_dof > P.shapes[b].n_dof; });
+  std::vector<DgBlock> blocks;
+  std::vector<DgRow> rows;
+  long long tiles = 0, tiles_bd = 0;
+  for (int sh : order) {
+    DgBlock b{};
+    b.n = (int)P.shapes[sh].n_dof;
+    b.n_bd = 3 * P.shapes[sh].n_bnd;
+    b.nk = dg_nk(b.n);
+    b.nk_bd = dg_nk(b.n_bd);
+    b.rows_pad = ((int)by[sh].size() + kDgM - 1) / kDgM * kDgM;
+    b.b_off = c->dg_b_off[sh];
+    b.b_off_bd = c->dg_b_off_bd[sh];
+    b.sb_off = c->dg_sb_off[sh];
+    b.sb_off_bd = c->dg_sb_off_bd[sh];
+    b.ld = (long long)((b.n + kDgN - 1) / kDgN) * kDgN;
+    b.ld_bd = (long long)((b.n_bd + kDgN - 1) / kDgN) * kDgN;
+    tiles += b.rows_pad / kDgM * (b.ld / kDgN);
+    tiles_bd += b.rows_pad / kDgM * (b.ld_bd / kDgN);
+    for (size_t k = 0; k < by[sh].size(); ++k) rows.push_back({by[sh][k], (int)blocks.size(), (int)k, 0});
+    c->dg_max_n = std::max(c->dg_max_n, b.n);
+    blocks.push_back(b);
+  }
+  if (blocks.empty()) return;
+  std::vector<DgCta> ctas, ctas_bd;
+  const int ch = dg_chunk_stages();
+  auto fill = [&](bool full, long long n_tiles, std::vector<DgCta>& out) {
+    const int want = (int)std::max(1LL, std::min(4LL, c->n_sm / std::max(1LL, n_tiles)));
+    long long a_off = 0, o_off = 0;
+    for (size_t k = 0; k < blocks.size(); ++k) {
+      DgBlock& b = blocks[k];
+      const int nk = full ? b.nk : b.nk_bd, n_ch = (nk + ch - 1) / ch, sp = std::min(want, n_ch);
+      const long long ld = full ? b.ld : b.ld_bd;
+      (full ? b.splits : b.splits_bd) = sp;
+      (full ? b.a_off : b.a_off_bd) = a_off;
+      (full ? b.o_off : b.o_off_bd) = o_off;
+      a_off += dg_a_elems(b.rows_pad, full ? b.n : b.n_bd);
+      for (int z = 0; z < sp; ++z)
+        for (int mt = 0; mt < b.rows_pad / kDgM; ++mt)
+          for (int nt = 0; nt < (int)(ld / kDgN); ++nt) {
+            DgCta q{};
+            q.blk = (int)k;
+            q.mt = mt;
+            q.nt = nt;
+            q.ks0 = z * n_ch / sp * ch;
+            q.ks1 = std::min(nk, (z + 1) * n_ch / sp * ch);
+            q.out_off = o_off + ((long long)z * b.rows_pad + mt * kDgM) * ld + nt * kDgN;
+            q.ld = ld;
+            out.push_back(q);
+          }
+      o_off += (long long)sp * b.rows_pad * ld;
+    }
+  };
+  fill(true, tiles, ctas);
+  fill(false, tiles_bd, ctas_bd);
+  cudaMemcpyAsync(c->d_dg_blocks, blocks.data(), sizeof(DgBlock) * blocks.size(), cudaMemcpyHostToDevice, c->st);
+  cudaMemcpyAsync(c->d_dg_rows, rows.data(), sizeof(DgRow) * rows.size(), cudaMemcpyHostToDevice, c->st);
+  cudaMemcpyAsync(c->d_dg_ctas, ctas.data(), sizeof(DgCta) * ctas.size(), cudaMemcpyHostToDevice, c->st);
+  cudaMemcpyAsync(c->d_dg_ctas_bd, ctas_bd.data(), sizeof(DgCta) * ctas_bd.size(), cudaMemcpyHostToDevice, c->st);
+  c->dg_rows = (int)rows.size();
+  c->dg_ctas = (int)ctas.size();
+  c->dg_ctas_bd = (int)ctas_bd.size();
 }
 
 // Items of the Dirichlet-preconditioner solves: elastic subdomains grouped R to a CTA
@@ -227,11 +312,14 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
   int n_pl = 0;
   for (int v : plastic_count) n_pl += v > 0;
   const int n_el = ns - n_pl;
+  build_dg(c, plastic_count);
   // FP64: one CTA per SM, so at most n_sm items; FP32: two CTAs per SM fit in shared memory
   const int slots64 = std::max(1, c->n_sm - n_pl), slots32 = std::max(1, 2 * c->n_sm - n_pl);
-  const int R64 = std::max(1, std::min((n_el + slots64 - 1) / slots64, c->rcap));
+  const int n_el64 = n_el - c->dg_rows;   // elastic subdomains that keep the banded FP64 sweeps
+  const int R64 = std::max(1, std::min((n_el64 + slots64 - 1) / slots64, c->rcap));
+  const int R64_all = std::max(1, std::min((n_el + slots64 - 1) / slots64, c->rcap));
   const int R32 = std::max(1, std::min((n_el + slots32 - 1) / slots32, c->rcap32));
-  build_item_list(c, plastic_count, R64, c->h_items);
+  build_item_list(c, plastic_count, R64, c->h_items, true);
   build_item_list(c, plastic_count, R32, c->h_items32);
   // for the Schur-block inner F-apply: elastic subdomains per shape, FP32 items of the plastic ones
   c->h_el.clear();
@@ -255,7 +343,9 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
   std::vector<SolveItem> pl, pl64;
   for (const SolveItem& it : c->h_items32)
     if (((it.fac & kOwnFac) && !wood(it.sub[0])) || !uses_schur(c->h_subs[it.sub[0]].shape)) pl.push_back(it);
-  for (const SolveItem& it : c->h_items)
+  std::vector<SolveItem> all;   // the FP64 Schur F-apply has its own split of the banded items
+  build_item_list(c, plastic_count, R64_all, all);
+  for (const SolveItem& it : all)
     if ((it.fac & kOwnFac) || !uses_schur(c->h_subs[it.sub[0]].shape)) pl64.push_back(it);
   c->n_items_pl = (int)pl.size();
   c->n_items_pl64 = (int)pl64.size();
@@ -272,7 +362,7 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
   c->g_inner_stale = true;
   c->lump_stale = true;
   if (c->dirichlet) {
-    build_dir_item_list(c, plastic_count, R64, c->h_items_d);
+    build_dir_item_list(c, plastic_count, R64_all, c->h_items_d);
     build_dir_item_list(c, plastic_count, R32, c->h_items_d32);
     c->n_items_d = (int)c->h_items_d.size();
     c->n_items_d32 = (int)c->h_items_d32.size();
@@ -281,8 +371,9 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
     cudaMemcpyAsync(c->d_items_d32, c->h_items_d32.data(), sizeof(SolveItem) * c->h_items_d32.size(),
                     cudaMemcpyHostToDevice, c->st);
   }
-  cudaMemcpyAsync(c->d_items, c->h_items.data(), sizeof(SolveItem) * c->h_items.size(), cudaMemcpyHostToDevice,
-                  c->st);
+  if (!c->h_items.empty())
+    cudaMemcpyAsync(c->d_items, c->h_items.data(), sizeof(SolveItem) * c->h_items.size(), cudaMemcpyHostToDevice,
+                    c->st);
   cudaMemcpyAsync(c->d_items32, c->h_items32.data(), sizeof(SolveItem) * c->h_items32.size(),
                   cudaMemcpyHostToDevice, c->st);
 }
@@ -375,14 +466,63 @@ void wood_correct_end(tfeti_ctx* c, const SolveArgs& a) {
   c->launches += launch_wood_add64(c->M, c->wood, to_c ? a.cbuf : nullptr, to_d ? a.dst : nullptr, c->st);
 }
 
+// One FP64 pass K^+ x over all subdomains (in_mode 0 or 1): the elastic subdomains of the shapes
+// with digit tiles by one tensor-core product, the others (own factors, shapes without tiles) by the
+// banded sweeps, concurrently on the second stream; the items with own records wait for a deferred
+// refactorisation.  Both write their own subdomains' entries only.
+void fp64_pass(tfeti_ctx* c, const SolveArgs& a) {
+  const bool dg = c->dg_rows > 0, rest = a.n_items > 0;
+  cudaStream_t sb = dg ? c->st2 : c->st;
+  if (dg && rest) {
+    cudaEventRecord(c->ev_fork, c->st);
+    cudaStreamWaitEvent(sb, c->ev_fork, 0);
+  }
+  if (rest && c->fac_pending && c->n_items_el < a.n_items) {
+    SolveArgs e = a;
+    e.n_items = c->n_items_el;
+    launch_sub_solve(c->M, e, c->solve_smem, sb);
+    if (dg) cudaStreamWaitEvent(sb, c->ev_fac_done, 0);   // the context stream joins below, past ev_join
+    else join_factorisation(c);
+    SolveArgs o = a;
+    o.items = a.items + c->n_items_el;
+    o.n_items = a.n_items - c->n_items_el;
+    launch_sub_solve(c->M, o, c->solve_smem, sb);
+    c->launches += 2;
+  } else if (rest) {
+    launch_sub_solve(c->M, a, c->solve_smem, sb);
+    c->launches += 1;
+  }
+  if (dg) {
+    if (rest) cudaEventRecord(c->ev_join, sb);
+    DgArgs d;
+    d.blocks = c->d_dg_blocks;
+    d.rows = c->d_dg_rows;
+    d.n_rows = c->dg_rows;
+    d.full = a.in_mode != 0 || a.out_mode != 0;
+    d.ctas = d.full ? c->d_dg_ctas : c->d_dg_ctas_bd;
+    d.n_ctas = d.full ? c->dg_ctas : c->dg_ctas_bd;
+    d.max_n = c->dg_max_n;
+    d.A = c->dg_A;
+    d.B = c->dg_B;
+    d.sA = c->dg_sA;
+    d.sB = c->dg_sB;
+    d.out = c->dg_out;
+    d.err = c->d_err;
+    const bool to_c = a.out_mode == 0 || a.out_mode == 3, to_d = a.out_mode == 1 || a.out_mode == 3;
+    c->launches += launch_dg_product(c->M, d, a.in_mode == 1 ? a.src : nullptr, a.lam, a.in_mode == 0 ? 1.0 : -1.0,
+                                     to_c ? a.cbuf : nullptr, to_d ? a.dst : nullptr, c->st);
+    if (rest) cudaStreamWaitEvent(c->st, c->ev_join, 0);
+  }
+  join_factorisation(c);
+}
+
 void timed_sub_solve(tfeti_ctx* c, const SolveArgs& a) {
   // subdomains on their elastic factor + Woodbury correction
   const bool corr = wood_correct_begin(c, a);
   cudaEvent_t e1 = timed_begin(c, 0);
-  launch_sub_solve(c->M, a, c->solve_smem, c->st);
+  fp64_pass(c, a);
   if (e1) cudaEventRecord(e1, c->st);
   if (corr) wood_correct_end(c, a);
-  c->launches += 1;
   c->f_launches += 1;
 }
 
@@ -607,9 +747,10 @@ int ensure_schur_bf16(tfeti_ctx* c) {
   return cuda_check(c, "forming BF16 Schur tiles");
 }
 
-// Dense FP64 K^+ (fixing-dof generalised inverse of the elastic template) of every shape with a
-// formed dual Schur block and at most kWoodMaxN dofs, from unit right-hand sides through the FP64
-// banded solve; formed once (a case context shares its base's).  Used by the Woodbury set-up.
+// Dense FP64 K^+ (fixing-dof generalised inverse of the elastic template) of every shape with at
+// least kSchurMinCount subdomains and at most kWoodMaxN dofs, from unit right-hand sides through the
+// FP64 banded solve; formed once (a case context shares its base's).  Used by the Woodbury set-up
+// and by the tensor-core FP64 products.
 int ensure_kinv(tfeti_ctx* c) {
   if (c->kinv) return TFETI_OK;
   if (c->base) {
@@ -622,41 +763,42 @@ int ensure_kinv(tfeti_ctx* c) {
   }
   const Plan& P = c->plan;
   const size_t nsh = P.shapes.size();
+  std::vector<int> count(nsh, 0);
+  for (const SubDev& sd : c->h_subs) ++count[sd.shape];
   std::vector<long long> off(nsh, -1);
+  std::vector<SolveItem> items;
+  std::vector<size_t> first(nsh, 0), num(nsh, 0);
   long long tot = 0;
   for (size_t sh = 0; sh < nsh; ++sh) {
     const int n = (int)P.shapes[sh].n_dof;
-    if (!c->schur_formed[sh] || n > kWoodMaxN) continue;
+    if (count[sh] < kSchurMinCount || n > kWoodMaxN) continue;
     off[sh] = tot;
     tot += (long long)n * n;
-  }
-  double* kinv = nullptr;
-  try {
-    kinv = dalloc<double>(c, (size_t)std::max(1LL, tot));
-    c->d_kinv_off = upload(c, off);
-  } catch (const std::bad_alloc&) {
-    dfree(c, kinv, (size_t)std::max(1LL, tot));
-    return fail(c, TFETI_ERR_OOM, "device allocation failed");
-  }
-  for (size_t sh = 0; sh < nsh; ++sh) {
-    if (off[sh] < 0) continue;
-    const int n = (int)P.shapes[sh].n_dof;
-    std::vector<SolveItem> items;
+    first[sh] = items.size();
     for (int j = 0; j < n; j += c->rcap) {
       SolveItem it{};
       it.fac = c->tmpl_fac_off[sh];
       for (int r = 0; r < c->rcap && j + r < n; ++r) it.sub[it.count++] = j + r;
       items.push_back(it);
     }
-    SolveItem* d_items = nullptr;
-    try {
-      d_items = upload(c, items);
-    } catch (const std::bad_alloc&) {
-      return fail(c, TFETI_ERR_OOM, "device allocation failed");
-    }
+    num[sh] = items.size() - first[sh];
+  }
+  double* kinv = nullptr;
+  SolveItem* d_items = nullptr;
+  try {
+    kinv = dalloc<double>(c, (size_t)std::max(1LL, tot));
+    d_items = upload(c, items);
+    c->d_kinv_off = upload(c, off);
+  } catch (const std::bad_alloc&) {
+    dfree(c, d_items, items.size());
+    dfree(c, kinv, (size_t)std::max(1LL, tot));
+    return fail(c, TFETI_ERR_OOM, "device allocation failed");
+  }
+  for (size_t sh = 0; sh < nsh; ++sh) {
+    if (off[sh] < 0) continue;
     SolveArgs a = solve_args(c);
-    a.items = d_items;
-    a.n_items = (int)items.size();
+    a.items = d_items + first[sh];
+    a.n_items = (int)num[sh];
     a.in_mode = 5;
     a.out_mode = 4;
     a.rep_sub = P.shapes[sh].rep_sub;
@@ -664,12 +806,97 @@ int ensure_kinv(tfeti_ctx* c) {
     a.s_off = off[sh];
     launch_sub_solve(c->M, a, c->solve_smem, c->st);
     c->launches += 1;
-    sync(c);
-    dfree(c, d_items, items.size());
   }
+  sync(c);
+  dfree(c, d_items, items.size());
   c->kinv = kinv;
   c->kinv_off = off;
   return cuda_check(c, "forming dense K^+ blocks");
+}
+
+// Digit tiles of the shapes with a dense K^+ (a case context shares its base's) and this context's
+// work space for the tensor-core FP64 product.  A device without room for them leaves the shapes on
+// the banded sweeps.
+int ensure_digits(tfeti_ctx* c) {
+  if (c->dg_B) return TFETI_OK;
+  const Plan& P = c->plan;
+  const size_t nsh = P.shapes.size();
+  const int ns = (int)c->h_subs.size();
+  if (c->base) {
+    c->dg_b_off = c->base->dg_b_off;
+    c->dg_b_off_bd = c->base->dg_b_off_bd;
+    c->dg_sb_off = c->base->dg_sb_off;
+    c->dg_sb_off_bd = c->base->dg_sb_off_bd;
+    c->dg_sB = c->base->dg_sB;
+    if (!c->base->dg_B) return TFETI_OK;
+  }
+  void* B = c->base ? c->base->dg_B : nullptr;
+  std::vector<int> count(nsh, 0);
+  for (const SubDev& sd : c->h_subs) ++count[sd.shape];
+  std::vector<long long> b_off(nsh, -1), b_off_bd(nsh, -1), sb_off(nsh, -1), sb_off_bd(nsh, -1);
+  long long b_tot = 0, sb_tot = 0, a_tot = 0, o_tot = 0, ctas = 0;
+  for (size_t sh = 0; sh < nsh; ++sh) {
+    const int n = (int)P.shapes[sh].n_dof, n_bd = 3 * P.shapes[sh].n_bnd;
+    if (count[sh] < kSchurMinCount || n > kWoodMaxN) continue;
+    const long long ld = (long long)(n + kDgN - 1) / kDgN * kDgN, ld_bd = (long long)(n_bd + kDgN - 1) / kDgN * kDgN;
+    const int rp = (count[sh] + kDgM - 1) / kDgM * kDgM;
+    b_off[sh] = b_tot;
+    b_off_bd[sh] = b_tot + dg_b_elems(n);
+    b_tot += dg_b_elems(n) + dg_b_elems(n_bd);
+    sb_off[sh] = sb_tot;
+    sb_off_bd[sh] = sb_tot + ld;
+    sb_tot += ld + ld_bd;
+    a_tot += dg_a_elems(rp, n);
+    o_tot += 4LL * rp * ld;     // at most four K splits
+    ctas += 4LL * (rp / kDgM) * (ld / kDgN);
+  }
+  if (b_tot == 0) return TFETI_OK;
+  const size_t keep = c->allocs.size();
+  const size_t keep_bytes = c->bytes;
+  const bool had_kinv = c->kinv != nullptr;
+  try {
+    if (!c->base) {
+      const int st = ensure_kinv(c);
+      if (st == TFETI_ERR_OOM) return TFETI_OK;
+      if (st != TFETI_OK) return st;
+      B = dalloc<uint16_t>(c, (size_t)b_tot);
+      c->dg_sB = dalloc<double>(c, (size_t)sb_tot);
+    }
+    c->dg_A = dalloc<uint16_t>(c, (size_t)a_tot);
+    c->dg_sA = dalloc<double>(c, ns);
+    c->dg_out = dalloc<long long>(c, (size_t)o_tot);
+    c->d_dg_blocks = dalloc<DgBlock>(c, nsh);
+    c->d_dg_rows = dalloc<DgRow>(c, ns);
+    c->d_dg_ctas = dalloc<DgCta>(c, (size_t)ctas);
+    c->d_dg_ctas_bd = dalloc<DgCta>(c, (size_t)ctas);
+  } catch (const std::bad_alloc&) {
+    while (c->allocs.size() > keep) {
+      cudaFree(c->allocs.back());
+      c->allocs.pop_back();
+    }
+    c->bytes = keep_bytes;
+    if (!had_kinv) c->kinv = nullptr;
+    c->dg_b_off.clear();
+    return TFETI_OK;
+  }
+  if (!c->base) {
+    auto* b16 = static_cast<uint16_t*>(B);
+    for (size_t sh = 0; sh < nsh; ++sh) {
+      if (b_off[sh] < 0) continue;
+      const int n = (int)P.shapes[sh].n_dof, n_bd = 3 * P.shapes[sh].n_bnd;
+      launch_dg_split_k(c->M, P.shapes[sh].bnd_off, n, n_bd, true, c->kinv + c->kinv_off[sh], b16 + b_off[sh],
+                        c->dg_sB + sb_off[sh], c->st);
+      launch_dg_split_k(c->M, P.shapes[sh].bnd_off, n, n_bd, false, c->kinv + c->kinv_off[sh], b16 + b_off_bd[sh],
+                        c->dg_sB + sb_off_bd[sh], c->st);
+      c->launches += 2;
+    }
+    c->dg_b_off = b_off;
+    c->dg_b_off_bd = b_off_bd;
+    c->dg_sb_off = sb_off;
+    c->dg_sb_off_bd = sb_off_bd;
+  }
+  c->dg_B = B;
+  return cuda_check(c, "forming the digit tiles");
 }
 
 // Grows a scratch pool (contents not kept) to at least `need` elements, doubling.
@@ -1693,18 +1920,10 @@ void residual_solve(tfeti_ctx* c, const double* f, const double* lam, double* r_
   a.in_mode = 1;
   a.out_mode = 3;
   if (c->fac_pending && c->n_items_el < c->n_items) {
-    // template items while the own records are factorised on st_fac, then the others; such a
-    // split pass is not among the timed F-apply passes (its span includes the factorisation)
-    SolveArgs e = a;
-    e.n_items = c->n_items_el;
-    launch_sub_solve(c->M, e, c->solve_smem, c->st);
-    join_factorisation(c);
-    SolveArgs o = a;
-    o.items = a.items + c->n_items_el;
-    o.n_items = c->n_items - c->n_items_el;
-    launch_sub_solve(c->M, o, c->solve_smem, c->st);
+    // such a pass, whose span includes the rest of a refactorisation on st_fac, is not among the
+    // timed F-apply passes
+    fp64_pass(c, a);
     wood_correct_solve(c, a, c->st);
-    c->launches += 2;
     c->f_split += 1;
   } else {
     join_factorisation(c);
@@ -2580,13 +2799,10 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     long long len = 0;
     for (const ShapeInfo& sh : P.shapes) len = std::max<long long>(len, P.subs[sh.rep_sub].fac_size);
     launch_fac_to_f32(c->fac, c->fac32, dfac, (int)reps.size(), len, c->st);
-    build_items(c, std::vector<int>(ns, 0));
     std::vector<long long> kt;
     for (const ShapeInfo& sh : P.shapes) kt.push_back(sh.kbb_off);
     long long* dkt = upload(c, kt);
     launch_kbb_fill(M, dl, dkt, (int)reps.size(), c->max_bnd, c->elem_np, c->dKe, c->kbb, nullptr, 1, c->st);
-    } else {
-      build_items(c, std::vector<int>(ns, 0));
     }
     for (int p = 0; p < ns; ++p) c->h_kbb_off[p] = c->h_kbb_off32[p] = P.shapes[c->h_subs[p].shape].kbb_off;
     cudaMemcpyAsync(c->d_kbb_off, c->h_kbb_off.data(), sizeof(long long) * ns, cudaMemcpyHostToDevice, c->st);
@@ -2613,6 +2829,11 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     c->ev_pool.push_back(e);
   }
   c->ev_kind.assign(c->ev_pool.size() / 2 + 1, 0);
+  {
+    const int st = ensure_digits(c);
+    if (st != TFETI_OK) return st;
+    build_items(c, std::vector<int>(ns, 0));
+  }
   sync(c);
   return cuda_check(c, "tfeti_setup");
 }
@@ -3353,9 +3574,8 @@ int tfeti_apply_kdag(tfeti_ctx* c, const double* x, double* y) {
   a.dst = y;
   a.in_mode = 1;
   a.out_mode = 1;
-  launch_sub_solve(c->M, a, c->solve_smem, c->st);
+  fp64_pass(c, a);
   wood_correct_solve(c, a, c->st);
-  c->launches += 1;
   sync(c);
   return cuda_check(c, "tfeti_apply_kdag");
 }

@@ -95,6 +95,20 @@ struct tfeti_ctx {
   double* kinv = nullptr;
   std::vector<long long> kinv_off;
   long long* d_kinv_off = nullptr;
+  // FP64 products with the dense K^+ on the tensor cores (kernels_digits.cu): per shape the
+  // offsets of its digit tiles and row scales, full and boundary form (dg_b_off < 0: the shape
+  // keeps the banded sweeps; a case context shares the base's), and this context's rows, CTA lists
+  // and work space.
+  std::vector<long long> dg_b_off, dg_b_off_bd, dg_sb_off, dg_sb_off_bd;
+  void* dg_B = nullptr;
+  double* dg_sB = nullptr;
+  void* dg_A = nullptr;
+  double* dg_sA = nullptr;
+  long long* dg_out = nullptr;
+  tfeti::DgBlock* d_dg_blocks = nullptr;
+  tfeti::DgRow* d_dg_rows = nullptr;
+  tfeti::DgCta *d_dg_ctas = nullptr, *d_dg_ctas_bd = nullptr;
+  int dg_rows = 0, dg_ctas = 0, dg_ctas_bd = 0, dg_max_n = 0;
   std::vector<char> h_wood;                  // per subdomain: on the Woodbury correction
   std::vector<int> h_np_all;                 // plastic points per subdomain at the last assembly
   tfeti::WoodArgs wood;

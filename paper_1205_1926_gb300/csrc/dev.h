@@ -264,6 +264,50 @@ int launch_wood_corr64(const DevMesh& M, const WoodArgs& a, const double* src, c
                        cudaStream_t st);
 int launch_wood_add64(const DevMesh& M, const WoodArgs& a, double* cbuf, double* dst, cudaStream_t st);
 
+// FP64 products with the dense K^+ of a shape on the tensor cores (kernels_digits.cu).  A block is
+// a shape: n dofs, n_bd boundary dofs (the "bd" members describe the product restricted to them,
+// S = (K^+)_{boundary,boundary}), nk stages of 16 columns, rows_pad rows of X (its subdomains, padded
+// to 128).  Offsets: a_off into the digit tiles of X and b_off into those of K^+ (elements), o_off
+// into the integer results (row pitch ld, one set of rows_pad rows per K split), sb_off into the row
+// scales of K^+.
+constexpr int kDgM = 128, kDgN = 64;   // tile of a CTA: rows of X x rows of K^+
+struct DgBlock {
+  int n, n_bd, nk, nk_bd, splits, splits_bd, rows_pad, pad;
+  long long a_off, a_off_bd, b_off, b_off_bd, o_off, o_off_bd, ld, ld_bd, sb_off, sb_off_bd;
+};
+struct DgRow {
+  int sub, blk, local, pad;            // subdomain, its block, its row within the block
+};
+struct DgCta {
+  int blk, mt, nt, ks0, ks1, pad;      // output tile and stages [ks0, ks1) of a CTA
+  long long out_off, ld;
+};
+struct DgArgs {
+  const DgBlock* blocks = nullptr;
+  const DgRow* rows = nullptr;
+  int n_rows = 0, n_ctas = 0, max_n = 0;
+  bool full = false;                   // all dofs (else boundary dofs)
+  const DgCta* ctas = nullptr;
+  void* A = nullptr;
+  const void* B = nullptr;
+  double* sA = nullptr;
+  const double* sB = nullptr;
+  long long* out = nullptr;
+  int* err = nullptr;                  // bit 4 set if a bounded wait gives up
+};
+int dg_nk(int n);                      // stages of 16 columns
+int dg_chunk_stages();                 // K splits are multiples of this many stages
+long long dg_a_elems(int rows_pad, int n);
+long long dg_b_elems(int n);
+// Digit tiles and row scales of one shape's K^+ (full) or S, from its dense kinv (set-up).
+void launch_dg_split_k(const DevMesh& M, long long bnd_off, int n, int n_bd, bool full, const double* kinv, void* B,
+                       double* sB, cudaStream_t st);
+// y = K^+ x of the rows' subdomains.  Boundary form: x = B^T lam, y at the interface slots to cbuf;
+// full form: x = src + sign B^T lam (src, lam nullable), y to dst and, at the copy slots, to cbuf (each
+// nullable).  Returns the number of launches.
+int launch_dg_product(const DevMesh& M, const DgArgs& a, const double* src, const double* lam, double sign, double* cbuf,
+                      double* dst, cudaStream_t st);
+
 // dst[i] = (float) src[i], i < n.
 void launch_to_f32(const double* src, float* dst, long long n, cudaStream_t st);
 // FP32 copies of factor records (offsets in entries, same for both pools)
