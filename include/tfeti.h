@@ -391,7 +391,11 @@ int tfeti_mlp_train(tfeti_ctx* ctx, const double* la, const double* lb, const do
 
 /* How the FP64 F-apply of the PCGP iterations treats subdomains still on their
  * shape's elastic tangent (Sec. 4.2 leaves the K^+ apply open).  BANDED (default):
- * forward and backward substitution with the shape's factor.  SCHUR: one DGEMM per
+ * forward and backward substitution with the shape's factor or, for shapes with at least four
+ * subdomains and at most 3072 dofs, the product with the shape's dense K^+ (formed at set-up from
+ * the same factor) on the tensor cores, both operands split into integer digits so that the
+ * product has FP64 accuracy; the other FP64 K^+ applies (residuals, recovery, tfeti_apply_kdag)
+ * take the same path in either mode.  SCHUR: one DGEMM per
  * shape with the shape's dual Schur block S = (K^+)_{boundary,boundary} (formed once
  * in FP64 from the same factor, 1158^2 doubles for an 8^3 box), which has the same
  * flop count but keeps all SMs busy; subdomains with plastic points keep their

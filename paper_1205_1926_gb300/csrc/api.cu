@@ -2639,6 +2639,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   cudaMemsetAsync(c->d_ctr, 0, sizeof(int) * 4, c->st);
   c->sc = dalloc<double>(c, kNumScalars);
   c->d_err = dalloc<int>(c, 1);
+  cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
   if (cudaMallocHost(&c->h_sc, kNumScalars * sizeof(double)) != cudaSuccess) throw std::bad_alloc();
   cudaMemsetAsync(c->u, 0, sizeof(double) * P.n_dof, c->st);
   cudaMemsetAsync(c->sig, 0, sizeof(double) * 6 * P.n_gp, c->st);

@@ -2,24 +2,28 @@
 //
 // The FP64 pipe of this part issues two FMAs per SM and clock (1.06 TFLOP/s for the whole
 // device), so the banded sweeps of the subdomains that share their shape's elastic factor
-// are bound by it (1.60 ms a pass over 512 boxes of 8^3 elements, 73 % of the pipe).  Their
-// K^+ apply is a contraction, Y = X K^+ with one row of X per subdomain, and BF16 tensor
-// cores run 1800 times faster; FP64 accuracy comes from an error-free splitting of both
-// operands into integer digits (the scheme of Ozaki, Ogita, Oishi and Rump, "Error-free
-// transformations of matrix multiplication by using fast routines of matrix
-// multiplication and its applications", Numer. Algorithms 59, 2012):
+// are bound by it: 1600 us a pass over 512 boxes of 8^3 elements (2187 dofs, 1158 at the
+// boundary), 4750 us over 1728.  Their K^+ apply is a contraction, Y = X K^+ with one row of X
+// per subdomain, and BF16 tensor cores run 1800 times faster.  Measured with these kernels: 135
+// us for the pass on all dofs of the 512 boxes (split 15, GEMM 102, scatter 18) and 75 us on the
+// boundary dofs; the GEMM's 141 GFLOP of digit products run at 1.4 PFLOP/s, bound by the MMAs
+// (95 us without copies and without draining the accumulators, 58 us without the MMAs).
 //
-//   a row of X, scaled by the power of two above its largest entry, is
-//       x = 2^(e-7) sum_i d_i 2^(-8 i),  i = 0..6,  integers |d_i| <= 128,
-//   i.e. 55 bits below 2^e (round to nearest), and likewise every row of K^+.  A digit
-//   times 2^(-8 i) is exact in BF16.  The products d_i d'_j with i + j = g have weight
-//   2^(-8 g); the 28 pairs with i + j <= 6 are formed, the dropped ones lie below 2^-55 of
-//   the leading one.  Sums over K of the groups g = 0..3 are integers times 2^(-8 g): at
-//   most 4 x 256 x 2^14 = 2^24 over a chunk of 256 of K, so the FP32 accumulators in TMEM
-//   hold them exactly; after each chunk they are added, as integers, into a 64-bit sum.
-//   The groups 4..6 carry at most 2^-32 of the leading weight, so they share one FP32
-//   accumulator over the whole K range, whose rounding lies below 2^-52 of the leading
-//   products.  The total is an integer in units of 2^-32 and is converted to FP64 once.
+// FP64 accuracy comes from an error-free splitting of both operands into integer digits (the
+// scheme of Ozaki, Ogita, Oishi and Rump, "Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication and its applications",
+// Numer. Algorithms 59, 2012): a row of X, scaled by the power of two above its largest entry, is
+//     x = 2^(e-7) sum_i d_i 2^(-8 i),  i = 0..6,  integers |d_i| <= 128,
+// i.e. 55 bits below 2^e (round to nearest), and likewise every row of K^+.  A digit
+// times 2^(-8 i) is exact in BF16.  The products d_i d'_j with i + j = g have weight
+// 2^(-8 g); the 28 pairs with i + j <= 6 are formed, the dropped ones lie below 2^-55 of
+// the leading one.  Sums over K of the groups g = 0..4 are integers times 2^(-8 g): at
+// most 5 x 192 x 2^14 < 2^24 over a chunk of 192 of K, so the FP32 accumulators in TMEM
+// hold them exactly; after each chunk they are added, as integers, into a 64-bit sum.
+// The groups 5 and 6 carry at most 2^-40 of the leading weight, so they are accumulated in
+// FP32 over the whole K range.  The total is an integer in units of 2^-37 and is converted to
+// FP64 once.  Against extended precision the product of a 2187-dof box is off by 2.2e-15 (norm),
+// a sequential FP64 sum by 2.4e-15 (with four exact groups instead of five: 3.9e-14).
 //
 // Non-finite entries make the row's scale NaN, so that the whole result of that subdomain
 // is NaN, as it is after the banded sweeps.
@@ -27,9 +31,10 @@
 // Tiles: 128 rows of X (subdomains) x 64 rows of K^+ (output dofs) per CTA.  The digits of a
 // stage's K^+ tile are stacked as 7 x 64 rows, so the products of digit i of X with the digits
 // j = 0..6 - i are one run of 64 (7 - i) columns of accumulators starting at group i: ten MMAs
-// of up to 256 columns per 16 columns of K instead of 28 of 64 (an MMA takes 64 cycles however
-// narrow it is: 28 MMAs of 80, 64, 48 or 32 columns all measured 126 us for the 8^3 box shape
-// below, without copies).  The seven accumulators fill 448 of the 512 TMEM columns.
+// of up to 256 columns per 16 columns of K instead of 28 of 64 (a narrow MMA takes about 64
+// cycles whatever its width: 28 MMAs of 80, 64, 48 or 32 columns each took 126 us a wave for
+// the 2187-dof boxes).  Stages of 16 columns of K, 43 KB, five in flight.  The seven
+// accumulators fill 448 of the 512 TMEM columns.
 #include <cuda_bf16.h>
 
 #include "async_common.cuh"
