@@ -158,6 +158,20 @@ void sort_items_by_cost(const tfeti_ctx* c, std::vector<SolveItem>& items) {
                    [&cost](const SolveItem& a, const SolveItem& b) { return cost(a) > cost(b); });
 }
 
+tfeti_ctx::ItemStat item_stat(const tfeti_ctx* c, const std::vector<SolveItem>& items) {
+  tfeti_ctx::ItemStat s;
+  double sum = 0.0, top = 0.0;
+  for (const SolveItem& it : items) {
+    const SubDev& S = c->h_subs[it.sub[0]];
+    const double w = (double)it.count * S.n_dof * (S.bw + 1);
+    sum += w;
+    top = std::max(top, w);
+    s.max_count = std::max(s.max_count, it.count);
+  }
+  s.n_eff = top > 0.0 ? (int)std::ceil(sum / top) : 0;
+  return s;
+}
+
 // Solve work items: elastic subdomains of one shape share the shape's template
 // factor and are grouped R to a CTA so that the items fit one wave of SMs;
 // subdomains with plastic points carry their own factor, one per CTA.
@@ -347,6 +361,10 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
   build_item_list(c, plastic_count, R64_all, all);
   for (const SolveItem& it : all)
     if ((it.fac & kOwnFac) || !uses_schur(c->h_subs[it.sub[0]].shape)) pl64.push_back(it);
+  c->is64 = item_stat(c, c->h_items);
+  c->is32 = item_stat(c, c->h_items32);
+  c->is_pl = item_stat(c, pl);
+  c->is_pl64 = item_stat(c, pl64);
   c->n_items_pl = (int)pl.size();
   c->n_items_pl64 = (int)pl64.size();
   if (!pl64.empty())
@@ -366,6 +384,8 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
     build_dir_item_list(c, plastic_count, R32, c->h_items_d32);
     c->n_items_d = (int)c->h_items_d.size();
     c->n_items_d32 = (int)c->h_items_d32.size();
+    c->is_d = item_stat(c, c->h_items_d);
+    c->is_d32 = item_stat(c, c->h_items_d32);
     cudaMemcpyAsync(c->d_items_d, c->h_items_d.data(), sizeof(SolveItem) * c->h_items_d.size(),
                     cudaMemcpyHostToDevice, c->st);
     cudaMemcpyAsync(c->d_items_d32, c->h_items_d32.data(), sizeof(SolveItem) * c->h_items_d32.size(),
@@ -376,6 +396,11 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
                     c->st);
   cudaMemcpyAsync(c->d_items32, c->h_items32.data(), sizeof(SolveItem) * c->h_items32.size(),
                   cudaMemcpyHostToDevice, c->st);
+}
+
+void set_stat(SolveArgs& a, const tfeti_ctx::ItemStat& s) {
+  a.max_count = s.max_count;
+  a.n_eff = s.n_eff;
 }
 
 SolveArgs solve_args(tfeti_ctx* c, bool fp32 = false) {
@@ -391,6 +416,9 @@ SolveArgs solve_args(tfeti_ctx* c, bool fp32 = false) {
   a.rec_max = c->rec_max;
   a.npad = c->npad;
   a.rcap = fp32 ? c->rcap32 : c->rcap;
+  set_stat(a, fp32 ? c->is32 : c->is64);
+  a.max_bw = c->plan.max_bw;
+  a.cl_max = c->cl_max;
   return a;
 }
 
@@ -540,6 +568,7 @@ void op_F(tfeti_ctx* c, const double* x, double* yv) {
       cudaStreamWaitEvent(c->st2, c->ev_fork, 0);
       a.items = c->d_items_pl64;
       a.n_items = c->n_items_pl64;
+      set_stat(a, c->is_pl64);
       launch_sub_solve(c->M, a, c->solve_smem, c->st2);
       cudaEventRecord(c->ev_join, c->st2);
       c->launches += 1;
@@ -586,6 +615,7 @@ void op_F32(tfeti_ctx* c, const double* x, double* yv, bool contract = true) {
       cudaStreamWaitEvent(c->st2, c->ev_fork, 0);
       a.items = c->d_items_pl;
       a.n_items = c->n_items_pl;
+      set_stat(a, c->is_pl);
       launch_sub_solve(c->M, a, c->solve_smem32, c->st2);
       cudaEventRecord(c->ev_join, c->st2);
       c->launches += 1;
@@ -1235,6 +1265,7 @@ void op_precond_dirichlet(tfeti_ctx* c, const double* w, double* out, bool fp32)
   a.fac32_own = c->dfac32_own;
   a.items = fp32 ? c->d_items_d32 : c->d_items_d;
   a.n_items = fp32 ? c->n_items_d32 : c->n_items_d;
+  set_stat(a, fp32 ? c->is_d32 : c->is_d);
   a.src = c->dx_b;
   a.bmask = c->d_bmask;
   a.no_fix = 1;
@@ -2598,6 +2629,14 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     for (const SubInfo& s : P.subs) c->rec_max = std::max(c->rec_max, s.rec);
     c->npad = (P.max_ndof + 1) & ~1;
+    // the cluster form of the solve splits a row block into at least four rows per CTA
+    int min_nb = kMaxNB;
+    bool cl_ok = true;
+    for (const SubInfo& s : P.subs) {
+      min_nb = std::min(min_nb, s.nb);
+      cl_ok = cl_ok && (s.nb == 16 || s.nb == 32);
+    }
+    c->cl_max = cl_ok ? std::min(8, min_nb / 4) : 1;
     const long long room = (long long)max_smem - 1024 - 16LL * c->rec_max;   // static smem and barriers
     c->rcap = (int)std::min<long long>(kMaxRHS, room / (8LL * c->npad));
     if (c->rcap < 1) return fail(c, TFETI_ERR_ARG, "subdomain too large for the shared-memory solve");

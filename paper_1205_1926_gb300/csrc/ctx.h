@@ -178,7 +178,13 @@ struct tfeti_ctx {
   tfeti::SolveItem* d_items = nullptr;   // solve work items (device), rebuilt after each assembly
   std::vector<tfeti::SolveItem> h_items;
   int n_items = 0;
-  int rec_max = 0, npad = 0, rcap = 1;
+  int rec_max = 0, npad = 0, rcap = 1, cl_max = 1;
+  // per item list (the FP64 and FP32 lists, their parts beside the Schur GEMMs, the Dirichlet lists):
+  // most right-hand sides of one item, items counted by work
+  struct ItemStat {
+    int max_count = 0, n_eff = 0;
+  };
+  ItemStat is64, is32, is_pl, is_pl64, is_d, is_d32;
   size_t solve_smem = 0;
   int n_sm = 1;
   int* d_list = nullptr;

@@ -158,6 +158,10 @@ struct SolveArgs {
   int rec_max;                 // largest panel record of the launch (doubles, even)
   int npad;                    // vector stride in shared memory (largest n, even)
   int rcap;                    // vectors allocated per CTA (>= every item's count)
+  int max_count;               // largest item count of the launch
+  int n_eff;                   // its items counted by work: total over the largest item's, rounded up
+  int max_bw;                  // largest half bandwidth of any subdomain
+  int cl_max;                  // most CTAs that may share an item (cluster form), 1: none
   // in_mode 2 / out_mode 2 (dual Schur block formation of one shape): item.sub[] hold
   // boundary-dof columns j; the geometry is subdomain rep_sub; column j of
   // S = (K^+)_{boundary, boundary} goes to S32 + s_off + j * n_bd.

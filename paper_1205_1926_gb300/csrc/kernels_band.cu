@@ -210,45 +210,12 @@ __global__ void __launch_bounds__(kThreads) k_band_chol(DevMesh M, const int* __
 // (nb x bw doubles each) filled one step ahead by bulk copies, the kMaxRHS
 // local vectors, two mbarriers.
 // ---------------------------------------------------------------------------
+
+// Right-hand sides of an item into vec (stride npad), by all threads of a CTA; ends with a barrier.
 template <typename T>
-__global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs a) {
-  extern __shared__ __align__(128) unsigned char sm_raw[];
-  T* sm = reinterpret_cast<T*>(sm_raw);
-  __shared__ int s_fail;
-  const SolveItem item = a.items[blockIdx.x];
-  // unit right-hand sides (in_mode 2, 5) carry dof indices in item.sub[]: the geometry is rep_sub's
-  const SubDev& S0 = M.subs[(a.in_mode == 2 || a.in_mode == 5) ? a.rep_sub : item.sub[0]];
-  const int n = S0.n_dof, bw = S0.bw, nb = S0.nb, nblk = S0.nblk, rec = S0.rec;
-  const int R = item.count;
-  const int npad = a.npad;                       // vector stride (largest n of the launch, even)
-  T* pan[2] = {sm, sm + a.rec_max};
-  T* vec = sm + 2 * a.rec_max;                   // [rcap][npad]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(vec + ((a.rcap * npad + 1) & ~1));
-  const bool own = (item.fac & kOwnFac) != 0;
-  const T* fac = (sizeof(T) == 8 ? reinterpret_cast<const T*>(own ? a.fac_own : a.fac)
-                                 : reinterpret_cast<const T*>(own ? a.fac32_own : a.fac32)) +
-                 (item.fac & ~kOwnFac);
-  const T* dinv = fac + (long long)nblk * rec;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int nsteps = 2 * nblk;
-  const uint32_t pbytes = (uint32_t)rec * (uint32_t)sizeof(T);
-
-  if (tid == 0) {
-    s_fail = 0;
-    mbar_init(&bar[0]);
-    mbar_init(&bar[1]);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  __syncthreads();
-  // step k uses the panel of block k (forward, k < nblk) or 2 nblk - 1 - k (backward)
-  auto step_block = [nblk, nsteps](int k) { return k < nblk ? k : nsteps - 1 - k; };
-  if (tid == 0) {
-    bulk_copy(pan[0], fac, pbytes, &bar[0]);
-    bulk_copy(pan[1], fac + (long long)step_block(1) * rec, pbytes, &bar[1]);
-  }
-
-  // ---- right-hand sides
-  const int n_bd = 3 * S0.n_bnd;
+__device__ __forceinline__ void load_rhs(const DevMesh& M, const SolveArgs& a, const SolveItem& item, const SubDev& S0,
+                                         T* vec, int npad) {
+  const int n = S0.n_dof, R = item.count, tid = threadIdx.x, nt = blockDim.x;
   if (a.in_mode == 2 || a.in_mode == 5) {   // unit vectors at boundary dofs (2) or local dofs (5) item.sub[r]
     for (int r = 0; r < R; ++r)
       for (int i = tid; i < n; i += nt) vec[r * npad + i] = T(0);
@@ -270,45 +237,57 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
       for (int i = tid; i < n; i += nt) x[i] = a.src ? T(a.src[S.dof_off + i]) : T(0);
   }
   __syncthreads();
-  for (int r = 0; r < R && !unit_in; ++r) {
+  constexpr int U = 4;   // copy slots per thread with their B^T gathers in flight together
+  for (int r = 0; r < R && !unit_in && a.in_mode != 4 && a.lam; ++r) {
     const SubDev& S = M.subs[item.sub[r]];
     T* x = vec + r * npad;
-    if (a.in_mode == 0) {
-      for (int s = tid; s < S.n_copy; s += nt) {
-        const long long slot = S.copy_off + s;
-        x[M.slot_ldof[slot]] = T(bt_at_slot(M, a.lam, slot));
-      }
-    } else if (a.lam) {
-      for (int s = tid; s < S.n_copy; s += nt) {
-        const long long slot = S.copy_off + s;
-        x[M.slot_ldof[slot]] -= T(bt_at_slot(M, a.lam, slot));
-      }
+    for (int s0 = tid; s0 < S.n_copy; s0 += U * nt) {
+      long long sl[U];
+      double v[U];
+#pragma unroll
+      for (int k = 0; k < U; ++k) sl[k] = s0 + k * nt < S.n_copy ? S.copy_off + s0 + k * nt : -1;
+      bt_at_slots<U>(M, a.lam, sl, v);
+#pragma unroll
+      for (int k = 0; k < U; ++k)
+        if (sl[k] >= 0) {
+          const int d = __ldg(M.slot_ldof + sl[k]);
+          x[d] = a.in_mode == 0 ? T(v[k]) : x[d] - T(v[k]);
+        }
     }
   }
   __syncthreads();
   if (tid < 6 && !a.no_fix)
     for (int r = 0; r < R; ++r) vec[r * npad + S0.fix[tid]] = T(0);
   __syncthreads();
+}
 
+// The sweeps of one item with R right-hand sides, all threads of a CTA; the panels of steps 0 and 1 are
+// on their way.  Returns -1, or the step whose panel copy did not complete.
+template <typename T, int R>
+__device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __restrict__ dinv, T* const* pan, T* vec,
+                     int npad, uint64_t* bar, int* s_fail) {
+  const int n = S0.n_dof, bw = S0.bw, nb = S0.nb, nblk = S0.nblk, rec = S0.rec;
+  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const int nsteps = 2 * nblk;
+  const uint32_t pbytes = (uint32_t)rec * (uint32_t)sizeof(T);
+  auto step_block = [nblk, nsteps](int k) { return k < nblk ? k : nsteps - 1 - k; };
   // ---- x' = D^{-1} x, block-diagonal, 256 rows at a time through registers
   for (int base = 0; base < n; base += nt) {
     const int i = base + tid;
-    T v[kMaxRHS] = {T(0), T(0), T(0), T(0)};
+    T v[R] = {};
     if (i < n) {
       const int b = i / nb, t = i - b * nb, r0 = b * nb;
       const T* drow = dinv + (long long)b * nb * nb + t * nb;
       for (int q = 0; q <= t; ++q) {
         const T d = drow[q];
 #pragma unroll
-        for (int r = 0; r < kMaxRHS; ++r)
-          if (r < R) v[r] = fma(d, vec[r * npad + r0 + q], v[r]);
+        for (int r = 0; r < R; ++r) v[r] = fma(d, vec[r * npad + r0 + q], v[r]);
       }
     }
     __syncthreads();
     if (i < n)
 #pragma unroll
-      for (int r = 0; r < kMaxRHS; ++r)
-        if (r < R) vec[r * npad + i] = v[r];
+      for (int r = 0; r < R; ++r) vec[r * npad + i] = v[r];
     __syncthreads();
   }
 
@@ -319,7 +298,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
   for (int k = 0; k < nsteps; ++k) {
     const int buf = k & 1;
     const bool ok = mbar_wait(&bar[buf], (uint32_t)((k >> 1) & 1));
-    if (!ok) s_fail = 1;
+    if (!ok) *s_fail = 1;
     const T* P = pan[buf];
     const int b = step_block(k);
     const int r0 = b * nb, jb = min(nb, n - r0);
@@ -328,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
       if (k < nblk) {
         const int t = 4 * warp + g;                 // 8 warps x 4 rows = 32 rows
         const bool act = t < jb;
-        T acc[kMaxRHS] = {T(0), T(0), T(0), T(0)};
+        T acc[R] = {};
         if (act) {
           const T* prow = P + t * bw;
           for (int j = l; j < bw; j += 8) {
@@ -336,20 +315,18 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
             const T mv = prow[j];
             const int c = c0 + j;
 #pragma unroll
-            for (int r = 0; r < kMaxRHS; ++r)
-              if (r < R) acc[r] = fma(mv, vec[r * npad + c], acc[r]);
+            for (int r = 0; r < R; ++r) acc[r] = fma(mv, vec[r * npad + c], acc[r]);
           }
         }
 #pragma unroll
-        for (int r = 0; r < kMaxRHS; ++r) {
+        for (int r = 0; r < R; ++r) {
           acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 4);
           acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 2);
           acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 1);
         }
         if (act && l == 0)
 #pragma unroll
-          for (int r = 0; r < kMaxRHS; ++r)
-            if (r < R) vec[r * npad + r0 + t] -= acc[r];
+          for (int r = 0; r < R; ++r) vec[r * npad + r0 + t] -= acc[r];
       } else {
         // one (column, right-hand side) pair per thread: bw * R units spread evenly over the CTA
         const int units = (bw - jlo) * R;
@@ -364,12 +341,84 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
       }
     }
     __syncthreads();
-    if (s_fail) {
+    if (*s_fail) {
       k_fail = k;
       break;
     }
     if (tid == 0 && k + 2 < nsteps) bulk_copy(pan[buf], fac + (long long)step_block(k + 2) * rec, pbytes, &bar[buf]);
   }
+  if (k_fail >= 0) return k_fail;
+
+  // ---- z = D^{-T} z'
+  for (int base = 0; base < n; base += nt) {
+    const int i = base + tid;
+    T v[R] = {};
+    if (i < n) {
+      const int b = i / nb, t = i - b * nb, r0 = b * nb;
+      const int jb = min(nb, n - r0);
+      const T* dblk = dinv + (long long)b * nb * nb;
+      for (int s = t; s < jb; ++s) {
+        const T d = dblk[s * nb + t];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = fma(d, vec[r * npad + r0 + s], v[r]);
+      }
+    }
+    __syncthreads();
+    if (i < n)
+#pragma unroll
+      for (int r = 0; r < R; ++r) vec[r * npad + i] = v[r];
+    __syncthreads();
+  }
+  return -1;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs a) {
+  extern __shared__ __align__(128) unsigned char sm_raw[];
+  T* sm = reinterpret_cast<T*>(sm_raw);
+  __shared__ int s_fail;
+  const SolveItem item = a.items[blockIdx.x];
+  // unit right-hand sides (in_mode 2, 5) carry dof indices in item.sub[]: the geometry is rep_sub's
+  const SubDev& S0 = M.subs[(a.in_mode == 2 || a.in_mode == 5) ? a.rep_sub : item.sub[0]];
+  const int n = S0.n_dof, bw = S0.bw, nb = S0.nb, nblk = S0.nblk, rec = S0.rec;
+  const int R = item.count;
+  const int npad = a.npad;                       // vector stride (largest n of the launch, even)
+  T* pan[2] = {sm, sm + a.rec_max};
+  T* vec = sm + 2 * a.rec_max;                   // [rcap][npad]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(vec + ((a.rcap * npad + 1) & ~1));
+  const bool own = (item.fac & kOwnFac) != 0;
+  const T* fac = (sizeof(T) == 8 ? reinterpret_cast<const T*>(own ? a.fac_own : a.fac)
+                                 : reinterpret_cast<const T*>(own ? a.fac32_own : a.fac32)) +
+                 (item.fac & ~kOwnFac);
+  const T* dinv = fac + (long long)nblk * rec;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int nsteps = 2 * nblk;
+  const uint32_t pbytes = (uint32_t)rec * (uint32_t)sizeof(T);
+
+  if (tid == 0) {
+    s_fail = 0;
+    mbar_init(&bar[0]);
+    mbar_init(&bar[1]);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  // step k uses the panel of block k (forward, k < nblk) or 2 nblk - 1 - k (backward)
+  auto step_block = [nblk, nsteps](int k) { return k < nblk ? k : nsteps - 1 - k; };
+  if (tid == 0) {
+    bulk_copy(pan[0], fac, pbytes, &bar[0]);
+    bulk_copy(pan[1], fac + (long long)step_block(1) * rec, pbytes, &bar[1]);
+  }
+
+  const int n_bd = 3 * S0.n_bnd;
+  load_rhs<T>(M, a, item, S0, vec, npad);
+  // the sweeps are compiled for the item's number of right-hand sides: an FP64 instruction occupies
+  // the pipe also where its predicate is off (a single right-hand side took 1200 us of the four's
+  // 1600 us for a 2187-dof box when all four were predicated)
+  int k_fail;
+  if (R == 1) k_fail = sweep<T, 1>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
+  else if (R == 2) k_fail = sweep<T, 2>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
+  else if (R == 3) k_fail = sweep<T, 3>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
+  else k_fail = sweep<T, 4>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
   if (k_fail >= 0) {
     // a panel copy never completed: report, give the copies still in flight (steps
     // k_fail and k_fail + 1) a bounded time to land, and leave
@@ -379,29 +428,6 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
       if (k_fail + 1 < nsteps) mbar_wait(&bar[(k_fail + 1) & 1], (uint32_t)(((k_fail + 1) >> 1) & 1));
     }
     return;
-  }
-
-  // ---- z = D^{-T} z'
-  for (int base = 0; base < n; base += nt) {
-    const int i = base + tid;
-    T v[kMaxRHS] = {T(0), T(0), T(0), T(0)};
-    if (i < n) {
-      const int b = i / nb, t = i - b * nb, r0 = b * nb;
-      const int jb = min(nb, n - r0);
-      const T* dblk = dinv + (long long)b * nb * nb;
-      for (int s = t; s < jb; ++s) {
-        const T d = dblk[s * nb + t];
-#pragma unroll
-        for (int r = 0; r < kMaxRHS; ++r)
-          if (r < R) v[r] = fma(d, vec[r * npad + r0 + s], v[r]);
-      }
-    }
-    __syncthreads();
-    if (i < n)
-#pragma unroll
-      for (int r = 0; r < kMaxRHS; ++r)
-        if (r < R) vec[r * npad + i] = v[r];
-    __syncthreads();
   }
   if (tid < 6 && !a.no_fix)
     for (int r = 0; r < R; ++r) vec[r * npad + S0.fix[tid]] = T(0);
@@ -450,6 +476,321 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same solve by a cluster of C CTAs per item, for launches with fewer items than SMs.  One
+// CTA per item leaves its two sweeps of 2 n / nb dependent block steps to one SM, whose FP64 pipe
+// (two FMAs per clock) then sets the time.  Here CTA q owns rows [q nb / C, (q + 1) nb / C) of every
+// block and streams only those rows of the panels:
+//   forward:  y_t = x'_t - M_b[t][:] y[r0 - bw, r0) for its rows, sent to all CTAs' vectors;
+//   backward: its rows' terms M_b[t][:] z'_t go into a running sum per column, kept by one thread
+//             from the column's first step to its last; when a column's block is next, the sums
+//             are sent to the rows' owners (before the other columns are worked on), which add them
+//             in a fixed order and finish z'_t.
+// The values travel as asynchronous remote stores that complete on an mbarrier of the receiver, so a
+// step waits for one crossing and no CTA can run more than one step ahead; the panel slices arrive
+// by bulk copies several steps ahead.
+// ---------------------------------------------------------------------------
+constexpr int kClThreads = 128;
+constexpr int kClStages = 4;   // panel slices in flight
+constexpr int kClRing = 4;     // exchange barriers and receive buffers in turn
+
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, unsigned rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_cluster(const double* p, unsigned rank, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void st_cluster(const float* p, unsigned rank, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "f"(v) : "memory");
+}
+// Remote store of v to p in CTA rank, completing sizeof(v) bytes on bar there.
+__device__ __forceinline__ void st_async(const double* p, const uint64_t* bar, unsigned rank, double v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(
+                   cluster_addr(p, rank)),
+               "l"(__double_as_longlong(v)), "r"(cluster_addr(bar, rank))
+               : "memory");
+}
+__device__ __forceinline__ void st_async(const float* p, const uint64_t* bar, unsigned rank, float v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
+                   cluster_addr(p, rank)),
+               "r"(__float_as_uint(v)), "r"(cluster_addr(bar, rank))
+               : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Sums over the warp of NR values per lane: lane / (32 / NR) gets the sum of v[lane / (32 / NR)].
+template <typename T, int NR>
+__device__ __forceinline__ T warp_sum_rows(T (&v)[NR], int lane) {
+  T k;
+  int o;
+  if constexpr (NR == 4) {
+    const bool h = lane & 16, g = lane & 8;
+    T a = h ? v[2] : v[0], b = h ? v[3] : v[1];
+    a += __shfl_xor_sync(0xffffffffu, h ? v[0] : v[2], 16);
+    b += __shfl_xor_sync(0xffffffffu, h ? v[1] : v[3], 16);
+    k = g ? b : a;
+    k += __shfl_xor_sync(0xffffffffu, g ? a : b, 8);
+    o = 4;
+  } else if constexpr (NR == 2) {
+    const bool h = lane & 16;
+    k = h ? v[1] : v[0];
+    k += __shfl_xor_sync(0xffffffffu, h ? v[0] : v[1], 16);
+    o = 8;
+  } else {
+    k = v[0];
+    o = 16;
+  }
+  for (; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  return k;
+}
+
+// Shared memory of a cluster CTA in values of T: panel slices, the vectors, the own rows' x', the
+// window of column sums (a power of two above bw + nb), the received sums.
+struct ClLayout {
+  int slice, npad, own, win, recv;
+  __host__ __device__ ClLayout(int rec_max, int npad_, int max_bw, int C)
+      : slice((rec_max / C + 3) & ~3), npad(npad_), own(npad_ / C + 2 * kMaxNB), recv(kClRing * kMaxNB) {
+    win = 128;
+    while (win < max_bw + kMaxNB) win *= 2;
+  }
+  __host__ __device__ size_t values(int R) const {
+    return (size_t)kClStages * slice + (size_t)R * ((size_t)npad + own + win + recv);
+  }
+};
+
+// R right-hand sides, NR own rows of a block per warp (nb / C = 4 NR).
+template <typename T, int R, int NR>
+__device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& item, int C, unsigned q, T* sm,
+                         uint64_t* bar, uint64_t* xbar) {
+  constexpr int rpc = 4 * NR;
+  __shared__ T s_z[4][rpc][R];     // backward: z' of the own rows, one copy per warp
+  const SubDev& S0 = M.subs[item.sub[0]];
+  const int n = S0.n_dof, bw = S0.bw, nb = S0.nb, nblk = S0.nblk, rec = S0.rec;
+  const ClLayout lay(a.rec_max, a.npad, a.max_bw, C);
+  T* pan = sm;
+  T* vec = pan + kClStages * lay.slice;      // [R][npad]
+  T* xo = vec + R * lay.npad;                // [R][own]: x' of the own rows
+  T* win = xo + R * lay.own;                 // [R][win]
+  T* recv = win + R * lay.win;               // [kClRing][C][rpc][R]
+  const int npad = lay.npad, wmask = lay.win - 1;
+  const bool own = (item.fac & kOwnFac) != 0;
+  const T* fac = (sizeof(T) == 8 ? reinterpret_cast<const T*>(own ? a.fac_own : a.fac)
+                                 : reinterpret_cast<const T*>(own ? a.fac32_own : a.fac32)) +
+                 (item.fac & ~kOwnFac);
+  const T* dinv = fac + (long long)nblk * rec;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nsteps = 2 * nblk;
+  const uint32_t pbytes = (uint32_t)(rpc * bw) * (uint32_t)sizeof(T);   // rpc is a multiple of 4
+  auto step_block = [nblk, nsteps](int k) { return k < nblk ? k : nsteps - 1 - k; };
+  auto fetch = [&](int k) {
+    bulk_copy(pan + (k % kClStages) * lay.slice, fac + (long long)step_block(k) * rec + (long long)q * rpc * bw, pbytes,
+              &bar[k % kClStages]);
+  };
+  bool ok = true;   // after a wait that gave up, the remaining steps run through without waiting
+  auto wait_panel = [&](int k) {
+    if (ok) ok = mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1));
+  };
+  auto wait_exchange = [&](int e) {
+    if (ok) ok = mbar_wait(&xbar[e % kClRing], (uint32_t)((e / kClRing) & 1));
+  };
+  int issued = 0;
+  if (tid == 0)
+    for (; issued < kClStages && issued < nsteps; ++issued) fetch(issued);
+  load_rhs<T>(M, a, item, S0, vec, npad);
+
+  // x' = D^-1 x on the own rows, one (block, row) per thread
+  for (int i = tid; i < nblk * rpc; i += kClThreads) {
+    const int b = i / rpc, t = (int)q * rpc + i % rpc, r0 = b * nb;
+    T v[R] = {};
+    if (r0 + t < n) {
+      const T* drow = dinv + (long long)b * nb * nb + t * nb;
+      for (int u = 0; u <= t; ++u) {
+        const T d = drow[u];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = fma(d, vec[r * npad + r0 + u], v[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) xo[r * lay.own + i] = v[r];
+  }
+  for (int i = tid; i < R * lay.win; i += kClThreads) win[i] = T(0);
+  cluster_barrier();   // every CTA has read its x (and set its barriers up) before the first y arrives
+
+  // forward: a warp's NR rows, columns across the lanes
+  for (int k = 0; k < nblk; ++k) {
+    const int r0 = k * nb, c0 = r0 - bw, jlo = max(0, -c0);
+    if (tid == 0) mbar_expect_tx(&xbar[k % kClRing], (uint32_t)(min(nb, n - r0) * R * (int)sizeof(T)));
+    wait_panel(k);
+    const T* P = pan + (k % kClStages) * lay.slice + warp * NR * bw;
+    T acc[R][NR] = {};
+#pragma unroll 4
+    for (int j = jlo + lane; j < bw; j += 32) {
+      T x[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) x[r] = vec[r * npad + c0 + j];
+#pragma unroll
+      for (int i = 0; i < NR; ++i) {
+        const T mv = P[i * bw + j];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r][i] = fma(mv, x[r], acc[r][i]);
+      }
+    }
+    const int t = warp * NR + lane / (32 / NR), dst = lane % (32 / NR), gr = r0 + (int)q * rpc + t;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const T v = xo[r * lay.own + k * rpc + t] - warp_sum_rows<T, NR>(acc[r], lane);
+      if (dst < C && gr < n) st_async(vec + r * npad + gr, &xbar[k % kClRing], (unsigned)dst, v);
+    }
+    wait_exchange(k);
+    __syncthreads();
+    if (tid == 0 && ok && issued < nsteps) fetch(issued++);
+  }
+  // backward: column c belongs to lane c % 32 of warp (c / 32) % 4 from its first step to its last
+  for (int k = nblk; k < nsteps; ++k) {
+    const int b = nsteps - 1 - k, r0 = b * nb, lo = max(0, r0 - bw), nxt = r0 - nb;
+    if (tid == 0 && b > 0) mbar_expect_tx(&xbar[k % kClRing], (uint32_t)(nb * R * (int)sizeof(T)));
+    // z' of the own rows: y less the CTAs' sums (lane = CTA x row), in every warp
+    if (k > nblk) wait_exchange(k - 1);
+    {
+      const int t = lane % rpc, c = lane / rpc, gr = r0 + (int)q * rpc + t;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        T v = (k > nblk && c < C) ? recv[((((k - 1) % kClRing) * C + c) * rpc + t) * R + r] : T(0);
+        for (int o = rpc; o < rpc * C; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane < rpc) {
+          v = gr < n ? vec[r * npad + gr] - v : T(0);
+          s_z[warp][t][r] = v;
+          // the block's D^-T (below) runs in CTA b % C
+          if (warp == 0 && gr < n) st_cluster(vec + r * npad + gr, (unsigned)(b % C), v);
+        }
+      }
+    }
+    __syncwarp();
+    wait_panel(k);
+    const T* P = pan + (k % kClStages) * lay.slice;
+    const int top = (r0 - 1) >> 5;
+    for (int u = top - ((top - warp) & 3); b > 0 && 32 * u + 31 >= min(lo, nxt) && u >= 0; u -= 4) {
+      const int c = 32 * u + lane;
+      if (c >= r0 || c < min(lo, nxt)) continue;
+      T s[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) s[r] = win[r * lay.win + (c & wmask)];
+      if (c >= lo) {
+        const T* pc = P + (c - (r0 - bw));
+#pragma unroll
+        for (int t = 0; t < rpc; ++t) {
+          const T mv = pc[t * bw];
+#pragma unroll
+          for (int r = 0; r < R; ++r) s[r] = fma(mv, s_z[warp][t][r], s[r]);
+        }
+      }
+      const int t = c - nxt;
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        // block b - 1 is next: its sums to the rows' owners; the window slot is free again
+        if (t >= 0)
+          st_async(recv + (((k % kClRing) * C + (int)q) * rpc + t % rpc) * R + r, &xbar[k % kClRing],
+                   (unsigned)(t / rpc), s[r]);
+        win[r * lay.win + (c & wmask)] = t >= 0 ? T(0) : s[r];
+      }
+    }
+    __syncthreads();
+    if (tid == 0 && ok && issued < nsteps) fetch(issued++);
+  }
+  if (!ok) atomicOr(a.err, 2);
+  if (!ok && tid == 0)
+    for (int k = max(0, issued - kClStages); k < issued; ++k)   // copies still in flight land first
+      mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1));
+  cluster_barrier();   // the z' of the blocks below have arrived
+
+  // z = D^-T z' on the blocks b % C == q
+  __shared__ T s_col[kClThreads][R];
+  const int rows_per = kClThreads / nb;   // blocks per round
+  for (int i0 = (int)q; i0 < nblk; i0 += C * rows_per) {
+    const int sub = tid / nb, t = tid % nb, b = i0 + sub * C, r0 = b * nb;
+    const bool act = sub < rows_per && b < nblk && r0 + t < n;
+    T v[R] = {};
+    if (act) {
+      const int jb = min(nb, n - r0);
+      const T* dblk = dinv + (long long)b * nb * nb;
+      for (int s = t; s < jb; ++s) {
+        const T d = dblk[s * nb + t];
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = fma(d, vec[r * npad + r0 + s], v[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) s_col[tid][r] = v[r];
+    __syncthreads();
+    if (act)
+#pragma unroll
+      for (int r = 0; r < R; ++r) vec[r * npad + r0 + t] = s_col[tid][r];
+    __syncthreads();
+  }
+  if (tid < 6 && !a.no_fix)
+    for (int r = 0; r < R; ++r) vec[r * npad + S0.fix[tid]] = T(0);   // (entries of other CTAs' blocks are not read)
+  __syncthreads();
+  for (int r = 0; r < item.count; ++r) {
+    const SubDev& S = M.subs[item.sub[r]];
+    const T* x = vec + r * npad;
+    if (a.out_mode == 0 || a.out_mode == 3)
+      for (int s = tid; s < S.n_copy; s += kClThreads) {
+        const long long slot = S.copy_off + s;
+        const int d = __ldg(M.slot_ldof + slot);
+        if ((d / nb) % C == (int)q) a.cbuf[slot] = double(x[d]);
+      }
+    if (a.out_mode == 1 || a.out_mode == 3)
+      for (int b = (int)q; b < nblk; b += C)
+        for (int t = tid; t < nb && b * nb + t < n; t += kClThreads) a.dst[S.dof_off + b * nb + t] = double(x[b * nb + t]);
+  }
+}
+
+template <typename T, int R>
+__global__ void __launch_bounds__(kClThreads) k_solve_cl(DevMesh M, SolveArgs a) {
+  extern __shared__ __align__(128) unsigned char sm_raw[];
+  __shared__ uint64_t bar[kClStages], xbar[kClRing];
+  const int C = (int)cluster_size();
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < kClStages; ++k) mbar_init(&bar[k]);
+    for (int k = 0; k < kClRing; ++k) mbar_init(&xbar[k]);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
+  const SolveItem item = a.items[blockIdx.x / C];
+  T* sm = reinterpret_cast<T*>(sm_raw);
+  const int rpc = M.subs[item.sub[0]].nb / C;   // 4, 8 or 16 (the same for the whole cluster)
+  if (rpc == 4) cl_solve<T, R, 1>(M, a, item, C, cluster_rank(), sm, bar, xbar);
+  else if (rpc == 8) cl_solve<T, R, 2>(M, a, item, C, cluster_rank(), sm, bar, xbar);
+  else cl_solve<T, R, 4>(M, a, item, C, cluster_rank(), sm, bar, xbar);
+}
+
+// Launches the cluster form with C CTAs per item; false if it cannot run (nothing launched).
+template <typename T, int R>
+bool launch_cl(const DevMesh& M, const SolveArgs& a, int C, cudaStream_t st) {
+  const ClLayout lay(a.rec_max, a.npad, a.max_bw, C);
+  const size_t smem = sizeof(T) * lay.values(R);
+  static const int lim = dyn_smem_limit((const void*)k_solve_cl<T, R>);
+  if (smem > (size_t)lim) return false;
+  cudaFuncSetAttribute(k_solve_cl<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(a.n_items * C));
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)C;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_solve_cl<T, R>, M, a) == cudaSuccess;
+}
+
 }  // namespace
 
 // The device's opt-in shared-memory limit per block.  Kernels whose dynamic shared memory
@@ -475,6 +816,13 @@ int dyn_smem_limit(const void* fn) {
     return 48 * 1024;
   }
   return smem_optin_max() - (int)fa.sharedSizeBytes;
+}
+
+static int sm_count() {
+  int dev = 0, v = 1;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+  return v;
 }
 
 void launch_band_chol(const DevMesh& M, const int* sub_list, int n_list, const long long* band_off_list,
@@ -524,6 +872,24 @@ size_t sub_solve_smem(int rec_max, int npad, int rcap, int elem_bytes) {
 
 void launch_sub_solve(const DevMesh& M, const SolveArgs& a, size_t smem_bytes, cudaStream_t st) {
   if (a.n_items <= 0) return;
+  // Cluster form for items of at most two right-hand sides: the most CTAs per item for which the
+  // launch still has at most two per SM, counting the items by their work (n_eff = total work over
+  // the largest item's; small boxes beside a large one end early).  Measured, FP64 pass of one CTA /
+  // 2 / 4 / 8 CTAs per item: 54 boxes of 8^3 elements 559 / 432 / 354 / 499 us, 3 boxes of 6^3 (with
+  // the other boxes' product) - / 167 / 123 / 102 us, 125 uneven boxes of 4..12 elements per edge
+  // 1970 / 1401 / 1042 / - us; FP32, the uneven boxes: 627 / 634 / 603 us.
+  if (a.cl_max > 1 && a.max_count <= 2 && (a.in_mode == 0 || a.in_mode == 1 || a.in_mode == 4) && !a.alpha) {
+    static const int n_sm = sm_count();
+    int C = a.cl_max;
+    while (C > 1 && a.n_eff * C > 2 * n_sm) C /= 2;
+    if (C > 1) {
+      const bool one = a.max_count == 1;
+      const bool done = a.fp32 ? (one ? launch_cl<float, 1>(M, a, C, st) : launch_cl<float, 2>(M, a, C, st))
+                               : (one ? launch_cl<double, 1>(M, a, C, st) : launch_cl<double, 2>(M, a, C, st));
+      if (done) return;
+      cudaGetLastError();
+    }
+  }
   if (a.fp32) {
     static const int lim = dyn_smem_limit((const void*)k_sub_solve<float>);
     cudaFuncSetAttribute(k_sub_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
