@@ -2507,10 +2507,12 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   M.sigma_y = pr.sigma_y;
   M.H = pr.hardening;
   M.wdet = P.h[0] * P.h[1] * P.h[2] / 8.0;
+  const double ga = 0.5 * (1.0 + 1.0 / std::sqrt(3.0));
   for (int d = 0; d < 3; ++d) {
-    M.ga[d] = 0.5 * (1.0 + 1.0 / std::sqrt(3.0)) / P.h[d];
-    M.gb[d] = 0.5 * (1.0 - 1.0 / std::sqrt(3.0)) / P.h[d];
+    M.gs[d] = ga * ga / P.h[d];
+    M.gratio[d] = P.h[0] / P.h[d];
   }
+  M.wgs = M.wdet * M.gs[0];
   M.n_dof = P.n_dof;
   M.n_gp = P.n_gp;
   M.n_mult = P.n_mult;

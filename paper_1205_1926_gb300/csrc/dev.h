@@ -84,10 +84,9 @@ struct DevMesh {
   const float* GTv32;
   long long n_gpairs;
   double wdet;
-  // trilinear gradient weights on the uniform bricks: ga[d] = (1 + 1/sqrt 3) / (2 h_d) and
-  // gb[d] = (1 - 1/sqrt 3) / (2 h_d), the nodal weights of a Gauss point on the same and on the
-  // other side of the element along direction d, divided by h_d
-  double ga[3], gb[3];
+  // trilinear gradients on the uniform bricks: factors of the lane sums of kernels_fem.cu,
+  // gs[d] = ((1 + 1/sqrt 3) / 2)^2 / h_d, gratio[d] = h_x / h_d, wgs = wdet gs[0]
+  double gs[3], gratio[3], wgs;
   double lam, mu, sigma_y, H;
   long long n_dof, n_gp, n_mult, n_copy, n_elem;
   long long n_groups;

@@ -189,52 +189,74 @@ __global__ void k_traction(DevMesh M, int face, int nel0, int nel1, int nel2, do
 
 // ---------------------------------------------------------------------------
 // Trilinear gradients by sum factorisation over the 8 lanes of an element (lane bits x + 2y + 4z
-// give both the lane's Gauss point and the element node it loads).  For one displacement
-// component u (the lane's node value) the lane receives grad u at its Gauss point:
-//   along x: I = interpolant at the point's x, D = u(x=1) - u(x=0) on each x-edge;
-//   along y: DX = D interpolated in y, E = I(y=1) - I(y=0), J = I interpolated in y (/ h_z);
-//   along z: du/dx = DX interpolated in z / h_x, du/dy = E interpolated in z / h_y,
-//            du/dz = J(z=1) - J(z=0);
-// each interpolation step takes the lane's own value with weight (1 + 1/sqrt 3)/2 and its
-// partner's with (1 - 1/sqrt 3)/2 (the 2-point Gauss abscissae +-1/sqrt 3).  13 FP64 operations
-// per component and point instead of the 24 of the direct sum over the 8 nodes.
-// All 32 lanes of the warp take part.
-constexpr double kGa = 0.78867513459481288225;   // (1 + 1/sqrt 3) / 2
-constexpr double kGb = 0.21132486540518711775;   // (1 - 1/sqrt 3) / 2
+// give both the lane's Gauss point and the element node it loads).  An interpolation step takes the
+// lane's own value with weight (1 + 1/sqrt 3)/2 and its partner's with (1 - 1/sqrt 3)/2 (the 2-point
+// Gauss abscissae +-1/sqrt 3); as u + r u_partner with r = (1 - 1/sqrt 3)/(1 + 1/sqrt 3) it is one
+// FMA, the factor ((1 + 1/sqrt 3)/2)^2 of two steps left to the caller (M.gs).
+//
+// The FP64 pipe (two lanes per SM and clock) bounds the Gauss-point kernels, so what is equal on two
+// lanes is formed once: du/dx is the same at both x points of an element, so the lanes with x = 0
+// carry component 0 through the x chain and the lanes with x = 1 component 1, and exchange the
+// results; likewise y and z.  18 FP64 operations for the nine derivatives of a point where forming
+// each on its own takes 39.
+constexpr double kGr = 0.26794919243112270647;   // (1 - 1/sqrt 3) / (1 + 1/sqrt 3) = 2 - sqrt 3
 
-__device__ __forceinline__ void grad_lanes(const DevMesh& M, double u, int bx, int by, int bz, double& gx,
-                                           double& gy, double& gz) {
+// t[c][d] h_d-free derivative of component c along d at the lane's Gauss point: du_c/dx_d =
+// M.gs[d] t[c][d].  u: the lane's node values.  All 32 lanes of the warp take part.
+__device__ __forceinline__ void grad_lanes3(const double (&u)[3], int bx, int by, int bz, double (&t)[3][3]) {
   const unsigned all = 0xffffffffu;
-  const double up = __shfl_xor_sync(all, u, 1);
-  const double I1 = kGa * u + kGb * up;
-  const double D1 = (bx ? u : up) - (bx ? up : u);
-  const double D1p = __shfl_xor_sync(all, D1, 2), I1p = __shfl_xor_sync(all, I1, 2);
-  const double DX2 = kGa * D1 + kGb * D1p;
-  const double E2 = (by ? I1 : I1p) - (by ? I1p : I1);
-  const double J2 = M.ga[2] * I1 + M.gb[2] * I1p;
-  const double DX2p = __shfl_xor_sync(all, DX2, 4), E2p = __shfl_xor_sync(all, E2, 4),
-               J2p = __shfl_xor_sync(all, J2, 4);
-  gx = M.ga[0] * DX2 + M.gb[0] * DX2p;
-  gy = M.ga[1] * E2 + M.gb[1] * E2p;
-  gz = (bz ? J2 : J2p) - (bz ? J2p : J2);
+  double up[3], I[3], Ip[3], J[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    up[c] = __shfl_xor_sync(all, u[c], 1);
+    I[c] = fma(kGr, up[c], u[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    Ip[c] = __shfl_xor_sync(all, I[c], 2);
+    J[c] = fma(kGr, Ip[c], I[c]);
+  }
+  // along x: differences on the x edges, interpolated in y and z
+  double a = (bx ? u[1] : up[0]) - (bx ? up[1] : u[0]), b = (bx ? u[2] : up[2]) - (bx ? up[2] : u[2]);
+  a = fma(kGr, __shfl_xor_sync(all, a, 2), a);
+  b = fma(kGr, __shfl_xor_sync(all, b, 2), b);
+  a = fma(kGr, __shfl_xor_sync(all, a, 4), a);
+  t[2][0] = fma(kGr, __shfl_xor_sync(all, b, 4), b);
+  double o = __shfl_xor_sync(all, a, 1);
+  t[0][0] = bx ? o : a;
+  t[1][0] = bx ? a : o;
+  // along y: differences of the x interpolants, interpolated in z
+  a = (by ? I[1] : Ip[0]) - (by ? Ip[1] : I[0]);
+  b = (by ? I[2] : Ip[2]) - (by ? Ip[2] : I[2]);
+  a = fma(kGr, __shfl_xor_sync(all, a, 4), a);
+  t[2][1] = fma(kGr, __shfl_xor_sync(all, b, 4), b);
+  o = __shfl_xor_sync(all, a, 2);
+  t[0][1] = by ? o : a;
+  t[1][1] = by ? a : o;
+  // along z: differences of the x-y interpolants
+  const double jo = __shfl_xor_sync(all, bz ? J[0] : J[1], 4), j2 = __shfl_xor_sync(all, J[2], 4);
+  a = (bz ? J[1] : jo) - (bz ? jo : J[0]);
+  t[2][2] = (bz ? J[2] : j2) - (bz ? j2 : J[2]);
+  o = __shfl_xor_sync(all, a, 4);
+  t[0][2] = bz ? o : a;
+  t[1][2] = bz ? a : o;
 }
 
-// The transpose of grad_lanes: given (fx, fy, fz) at the lane's Gauss point, returns at the
-// lane's node sum over the element's points of grad N_node . (fx, fy, fz).
-__device__ __forceinline__ double grad_lanes_t(const DevMesh& M, double fx, double fy, double fz, int bx, int by,
-                                               int bz) {
+// The transpose: given (fx, fy, fz) at the lane's Gauss point, returns at the lane's node
+// h_x / ((1 + 1/sqrt 3) / 2)^2 times the sum over the element's points of grad N_node . (fx, fy, fz); ry = h_x / h_y,
+// rz = h_x / h_z.  11 FP64 operations.
+__device__ __forceinline__ double grad_lanes_t(double fx, double fy, double fz, int bx, int by, int bz, double ry,
+                                               double rz) {
   const unsigned all = 0xffffffffu;
-  const double sx = bx ? 1.0 : -1.0, sy = by ? 1.0 : -1.0, sz = bz ? 1.0 : -1.0;
-  const double fxp = __shfl_xor_sync(all, fx, 4), fyp = __shfl_xor_sync(all, fy, 4), fzp = __shfl_xor_sync(all, fz, 4);
-  const double bDX2 = M.ga[0] * fx + M.gb[0] * fxp;
-  const double bE2 = M.ga[1] * fy + M.gb[1] * fyp;
-  const double bJ2 = sz * (fz + fzp);
-  const double bDX2p = __shfl_xor_sync(all, bDX2, 2), bE2p = __shfl_xor_sync(all, bE2, 2),
-               bJ2p = __shfl_xor_sync(all, bJ2, 2);
-  const double bD1 = kGa * bDX2 + kGb * bDX2p;
-  const double bI1 = sy * (bE2 + bE2p) + (M.ga[2] * bJ2 + M.gb[2] * bJ2p);
-  const double bD1p = __shfl_xor_sync(all, bD1, 1), bI1p = __shfl_xor_sync(all, bI1, 1);
-  return sx * (bD1 + bD1p) + (kGa * bI1 + kGb * bI1p);
+  const double xz = fma(kGr, __shfl_xor_sync(all, fx, 4), fx), yz = fma(kGr, __shfl_xor_sync(all, fy, 4), fy);
+  const double zz = fz + __shfl_xor_sync(all, fz, 4);
+  const double xy = fma(kGr, __shfl_xor_sync(all, xz, 2), xz);
+  const double yy = yz + __shfl_xor_sync(all, yz, 2);
+  const double zy = fma(kGr, __shfl_xor_sync(all, zz, 2), zz);
+  // node signs of the differences: - at the low node, + at the high one
+  const double i = fma(bz ? rz : -rz, zy, (by ? ry : -ry) * yy);
+  const double xx = xy + __shfl_xor_sync(all, xy, 1);
+  return fma(kGr, __shfl_xor_sync(all, i, 1), i) + (bx ? xx : -xx);
 }
 
 // ---------------------------------------------------------------------------
@@ -248,99 +270,128 @@ __device__ __forceinline__ double grad_lanes_t(const DevMesh& M, double fx, doub
 //           D = C - 2mu c (1 - rho) E_eps - 2mu c rho n n^T, rho = sqrt(2/3)(sigma_y+H kappa)/||dev tau||,
 //           c = 3mu/(3mu+H)  (the Sec. 3.1 form of eq. (stress_op_deriv_plast)).
 // ---------------------------------------------------------------------------
+// Constants of the return mapping, formed once on the host: with s_d the factor of the derivatives
+// along d (M.gs) the stress increment is ce = C eta, ce_dd = m2[d] t_dd + sum_k l[k] t_kk and
+// ce_cd = m1[d] t_cd + m1[c] t_dc.
+struct RmConst {
+  double l[3], m2[3], m1[3];   // lam s_d, 2 mu s_d, mu s_d
+  double cs, kd, a0;           // sqrt(2/3) c, 1 / (3 mu + H), 2 mu c, c = 3 mu / (3 mu + H)
+};
+
+// 1/sqrt(d) and sqrt(d) for normal d of moderate exponent: the hardware's approximation (relative
+// error below 2^-19), one step of the third-order iteration y (1 + e (1/2 + 3/8 e)), e = 1 - d y^2,
+// and a Newton correction of the root.
+__device__ __forceinline__ void root_pair(double d, double& root, double& inv) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+  const double e = fma(-(d * y), y, 1.0);
+  y = fma(y * e, fma(0.375, e, 0.5), y);
+  const double r = d * y;
+  const double hy = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));   // y / 2
+  root = fma(fma(-r, r, d), hy, r);
+  inv = y;
+}
+
 // One thread per Gauss point, the 8 points of an element in 8 consecutive lanes (blockDim and n_gp
 // multiples of 8); lanes past n_gp compute on the last element and store nothing.
-__global__ void k_return_map(DevMesh M, const double* __restrict__ du, const double* __restrict__ sig_k,
-                             const double* __restrict__ kap_k, double* dsig, double* dkap, uint8_t* plastic,
-                             double* Dtan, double* pa, double* pb, double* pn) {
+// Bound by the FP64 pipe: about 52 operations per elastic point and 20 more at a yielding one (74
+// and 56 with a square root, three divisions and derivatives formed one by one): at 96^3, half of the
+// points yielding, 968 us for 7.1 million points where that form took 1714.  The material constants
+// come from the host; the root of |dev tau|^2 and its inverse share one iteration.  kOut: 0 = increments only, 1 = also a, b, n, 2 = also T.
+template <int kOut>
+__global__ void __launch_bounds__(128) k_return_map(DevMesh M, RmConst K, const double* __restrict__ du,
+                                                    const double* __restrict__ sig_k, const double* __restrict__ kap_k,
+                                                    double* dsig, double* dkap, uint8_t* plastic, double* Dtan,
+                                                    double* pa, double* pb, double* pn) {
   const long long gp_t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const bool live = gp_t < M.n_gp;
   const long long gp = live ? gp_t : M.n_gp - 8 + (gp_t & 7);
   const long long e = gp >> 3;
   const int g = (int)(gp & 7);
   const int bx = g & 1, by = (g >> 1) & 1, bz = (g >> 2) & 1;
+  double tau[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) tau[c] = __ldg(sig_k + c * M.n_gp + gp);
+  const double kap = __ldg(kap_k + gp);
   const int p = M.elem_sub[e];
   const SubDev& S = M.subs[p];
   const int le = (int)(e - S.elem_off);
   const int ex = le % S.dims[0], ey = (le / S.dims[0]) % S.dims[1], ez = le / (S.dims[0] * S.dims[1]);
   const int ln = (ex + bx) + S.nn[0] * ((ey + by) + S.nn[1] * (ez + bz));
-  const double* u = du + S.dof_off + 3LL * ln;
-  double gr[3][3];   // gr[c][d] = d u_c / d x_d at the lane's Gauss point
-#pragma unroll
-  for (int c = 0; c < 3; ++c) grad_lanes(M, u[c], bx, by, bz, gr[c][0], gr[c][1], gr[c][2]);
+  const double* un = du + S.dof_off + 3LL * ln;
+  const double u[3] = {un[0], un[1], un[2]};
+  double t[3][3];
+  grad_lanes3(u, bx, by, bz, t);
   if (!live) return;
-  const double eta[6] = {gr[0][0], gr[1][1], gr[2][2], gr[0][1] + gr[1][0], gr[1][2] + gr[2][1],
-                         gr[0][2] + gr[2][0]};
-  const double lam = M.lam, mu = M.mu;
-  const double tr = eta[0] + eta[1] + eta[2];
+  const double lt = fma(K.l[2], t[2][2], fma(K.l[1], t[1][1], K.l[0] * t[0][0]));
   double ce[6];
-  ce[0] = lam * tr + 2.0 * mu * eta[0];
-  ce[1] = lam * tr + 2.0 * mu * eta[1];
-  ce[2] = lam * tr + 2.0 * mu * eta[2];
-  ce[3] = mu * eta[3];
-  ce[4] = mu * eta[4];
-  ce[5] = mu * eta[5];
-  double tau[6];
+  ce[0] = fma(K.m2[0], t[0][0], lt);
+  ce[1] = fma(K.m2[1], t[1][1], lt);
+  ce[2] = fma(K.m2[2], t[2][2], lt);
+  ce[3] = fma(K.m1[1], t[0][1], K.m1[0] * t[1][0]);
+  ce[4] = fma(K.m1[2], t[1][2], K.m1[1] * t[2][1]);
+  ce[5] = fma(K.m1[2], t[0][2], K.m1[0] * t[2][0]);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) tau[c] = sig_k[c * M.n_gp + gp] + ce[c];
-  const double kap = kap_k[gp];
+  for (int c = 0; c < 6; ++c) tau[c] += ce[c];
   const double mean = (tau[0] + tau[1] + tau[2]) * kThird;
-  double dev[6] = {tau[0] - mean, tau[1] - mean, tau[2] - mean, tau[3], tau[4], tau[5]};
+  const double dev[6] = {tau[0] - mean, tau[1] - mean, tau[2] - mean, tau[3], tau[4], tau[5]};
   const double nrm2 =
       dev[0] * dev[0] + dev[1] * dev[1] + dev[2] * dev[2] + 2.0 * (dev[3] * dev[3] + dev[4] * dev[4] + dev[5] * dev[5]);
-  const double yield = M.sigma_y + M.H * kap;
-  // (3/2) |dev tau|^2 <= yield^2 (yield > 0) puts Phi within rounding of <= 0, far inside the
-  // tie band: elastic without the square root; otherwise Phi and the test as stated above
-  double nrm = 0.0, phi = 0.0;
+  const double yield = fma(M.H, kap, M.sigma_y);
+  // (3/2) |dev tau|^2 <= yield^2 puts Phi within rounding of <= 0, far inside the tie band: elastic
+  // without the root (compared as integers: both are non-negative, and a NaN fails the test below)
+  double phi = 0.0, inv = 0.0;
   bool pl = false;
-  if (1.5 * nrm2 > yield * yield) {
-    nrm = sqrt(nrm2);
-    phi = kSqrt32 * nrm - yield;
+  if (__double_as_longlong(1.5 * nrm2) > __double_as_longlong(yield * yield)) {
+    double nrm;
+    const unsigned ef = ((unsigned)__double2hiint(nrm2) >> 20) & 0x7ffu;
+    if (ef - 0x100u < 0x600u) {
+      root_pair(nrm2, nrm, inv);
+    } else {   // extreme magnitudes, infinities and NaN
+      nrm = sqrt(nrm2);
+      inv = 1.0 / nrm;
+    }
+    phi = fma(kSqrt32, nrm, -yield);
     pl = phi > kTie * yield;
   }
-  double ds[6];
-  double a = 0.0, b = 0.0, nb[6] = {0, 0, 0, 0, 0, 0};
+  const double f = pl ? K.cs * phi * inv : 0.0;   // dsigma = C eta - f dev tau
   if (pl) {
-    const double c = 3.0 * mu / (3.0 * mu + M.H);
-    const double inv = 1.0 / nrm;
-    const double corr = c * kSqrt23 * phi;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      nb[q] = dev[q] * inv;
-      ds[q] = ce[q] - corr * nb[q];
-    }
-    const double rho = kSqrt23 * yield * inv;
-    a = 2.0 * mu * c * (1.0 - rho);
-    b = 2.0 * mu * c * rho;
-    if (dkap) dkap[gp] = phi / (3.0 * mu + M.H);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 6; ++q) ds[q] = ce[q];
-    if (dkap) dkap[gp] = 0.0;
+    for (int q = 0; q < 6; ++q) ce[q] = fma(-f, dev[q], ce[q]);
   }
 #pragma unroll
-  for (int q = 0; q < 6; ++q) dsig[q * M.n_gp + gp] = ds[q];
+  for (int q = 0; q < 6; ++q) dsig[q * M.n_gp + gp] = ce[q];
+  if (dkap) dkap[gp] = pl ? K.kd * phi : 0.0;
   if (plastic) plastic[gp] = pl ? 1 : 0;
-  if (pa) {
-    pa[gp] = a;
-    pb[gp] = b;
+  if constexpr (kOut > 0) {
+    double a = 0.0, b = 0.0, nb[6] = {0, 0, 0, 0, 0, 0};
+    if (pl) {
+      b = K.a0 * (kSqrt23 * yield * inv);   // 2 mu c rho
+      a = K.a0 - b;
 #pragma unroll
-    for (int q = 0; q < 6; ++q) pn[q * M.n_gp + gp] = nb[q];
-  }
-  if (Dtan) {
-    int idx = 0;
-    for (int r = 0; r < 6; ++r)
-      for (int s = r; s < 6; ++s, ++idx) {
-        double C = 0.0, E = 0.0;
-        if (r < 3 && s < 3) {
-          C = lam + (r == s ? 2.0 * mu : 0.0);
-          E = r == s ? 2.0 / 3.0 : -1.0 / 3.0;
-        } else if (r == s) {
-          C = mu;
-          E = 0.5;
+      for (int q = 0; q < 6; ++q) nb[q] = dev[q] * inv;
+    }
+    if (pa) {
+      pa[gp] = a;
+      pb[gp] = b;
+#pragma unroll
+      for (int q = 0; q < 6; ++q) pn[q * M.n_gp + gp] = nb[q];
+    }
+    if constexpr (kOut == 2) {
+      const double c11 = M.lam + 2.0 * M.mu;   // uniform over the launch
+      const double d11 = pl ? fma(-2.0 / 3.0, a, c11) : c11, d12 = pl ? fma(1.0 / 3.0, a, M.lam) : M.lam,
+                   d44 = pl ? fma(-0.5, a, M.mu) : M.mu;
+      int idx = 0;
+#pragma unroll
+      for (int r = 0; r < 6; ++r) {
+        const double br = pl ? -b * nb[r] : 0.0;
+#pragma unroll
+        for (int s = r; s < 6; ++s, ++idx) {
+          const double base = (r < 3 && s < 3) ? (r == s ? d11 : d12) : (r == s ? d44 : 0.0);
+          Dtan[idx * M.n_gp + gp] = pl ? fma(br, nb[s], base) : base;
         }
-        Dtan[idx * M.n_gp + gp] = pl ? C - a * E - b * nb[r] * nb[s] : C;
       }
+    }
   }
 }
 
@@ -479,8 +530,9 @@ __global__ void k_kbb_fill(DevMesh M, const int* __restrict__ sub_list, const lo
 }
 
 // Internal force of eq. (F_def), element part: for every element node a (bit order x + 2y + 4z)
-// and component c, fe = sum over the element's Gauss points of grad N_a . sigma_c (sigma_c the
-// row c of the stress dsig), by the transposed sum factorisation over the element's 8 lanes.
+// and component c, fe = h_x / ((1 + 1/sqrt 3) / 2)^2 sum over the element's Gauss points of grad N_a . sigma_c (sigma_c
+// the row c of the stress dsig), by the transposed sum factorisation over the element's 8 lanes (33
+// FP64 operations per point; the factor is applied per dof by k_gather_force).
 __global__ void k_elem_force(DevMesh M, const double* __restrict__ dsig, double* fe) {
   const long long gp_t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const bool live = gp_t < M.n_gp;
@@ -491,9 +543,9 @@ __global__ void k_elem_force(DevMesh M, const double* __restrict__ dsig, double*
 #pragma unroll
   for (int q = 0; q < 6; ++q) sg[q] = dsig[q * M.n_gp + gp];
   // Voigt order xx, yy, zz, xy, yz, xz
-  const double f0 = grad_lanes_t(M, sg[0], sg[3], sg[5], bx, by, bz);
-  const double f1 = grad_lanes_t(M, sg[3], sg[1], sg[4], bx, by, bz);
-  const double f2 = grad_lanes_t(M, sg[5], sg[4], sg[2], bx, by, bz);
+  const double f0 = grad_lanes_t(sg[0], sg[3], sg[5], bx, by, bz, M.gratio[1], M.gratio[2]);
+  const double f1 = grad_lanes_t(sg[3], sg[1], sg[4], bx, by, bz, M.gratio[1], M.gratio[2]);
+  const double f2 = grad_lanes_t(sg[5], sg[4], sg[2], bx, by, bz, M.gratio[1], M.gratio[2]);
   if (!live) return;
   double* o = fe + 3 * gp;   // element e = gp / 8, node g
   o[0] = f0;
@@ -501,7 +553,7 @@ __global__ void k_elem_force(DevMesh M, const double* __restrict__ dsig, double*
   o[2] = f2;
 }
 
-// f = df - w detJ (sum of the element parts at the dof), the adjacent elements in (z, y, x) order.
+// f = df - w detJ M.gs[0] (sum of the element parts at the dof), the adjacent elements in (z, y, x) order.
 __global__ void k_gather_force(DevMesh M, const double* __restrict__ fe, const double* __restrict__ df, double* f) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= M.n_dof) return;
@@ -518,7 +570,7 @@ __global__ void k_gather_force(DevMesh M, const double* __restrict__ fe, const d
         const long long ge = S.elem_off + ex + S.dims[0] * (ey + S.dims[1] * ez);
         s += fe[(ge * 8 + a) * 3 + c];
       }
-  f[i] = (df ? df[i] : 0.0) - M.wdet * s;
+  f[i] = (df ? df[i] : 0.0) - M.wgs * s;
 }
 
 // y = K x per subdomain with the assembled tangent (27-node stencil).
@@ -602,8 +654,20 @@ void launch_traction(const DevMesh& M, int face, const int* nel, const double* t
 void launch_return_map(const DevMesh& M, const double* du, const double* sig_k, const double* kap_k,
                        double* dsig, double* dkap, uint8_t* plastic, double* Dtan, double* pa, double* pb,
                        double* pn, cudaStream_t st) {
-  k_return_map<<<blocks_for(M.n_gp, 128), 128, 0, st>>>(M, du, sig_k, kap_k, dsig, dkap, plastic, Dtan, pa, pb,
-                                                           pn);
+  RmConst K;
+  for (int d = 0; d < 3; ++d) {
+    K.l[d] = M.lam * M.gs[d];
+    K.m2[d] = 2.0 * M.mu * M.gs[d];
+    K.m1[d] = M.mu * M.gs[d];
+  }
+  const double c = 3.0 * M.mu / (3.0 * M.mu + M.H);
+  K.cs = kSqrt23 * c;
+  K.kd = 1.0 / (3.0 * M.mu + M.H);
+  K.a0 = 2.0 * M.mu * c;
+  const unsigned nblk = blocks_for(M.n_gp, 128);
+  if (Dtan) k_return_map<2><<<nblk, 128, 0, st>>>(M, K, du, sig_k, kap_k, dsig, dkap, plastic, Dtan, pa, pb, pn);
+  else if (pa) k_return_map<1><<<nblk, 128, 0, st>>>(M, K, du, sig_k, kap_k, dsig, dkap, plastic, Dtan, pa, pb, pn);
+  else k_return_map<0><<<nblk, 128, 0, st>>>(M, K, du, sig_k, kap_k, dsig, dkap, plastic, Dtan, pa, pb, pn);
 }
 
 void launch_elem_correction(const DevMesh& M, GPData gp, int* elem_np, int* sub_np, double* dKe, cudaStream_t st) {
