@@ -595,7 +595,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
     if (ok) ok = mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1));
   };
   auto wait_exchange = [&](int e) {
-    if (ok) ok = mbar_wait(&xbar[e % kClRing], (uint32_t)((e / kClRing) & 1));
+    if (ok) ok = mbar_wait_cluster(&xbar[e % kClRing], (uint32_t)((e / kClRing) & 1));
   };
   int issued = 0;
   if (tid == 0)
@@ -655,6 +655,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
     if (tid == 0 && b > 0) mbar_expect_tx(&xbar[k % kClRing], (uint32_t)(nb * R * (int)sizeof(T)));
     // z' of the own rows: y less the CTAs' sums (lane = CTA x row), in every warp
     if (k > nblk) wait_exchange(k - 1);
+    T zv[R];
     {
       const int t = lane % rpc, c = lane / rpc, gr = r0 + (int)q * rpc + t;
 #pragma unroll
@@ -664,9 +665,8 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
         if (lane < rpc) {
           v = gr < n ? vec[r * npad + gr] - v : T(0);
           s_z[warp][t][r] = v;
-          // the block's D^-T (below) runs in CTA b % C
-          if (warp == 0 && gr < n) st_cluster(vec + r * npad + gr, (unsigned)(b % C), v);
         }
+        zv[r] = v;
       }
     }
     __syncwarp();
@@ -699,6 +699,11 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
       }
     }
     __syncthreads();
+    // z' to CTA b % C, which applies the block's D^-T below (only now: until here every warp of that CTA
+    // may still read the y of its own rows from the same entries)
+    if (warp == 0 && lane < rpc && r0 + (int)q * rpc + lane < n)
+#pragma unroll
+      for (int r = 0; r < R; ++r) st_cluster(vec + r * npad + r0 + (int)q * rpc + lane, (unsigned)(b % C), zv[r]);
     if (tid == 0 && ok && issued < nsteps) fetch(issued++);
   }
   if (!ok) atomicOr(a.err, 2);
