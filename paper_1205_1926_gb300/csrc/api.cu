@@ -2494,11 +2494,13 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   M.helm = upload(c, helm);
   double* dN = dalloc<double>(c, 8 * 8 * 3);
   double* Kel = dalloc<double>(c, 576);
-  double* Q = dalloc<double>(c, 8 * 576);
   double* R = dalloc<double>(c, P.r_total);
   M.dN = dN;
   M.Kel = Kel;
-  M.Q = Q;
+  double* Qt = dalloc<double>(c, 8 * kTri24);
+  double* Kst = dalloc<double>(c, 27 * 27 * 9);
+  M.Qt = Qt;
+  M.Kst = Kst;
   M.R = R;
   const double lam = pr.young * pr.poisson / ((1.0 + pr.poisson) * (1.0 - 2.0 * pr.poisson));
   const double mu = pr.young / (2.0 * (1.0 + pr.poisson));
@@ -2519,7 +2521,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   M.n_copy = P.n_copy;
   M.n_groups = (long long)gd.size();
   M.n_elem = P.n_elem;
-  launch_tables(P.h, lam, mu, dN, Kel, Q, c->st);
+  launch_tables(P.h, lam, mu, dN, Kel, Qt, Kst, c->st);
   for (const ShapeInfo& sh : P.shapes) launch_rigid_for_shape(c->h_subs[sh.rep_sub], P.h, R + sh.r_off, c->st);
   c->launches += 1 + (long long)P.shapes.size();
   {

@@ -67,7 +67,8 @@ struct DevMesh {
   const double* R;         // rigid-body bases per shape, [n_dof][6] row-major
   const double* dN;        // [8 g][8 a][3] physical shape-function gradients
   const double* Kel;       // [24][24] elastic brick stiffness
-  const double* Q;         // [8 g][24][24] w detJ B_g^T E_eps B_g
+  const double* Qt;        // [8 g][300] w detJ B_g^T E_eps B_g, packed lower triangles
+  const double* Kst;       // [27 node types][27 neighbours][9] assembled elastic stencils (kernels_fem.cu)
   const double* helm;      // [8 r][8 j] Helmert coefficients (row r = 1..7, copy j)
   // G = R^T B^T explicitly (it depends only on B and R): one entry per (multiplier
   // row, copy slot) with B[row][slot] != 0, value B[row][slot] * R[slot dof][0..5].
@@ -102,7 +103,8 @@ struct GPData {
 };
 
 // ---- launchers (all enqueue on `st`) -------------------------------------
-void launch_tables(const double* h, double lam, double mu, double* dN, double* Kel, double* Q, cudaStream_t st);
+void launch_tables(const double* h, double lam, double mu, double* dN, double* Kel, double* Qt, double* Kst,
+                   cudaStream_t st);
 void launch_rigid_for_shape(const SubDev& S, const double* h, double* R_shape, cudaStream_t st);
 void launch_traction(const DevMesh& M, int face, const int* nel, const double* t, const double* h, double* f,
                      cudaStream_t st);

@@ -38,7 +38,7 @@ __device__ __forceinline__ int find_sub(const SubDev* subs, int n_sub, long long
 // the elastic brick stiffness and w detJ B_g^T E_eps B_g (eq. (K_def) pieces).
 // ---------------------------------------------------------------------------
 __global__ void k_tables(double h0, double h1, double h2, double lam, double mu, double* dN, double* Kel,
-                         double* Q) {
+                         double* Qt) {
   __shared__ double B[8][6][24];
   __shared__ double dn[8][8][3];
   const double hh[3] = {h0, h1, h2};
@@ -100,8 +100,32 @@ __global__ void k_tables(double h0, double h1, double h2, double lam, double mu,
       const int g = which - 1;
       for (int r = 0; r < 6; ++r)
         for (int q = 0; q < 6; ++q) s += B[g][r][i] * E[r][q] * B[g][q][j];
-      Q[(size_t)g * 576 + i * 24 + j] = wdet * s;
+      if (j <= i) Qt[(size_t)g * kTri24 + tri_index(i, j)] = wdet * s;
     }
+  }
+}
+
+// Assembled elastic stencils: for a node whose position along each axis of its box is low (an element on its
+// high side only), inner or high (types 0, 1, 2 per axis, type tx + 3 ty + 9 tz) the 27 neighbour blocks
+// Kst[type][neighbour (dx + 1) + 3 (dy + 1) + 9 (dz + 1)][3 a + c], the sum of Kel over the adjacent elements that
+// hold both nodes.
+__global__ void k_stencils(const double* __restrict__ Kel, double* Kst) {
+  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < 27 * 27 * 9; idx += gridDim.x * blockDim.x) {
+    const int k = idx % 9, nbr = (idx / 9) % 27, type = idx / 243;
+    const int t[3] = {type % 3, (type / 3) % 3, type / 9}, d[3] = {nbr % 3 - 1, (nbr / 3) % 3 - 1, nbr / 9 - 1};
+    double s = 0.0;
+    for (int o = 0; o < 8; ++o) {   // element on the low (bit set) or high side of the node along each axis
+      int a = 0, b = 0;
+      bool in = true;
+      for (int x = 0; x < 3; ++x) {
+        const int low = (o >> x) & 1, other = d[x] + low;   // local coordinates of the node (low) and the neighbour
+        in = in && (low ? t[x] != 0 : t[x] != 2) && other >= 0 && other <= 1;
+        a += low << x;
+        b += other << x;
+      }
+      if (in) s += Kel[(3 * c_off2local[a] + k / 3) * 24 + 3 * c_off2local[b] + k % 3];
+    }
+    Kst[idx] = s;
   }
 }
 
@@ -397,79 +421,94 @@ __global__ void __launch_bounds__(128) k_return_map(DevMesh M, RmConst K, const 
 
 // ---------------------------------------------------------------------------
 // Element tangent correction dK_e = sum_{plastic g} (a_g Q_g + w detJ b_g v_g v_g^T),
-// v_g = B_g^T n_g.  K_e = K_el - dK_e.  One warp per element.
+// v_g = B_g^T n_g.  K_e = K_el - dK_e.  A warp looks through four elements (lane = 8 element + point)
+// and works on the ones with plastic points together: two FMAs per point and entry of the packed lower
+// triangle, bound by the FP64 pipe (4800 of them for an element that yields everywhere).
 // ---------------------------------------------------------------------------
-__global__ void k_elem_correction(DevMesh M, GPData gd, int* elem_np, int* sub_np, double* dKe) {
-  __shared__ double v[8][8][24];  // [warp][g][i]
+__global__ void __launch_bounds__(256) k_elem_correction(DevMesh M, GPData gd, int* elem_np, int* sub_np, double* dKe) {
+  __shared__ double v[8][8][24], bv[8][8][24];  // [warp][g][i]: v_g and w detJ b_g v_g
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long e = blockIdx.x * (long long)(blockDim.x >> 5) + warp;
-  if (e >= M.n_elem) return;
-  const long long gp0 = e * 8;
-  int flag = 0;
-  if (lane < 8) flag = gd.plastic[gp0 + lane];
-  const unsigned mask = __ballot_sync(0xffffffffu, flag != 0);
-  const int cnt = __popc(mask);
-  if (lane == 0) {
-    elem_np[e] = cnt;
-    if (cnt) atomicAdd(&sub_np[M.elem_sub[e]], cnt);
+  const long long e0 = 4 * (blockIdx.x * (long long)(blockDim.x >> 5) + warp);
+  if (e0 >= M.n_elem) return;
+  const int flag = e0 + (lane >> 3) < M.n_elem ? gd.plastic[e0 * 8 + lane] : 0;
+  const unsigned all = __ballot_sync(0xffffffffu, flag != 0);
+  if ((lane & 7) == 0 && e0 + (lane >> 3) < M.n_elem) {
+    const int cnt = __popc((all >> lane) & 0xffu);
+    elem_np[e0 + (lane >> 3)] = cnt;
+    if (cnt) atomicAdd(&sub_np[M.elem_sub[e0 + (lane >> 3)]], cnt);
   }
-  if (!cnt) return;
-  if (lane < 8 && flag) {
-    const long long gp = gp0 + lane;
-    double n[6];
+  for (int k = 0; k < 4; ++k) {
+    const unsigned mask = (all >> (8 * k)) & 0xffu;
+    if (!mask) continue;
+    const long long gp0 = (e0 + k) * 8;
+    __syncwarp();
+    // lane = point + 8 x node pair: B_g^T n_g at nodes 2 (lane / 8), 2 (lane / 8) + 1
+    if ((mask >> (lane & 7)) & 1u) {
+      const int g = lane & 7;
+      const long long gp = gp0 + g;
+      const double wb = M.wdet * gd.pb[gp];
+      double n[6];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) n[q] = gd.pn[q * M.n_gp + gp];
-    const double* dn = M.dN + lane * 24;
-    for (int a = 0; a < 8; ++a) {
-      const double dx = dn[3 * a], dy = dn[3 * a + 1], dz = dn[3 * a + 2];
-      v[warp][lane][3 * a + 0] = dx * n[0] + dy * n[3] + dz * n[5];
-      v[warp][lane][3 * a + 1] = dy * n[1] + dx * n[3] + dz * n[4];
-      v[warp][lane][3 * a + 2] = dz * n[2] + dy * n[4] + dx * n[5];
+      for (int q = 0; q < 6; ++q) n[q] = gd.pn[q * M.n_gp + gp];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int a = 2 * (lane >> 3) + h;
+        const double* dn = M.dN + g * 24 + 3 * a;
+        const double dx = dn[0], dy = dn[1], dz = dn[2];
+        const double w[3] = {dx * n[0] + dy * n[3] + dz * n[5], dy * n[1] + dx * n[3] + dz * n[4],
+                             dz * n[2] + dy * n[4] + dx * n[5]};
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          v[warp][g][3 * a + c] = w[c];
+          bv[warp][g][3 * a + c] = wb * w[c];
+        }
+      }
     }
-  }
-  __syncwarp();
-  double ag[8], bg[8];
+    __syncwarp();
+    double ag[8];
 #pragma unroll
-  for (int g = 0; g < 8; ++g) {
-    const bool pl = (mask >> g) & 1u;
-    ag[g] = pl ? gd.pa[gp0 + g] : 0.0;
-    bg[g] = pl ? M.wdet * gd.pb[gp0 + g] : 0.0;
-  }
-  for (int idx = lane; idx < kTri24; idx += 32) {
-    int i = 0;
-    while ((i + 1) * (i + 2) / 2 <= idx) ++i;
-    const int j = idx - i * (i + 1) / 2;
-    double s = 0.0;
+    for (int g = 0; g < 8; ++g) ag[g] = (mask >> g) & 1u ? gd.pa[gp0 + g] : 0.0;
+    for (int idx = lane; idx < kTri24; idx += 32) {
+      int i = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+      while (i * (i + 1) / 2 > idx) --i;
+      while ((i + 1) * (i + 2) / 2 <= idx) ++i;
+      const int j = idx - i * (i + 1) / 2;
+      double s = 0.0;
 #pragma unroll
-    for (int g = 0; g < 8; ++g)
-      if ((mask >> g) & 1u) s += ag[g] * M.Q[g * 576 + i * 24 + j] + bg[g] * v[warp][g][i] * v[warp][g][j];
-    dKe[e * kTri24 + idx] = s;
+      for (int g = 0; g < 8; ++g)
+        if ((mask >> g) & 1u) s = fma(bv[warp][g][i], v[warp][g][j], fma(ag[g], __ldg(M.Qt + g * kTri24 + idx), s));
+      dKe[(e0 + k) * kTri24 + idx] = s;
+    }
   }
 }
 
-// K entry (true tangent) between local dofs r and c of subdomain S.
-__device__ double stiffness_entry(const DevMesh& M, const SubDev& S, const int* elem_np, const double* dKe, int r,
-                                  int c, bool elastic_only) {
-  const int nr = r / 3, ar = r % 3, nc = c / 3, ac = c % 3;
-  const int ri = nr % S.nn[0], rj = (nr / S.nn[0]) % S.nn[1], rk = nr / (S.nn[0] * S.nn[1]);
-  const int ci = nc % S.nn[0], cj = (nc / S.nn[0]) % S.nn[1], ck = nc / (S.nn[0] * S.nn[1]);
-  if (abs(ri - ci) > 1 || abs(rj - cj) > 1 || abs(rk - ck) > 1) return 0.0;
-  double sum = 0.0;
-  const int ex0 = max(max(ri, ci) - 1, 0), ex1 = min(min(ri, ci), S.dims[0] - 1);
-  const int ey0 = max(max(rj, cj) - 1, 0), ey1 = min(min(rj, cj), S.dims[1] - 1);
-  const int ez0 = max(max(rk, ck) - 1, 0), ez1 = min(min(rk, ck), S.dims[2] - 1);
-  for (int ez = ez0; ez <= ez1; ++ez)
-    for (int ey = ey0; ey <= ey1; ++ey)
-      for (int ex = ex0; ex <= ex1; ++ex) {
-        const int a = c_off2local[(ri - ex) + 2 * (rj - ey) + 4 * (rk - ez)];
-        const int b = c_off2local[(ci - ex) + 2 * (cj - ey) + 4 * (ck - ez)];
-        const int i = 3 * a + ar, j = 3 * b + ac;
-        double v = M.Kel[i * 24 + j];
-        if (!elastic_only) {
-          const long long ge = S.elem_off + ex + S.dims[0] * (ey + S.dims[1] * ez);
-          if (elem_np[ge]) v -= dKe[ge * kTri24 + tri_index(i, j)];
-        }
-        sum += v;
+// Stencil type of the node at (i, j, k) of a box with nn nodes per axis (see k_stencils).
+__device__ __forceinline__ int node_type(const SubDev& S, int i, int j, int k) {
+  return (i == 0 ? 0 : (i == S.nn[0] - 1 ? 2 : 1)) + 3 * (j == 0 ? 0 : (j == S.nn[1] - 1 ? 2 : 1)) +
+         9 * (k == 0 ? 0 : (k == S.nn[2] - 1 ? 2 : 1));
+}
+
+// K entry (true tangent) between component a of node r and component c of its neighbour r + d (inside the box):
+// the elastic stencil less the corrections of the elements with plastic points that hold both nodes.
+__device__ double stiffness_entry(const DevMesh& M, const SubDev& S, const int* elem_np, const double* dKe,
+                                  const int (&r)[3], const int (&d)[3], int a, int c, bool elastic_only) {
+  double sum = __ldg(M.Kst + (node_type(S, r[0], r[1], r[2]) * 27 + (d[0] + 1) + 3 * (d[1] + 1) + 9 * (d[2] + 1)) * 9 +
+                     3 * a + c);
+  if (elastic_only) return sum;
+  int lo[3], hi[3];
+#pragma unroll
+  for (int x = 0; x < 3; ++x) {
+    lo[x] = max(max(r[x], r[x] + d[x]) - 1, 0);
+    hi[x] = min(min(r[x], r[x] + d[x]), S.dims[x] - 1);
+  }
+  for (int ez = lo[2]; ez <= hi[2]; ++ez)
+    for (int ey = lo[1]; ey <= hi[1]; ++ey)
+      for (int ex = lo[0]; ex <= hi[0]; ++ex) {
+        const long long ge = S.elem_off + ex + S.dims[0] * (ey + S.dims[1] * ez);
+        if (!elem_np[ge]) continue;
+        const int na = c_off2local[(r[0] - ex) + 2 * (r[1] - ey) + 4 * (r[2] - ez)];
+        const int nc = c_off2local[(r[0] + d[0] - ex) + 2 * (r[1] + d[1] - ey) + 4 * (r[2] + d[2] - ez)];
+        sum -= dKe[ge * kTri24 + tri_index(3 * na + a, 3 * nc + c)];
       }
   return sum;
 }
@@ -478,31 +517,44 @@ __device__ double stiffness_entry(const DevMesh& M, const SubDev& S, const int* 
 // band[r*(bw+1) + k] = K[r][r - bw + k] (lower band, row-major).
 // With bmask == null the six fixing dofs of Remark 1 get identity rows and columns
 // (K_rr of the generalised inverse); with bmask the dofs marked in it do (K_ii of the
-// Dirichlet preconditioner: the constrained nodes eliminated, Sec. 4.2).
+// Dirichlet preconditioner: the constrained nodes eliminated, Sec. 4.2).  The band is cleared first;
+// then one thread per (node, neighbour not after it, component pair) writes the stencil's entries: 126
+// per node instead of an index decode for every of the 3 (bw + 1) band entries.
+__global__ void k_band_clear(DevMesh M, const int* __restrict__ sub_list, double* band,
+                             const long long* __restrict__ band_off_list) {
+  const SubDev& S = M.subs[sub_list[blockIdx.y]];
+  double* b = band + band_off_list[blockIdx.y];
+  const long long total = (long long)S.n_dof * (S.bw + 1);
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
+    b[i] = 0.0;
+}
+
 __global__ void k_band_fill(DevMesh M, const int* __restrict__ sub_list, const int* elem_np, const double* dKe,
                             double* band, const long long* __restrict__ band_off_list, int elastic_only,
                             const uint8_t* __restrict__ bmask) {
   const int item = blockIdx.y;
   const int p = sub_list[item];
   const SubDev& S = M.subs[p];
-  const long long total = (long long)S.n_dof * (S.bw + 1);
-  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  const int r = (int)(idx / (S.bw + 1)), k = (int)(idx % (S.bw + 1));
-  const int c = r - S.bw + k;
-  double v = 0.0;
-  if (c >= 0) {
-    bool fixed = false;
-    if (bmask) {
-      fixed = bmask[S.dof_off + r] | bmask[S.dof_off + c];
-    } else {
+  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const int node = idx / 126, m = (idx / 9) % 14, k = idx % 9;   // neighbours 0..13: those not after the node
+  if (node >= S.n_dof / 3) return;
+  const int r[3] = {node % S.nn[0], (node / S.nn[0]) % S.nn[1], node / (S.nn[0] * S.nn[1])};
+  const int d[3] = {m % 3 - 1, (m / 3) % 3 - 1, m / 9 - 1};
 #pragma unroll
-      for (int t = 0; t < 6; ++t) fixed |= (S.fix[t] == r) | (S.fix[t] == c);
-    }
-    if (fixed) v = (r == c) ? 1.0 : 0.0;
-    else v = stiffness_entry(M, S, elem_np, dKe, r, c, elastic_only != 0);
+  for (int x = 0; x < 3; ++x)
+    if (r[x] + d[x] < 0 || r[x] + d[x] >= S.nn[x]) return;
+  const int row = 3 * node + k / 3, col = 3 * (node + d[0] + S.nn[0] * (d[1] + S.nn[1] * d[2])) + k % 3;
+  if (col > row) return;
+  bool fixed = false;
+  if (bmask) {
+    fixed = bmask[S.dof_off + row] | bmask[S.dof_off + col];
+  } else {
+#pragma unroll
+    for (int t = 0; t < 6; ++t) fixed |= (S.fix[t] == row) | (S.fix[t] == col);
   }
-  band[band_off_list[item] + idx] = v;
+  if (fixed && row != col) return;
+  band[band_off_list[item] + (long long)row * (S.bw + 1) + S.bw - (row - col)] =
+      fixed ? 1.0 : stiffness_entry(M, S, elem_np, dKe, r, d, k / 3, k % 3, elastic_only != 0);
 }
 
 // Lumped-preconditioner blocks of one subdomain (or its shape's elastic template):
@@ -521,9 +573,10 @@ __global__ void k_kbb_fill(DevMesh M, const int* __restrict__ sub_list, const lo
   const int nu = M.shape_tnbr[(S.bnd_off + b) * 27 + t];
   double v = 0.0;
   if (nu >= 0) {
-    const int r = 3 * M.shape_bln[S.bnd_off + b] + a;
-    const int c = 3 * M.shape_bln[S.bnd_off + nu] + cc;
-    v = stiffness_entry(M, S, elem_np, dKe, r, c, elastic_only != 0);
+    const int nr_ = M.shape_bln[S.bnd_off + b], nc = M.shape_bln[S.bnd_off + nu];
+    const int r[3] = {nr_ % S.nn[0], (nr_ / S.nn[0]) % S.nn[1], nr_ / (S.nn[0] * S.nn[1])};
+    const int d[3] = {nc % S.nn[0] - r[0], (nc / S.nn[0]) % S.nn[1] - r[1], nc / (S.nn[0] * S.nn[1]) - r[2]};
+    v = stiffness_entry(M, S, elem_np, dKe, r, d, a, cc, elastic_only != 0);
   }
   kbb[dst_off[blockIdx.y] + idx] = v;
   if (kbb32) kbb32[dst_off[blockIdx.y] + idx] = (float)v;
@@ -573,27 +626,59 @@ __global__ void k_gather_force(DevMesh M, const double* __restrict__ fe, const d
   f[i] = (df ? df[i] : 0.0) - M.wgs * s;
 }
 
-// y = K x per subdomain with the assembled tangent (27-node stencil).
-__global__ void k_apply_K(DevMesh M, const int* elem_np, const double* dKe, const double* __restrict__ x,
-                          double* y) {
+// y = K x per subdomain with the assembled tangent, one thread per node: the elastic 27-node stencil of the
+// node's type (243 FMAs for its three rows, bound by the FP64 pipe; the coefficients, mostly the same for a
+// warp, come from L1), less the corrections of the adjacent elements with plastic points.
+__global__ void __launch_bounds__(128) k_apply_K(DevMesh M, const int* __restrict__ elem_np,
+                                                 const double* __restrict__ dKe, const double* __restrict__ x,
+                                                 double* y) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= M.n_dof) return;
-  const int p = find_sub(M.subs, M.n_sub, i);
+  if (3 * i >= M.n_dof) return;
+  const int p = find_sub(M.subs, M.n_sub, 3 * i);
   const SubDev& S = M.subs[p];
-  const int r = (int)(i - S.dof_off);
-  const int node = r / 3;
-  const int li = node % S.nn[0], lj = (node / S.nn[0]) % S.nn[1], lk = node / (S.nn[0] * S.nn[1]);
-  double s = 0.0;
+  const int n0 = S.nn[0], n1 = S.nn[1];
+  const int node = (int)(i - S.dof_off / 3);
+  const int li = node % n0, lj = (node / n0) % n1, lk = node / (n0 * n1);
+  const double* xs = x + S.dof_off;
+  const double* kt = M.Kst + node_type(S, li, lj, lk) * 243;
+  double s[3] = {0.0, 0.0, 0.0};
   for (int dz = -1; dz <= 1; ++dz)
-    for (int dy = -1; dy <= 1; ++dy)
+    for (int dy = -1; dy <= 1; ++dy) {
+      const int b = lj + dy, c = lk + dz;
+      if (b < 0 || c < 0 || b >= n1 || c >= S.nn[2]) continue;
+#pragma unroll
       for (int dx = -1; dx <= 1; ++dx) {
-        const int a = li + dx, b = lj + dy, c = lk + dz;
-        if (a < 0 || b < 0 || c < 0 || a >= S.nn[0] || b >= S.nn[1] || c >= S.nn[2]) continue;
-        const int nn = a + S.nn[0] * (b + S.nn[1] * c);
+        const bool in = li + dx >= 0 && li + dx < n0;
+        const double* xn = xs + 3 * (in ? li + dx + n0 * (b + n1 * c) : node);
+        const double* kb = kt + ((dx + 1) + 3 * (dy + 1) + 9 * (dz + 1)) * 9;   // zero where there is no neighbour
+        const double v[3] = {__ldg(xn), __ldg(xn + 1), __ldg(xn + 2)};
+#pragma unroll
         for (int q = 0; q < 3; ++q)
-          s += stiffness_entry(M, S, elem_np, dKe, r, 3 * nn + q, false) * x[S.dof_off + 3 * nn + q];
+#pragma unroll
+          for (int r = 0; r < 3; ++r)
+            if (in) s[r] = fma(__ldg(kb + 3 * r + q), v[q], s[r]);
       }
-  y[i] = s;
+    }
+  for (int ez = max(lk - 1, 0); ez <= min(lk, S.dims[2] - 1); ++ez)
+    for (int ey = max(lj - 1, 0); ey <= min(lj, S.dims[1] - 1); ++ey)
+      for (int ex = max(li - 1, 0); ex <= min(li, S.dims[0] - 1); ++ex) {
+        const long long ge = S.elem_off + ex + S.dims[0] * (ey + S.dims[1] * ez);
+        if (!elem_np[ge]) continue;
+        const double* dk = dKe + ge * kTri24;
+        const int na = c_off2local[(li - ex) + 2 * (lj - ey) + 4 * (lk - ez)];
+        for (int o = 0; o < 8; ++o) {
+          const int nb = c_off2local[o];
+          const double* xn = xs + 3 * (ex + (o & 1) + n0 * (ey + ((o >> 1) & 1) + n1 * (ez + (o >> 2))));
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const double v = __ldg(xn + q);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) s[r] = fma(-__ldg(dk + tri_index(3 * na + r, 3 * nb + q)), v, s[r]);
+          }
+        }
+      }
+#pragma unroll
+  for (int r = 0; r < 3; ++r) y[3 * i + r] = s[r];
 }
 
 __global__ void k_commit(long long n_dof, long long n_gp, const double* du, const double* dsig,
@@ -637,8 +722,10 @@ inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) /
 
 }  // namespace
 
-void launch_tables(const double* h, double lam, double mu, double* dN, double* Kel, double* Q, cudaStream_t st) {
-  k_tables<<<1, 256, 0, st>>>(h[0], h[1], h[2], lam, mu, dN, Kel, Q);
+void launch_tables(const double* h, double lam, double mu, double* dN, double* Kel, double* Qt, double* Kst,
+                   cudaStream_t st) {
+  k_tables<<<1, 256, 0, st>>>(h[0], h[1], h[2], lam, mu, dN, Kel, Qt);
+  k_stencils<<<27, 256, 0, st>>>(Kel, Kst);
 }
 
 void launch_rigid_for_shape(const SubDev& S, const double* h, double* R_shape, cudaStream_t st) {
@@ -671,14 +758,16 @@ void launch_return_map(const DevMesh& M, const double* du, const double* sig_k, 
 }
 
 void launch_elem_correction(const DevMesh& M, GPData gp, int* elem_np, int* sub_np, double* dKe, cudaStream_t st) {
-  k_elem_correction<<<blocks_for(M.n_elem, 8), 256, 0, st>>>(M, gp, elem_np, sub_np, dKe);
+  k_elem_correction<<<blocks_for(M.n_elem, 32), 256, 0, st>>>(M, gp, elem_np, sub_np, dKe);
 }
 
 void launch_band_fill(const DevMesh& M, const int* sub_list, int n_list, const int* elem_np, const double* dKe,
                       double* band, const long long* band_off_list, int elastic_only, int max_rows, int max_bw,
                       cudaStream_t st, const uint8_t* bmask) {
   if (n_list <= 0) return;
-  dim3 grid(blocks_for((long long)max_rows * (max_bw + 1), 256), n_list);
+  k_band_clear<<<dim3(blocks_for((long long)max_rows * (max_bw + 1), 256 * 16), n_list), 256, 0, st>>>(M, sub_list, band,
+                                                                                                band_off_list);
+  dim3 grid(blocks_for((long long)max_rows / 3 * 126, 256), n_list);
   k_band_fill<<<grid, 256, 0, st>>>(M, sub_list, elem_np, dKe, band, band_off_list, elastic_only, bmask);
 }
 
@@ -698,7 +787,7 @@ void launch_internal_force(const DevMesh& M, const double* dsig, const double* d
 
 void launch_apply_K(const DevMesh& M, const int* elem_np, const double* dKe, const double* x, double* y,
                     cudaStream_t st) {
-  k_apply_K<<<blocks_for(M.n_dof, 128), 128, 0, st>>>(M, elem_np, dKe, x, y);
+  k_apply_K<<<blocks_for(M.n_dof / 3, 128), 128, 0, st>>>(M, elem_np, dKe, x, y);
 }
 
 void launch_commit(const DevMesh& M, const double* du, const double* dsig, const double* dkap, double* u,
