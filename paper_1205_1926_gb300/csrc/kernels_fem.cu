@@ -626,59 +626,62 @@ __global__ void k_gather_force(DevMesh M, const double* __restrict__ fe, const d
   f[i] = (df ? df[i] : 0.0) - M.wgs * s;
 }
 
-// y = K x per subdomain with the assembled tangent, one thread per node: the elastic 27-node stencil of the
-// node's type (243 FMAs for its three rows, bound by the FP64 pipe; the coefficients, mostly the same for a
-// warp, come from L1), less the corrections of the adjacent elements with plastic points.
-__global__ void __launch_bounds__(128) k_apply_K(DevMesh M, const int* __restrict__ elem_np,
+// y = K x per subdomain with the assembled tangent, one thread per dof: the elastic 27-node stencil of the
+// node's type (81 FMAs, bound by the FP64 pipe and the loads' latency; the coefficients, mostly the same for
+// a warp, come from L1), less the corrections of the adjacent elements with plastic points.
+__global__ void __launch_bounds__(192) k_apply_K(DevMesh M, const int* __restrict__ elem_np,
                                                  const double* __restrict__ dKe, const double* __restrict__ x,
                                                  double* y) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (3 * i >= M.n_dof) return;
-  const int p = find_sub(M.subs, M.n_sub, 3 * i);
+  if (i >= M.n_dof) return;
+  const int p = find_sub(M.subs, M.n_sub, i);
   const SubDev& S = M.subs[p];
   const int n0 = S.nn[0], n1 = S.nn[1];
-  const int node = (int)(i - S.dof_off / 3);
+  const int dof = (int)(i - S.dof_off), node = dof / 3, r = dof % 3;
   const int li = node % n0, lj = (node / n0) % n1, lk = node / (n0 * n1);
   const double* xs = x + S.dof_off;
-  const double* kt = M.Kst + node_type(S, li, lj, lk) * 243;
-  double s[3] = {0.0, 0.0, 0.0};
-  for (int dz = -1; dz <= 1; ++dz)
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int b = lj + dy, c = lk + dz;
-      if (b < 0 || c < 0 || b >= n1 || c >= S.nn[2]) continue;
+  const double* kt = M.Kst + node_type(S, li, lj, lk) * 243 + 3 * r;
+  double s = 0.0;
 #pragma unroll
-      for (int dx = -1; dx <= 1; ++dx) {
-        const bool in = li + dx >= 0 && li + dx < n0;
-        const double* xn = xs + 3 * (in ? li + dx + n0 * (b + n1 * c) : node);
-        const double* kb = kt + ((dx + 1) + 3 * (dy + 1) + 9 * (dz + 1)) * 9;   // zero where there is no neighbour
-        const double v[3] = {__ldg(xn), __ldg(xn + 1), __ldg(xn + 2)};
+  for (int dz = -1; dz <= 1; ++dz) {
+    double v[9][3], k[9][3];   // a plane of neighbours: loads issued together
+    bool in[9];
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
+    for (int m = 0; m < 9; ++m) {
+      const int a = li + m % 3 - 1, b = lj + m / 3 - 1, c = lk + dz;
+      in[m] = a >= 0 && a < n0 && b >= 0 && b < n1 && c >= 0 && c < S.nn[2];
+      const double* xn = xs + 3 * (in[m] ? a + n0 * (b + n1 * c) : node);
+      const double* kb = kt + (m + 9 * (dz + 1)) * 9;
 #pragma unroll
-          for (int r = 0; r < 3; ++r)
-            if (in) s[r] = fma(__ldg(kb + 3 * r + q), v[q], s[r]);
+      for (int q = 0; q < 3; ++q) {
+        v[m][q] = __ldg(xn + q);
+        k[m][q] = __ldg(kb + q);
       }
     }
+#pragma unroll
+    for (int m = 0; m < 9; ++m)
+      if (in[m])
+#pragma unroll
+        for (int q = 0; q < 3; ++q) s = fma(k[m][q], v[m][q], s);
+  }
   for (int ez = max(lk - 1, 0); ez <= min(lk, S.dims[2] - 1); ++ez)
     for (int ey = max(lj - 1, 0); ey <= min(lj, S.dims[1] - 1); ++ey)
       for (int ex = max(li - 1, 0); ex <= min(li, S.dims[0] - 1); ++ex) {
         const long long ge = S.elem_off + ex + S.dims[0] * (ey + S.dims[1] * ez);
         if (!elem_np[ge]) continue;
         const double* dk = dKe + ge * kTri24;
-        const int na = c_off2local[(li - ex) + 2 * (lj - ey) + 4 * (lk - ez)];
+        const int row = 3 * c_off2local[(li - ex) + 2 * (lj - ey) + 4 * (lk - ez)] + r;
+        double c = 0.0;
+#pragma unroll
         for (int o = 0; o < 8; ++o) {
           const int nb = c_off2local[o];
           const double* xn = xs + 3 * (ex + (o & 1) + n0 * (ey + ((o >> 1) & 1) + n1 * (ez + (o >> 2))));
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            const double v = __ldg(xn + q);
-#pragma unroll
-            for (int r = 0; r < 3; ++r) s[r] = fma(-__ldg(dk + tri_index(3 * na + r, 3 * nb + q)), v, s[r]);
-          }
+          for (int q = 0; q < 3; ++q) c = fma(__ldg(dk + tri_index(row, 3 * nb + q)), __ldg(xn + q), c);
         }
+        s -= c;
       }
-#pragma unroll
-  for (int r = 0; r < 3; ++r) y[3 * i + r] = s[r];
+  y[i] = s;
 }
 
 __global__ void k_commit(long long n_dof, long long n_gp, const double* du, const double* dsig,
@@ -787,7 +790,7 @@ void launch_internal_force(const DevMesh& M, const double* dsig, const double* d
 
 void launch_apply_K(const DevMesh& M, const int* elem_np, const double* dKe, const double* x, double* y,
                     cudaStream_t st) {
-  k_apply_K<<<blocks_for(M.n_dof / 3, 128), 128, 0, st>>>(M, elem_np, dKe, x, y);
+  k_apply_K<<<blocks_for(M.n_dof, 192), 192, 0, st>>>(M, elem_np, dKe, x, y);
 }
 
 void launch_commit(const DevMesh& M, const double* du, const double* dsig, const double* dkap, double* u,
