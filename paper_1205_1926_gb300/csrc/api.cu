@@ -2489,7 +2489,8 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   M.shape_tnbr = upload(c, P.shape_tnbr);
   M.sub_b2s = upload(c, P.sub_b2s);
   M.slot_bnd = upload(c, P.slot_bnd);
-  M.sub_nbr = upload(c, P.sub_nbr);
+  M.lump_ord = upload(c, P.lump_ord);
+  M.lump_nbr = upload(c, P.lump_nbr);
   M.elem_sub = upload(c, elem_sub);
   M.helm = upload(c, helm);
   double* dN = dalloc<double>(c, 8 * 8 * 3);

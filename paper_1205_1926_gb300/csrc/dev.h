@@ -59,7 +59,8 @@ struct DevMesh {
   const int* shape_tnbr;    // [boundary node][27] neighbour boundary index or -1, per shape
   const int* sub_b2s;       // boundary index -> first copy slot or -1, per subdomain
   const int* slot_bnd;      // copy slot -> boundary index of its node
-  const int* sub_nbr;       // [interface node][28] first slot of each stencil neighbour or -1
+  const int* lump_ord;      // interface nodes of a subdomain in the order of the lumped preconditioner
+  const int* lump_nbr;      //   [position][28] count, then its interface neighbours (t << 24) | first slot - copy_off
   const int* bt_ptr;        // B^T by copy slot (CSR over multiplier rows): bt_ptr[n_copy + 1],
   const int* bt_row;        //   rows bt_row[e] and coefficients bt_val[e]
   const double* bt_val;

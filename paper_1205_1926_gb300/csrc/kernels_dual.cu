@@ -365,38 +365,47 @@ __global__ void __launch_bounds__(256, 4) k_lumped(DevMesh M, const double* __re
       if (sl[k] >= 0) xs[s0 + k * blockDim.x] = T(v[k]);
   }
   __syncthreads();
-  // blocks stored [t][cc][3 b + a] (neighbour t, column cc, row 3 b + a of boundary node b), all 27
-  // neighbours present in the storage (zero where the stencil has none); the neighbours are
-  // visited in order, nb_batch<T>() of them with their slot and block loads issued together
+  // blocks stored [t][cc][3 b + a] (neighbour t, column cc, row 3 b + a of boundary node b).  A box
+  // face node has 9 of its 27 stencil neighbours on the interface, an edge node about 15: the nodes
+  // come ordered by that number and its pattern, so that a warp works through the neighbours its nodes
+  // have (an FP64 instruction with its predicate off occupies the pipe all the same); nb_batch<T>()
+  // of them with their block loads issued together, summed in stencil order.
   const T* kb = kbb + kbb_off[p];
   const long long nr = 3LL * S.n_bnd;
-  for (int q = threadIdx.x; q < S.n_copy; q += blockDim.x) {
-    const long long slot = S.copy_off + q;
-    const int b = M.slot_bnd[slot], a = q % 3;
-    const T* kv = kb + 3LL * b + a;
-    const int* nbp = M.sub_nbr + (slot / 3) * 28;
+  const long long pos0 = S.copy_off / 3;
+  for (int q0 = 0; q0 < S.n_copy; q0 += blockDim.x) {
+    const int q = q0 + threadIdx.x;
+    const bool act = q < S.n_copy;
+    const long long pos = pos0 + (act ? q / 3 : 0);
+    const int a = q % 3;
+    const long long slot = S.copy_off + 3LL * __ldg(M.lump_ord + pos) + a;
+    const int* nbp = M.lump_nbr + pos * 28;
+    const int cnt = act ? __ldg(nbp) : 0;
+    const int wcnt = __reduce_max_sync(0xffffffffu, cnt);
+    const T* kv = kb + 3LL * __ldg(M.slot_bnd + slot) + a;
     T s = T(0);
     constexpr int NB = nb_batch<T>();
-#pragma unroll
-    for (int t0 = 0; t0 < 27; t0 += NB) {
+    for (int t0 = 0; t0 < wcnt; t0 += NB) {
       int nb[NB];
       T k0[NB], k1[NB], k2[NB];
 #pragma unroll
       for (int u = 0; u < NB; ++u) {
-        const int t = t0 + u;
-        nb[u] = __ldg(nbp + t);
-        k0[u] = __ldg(kv + (3 * t) * nr);
-        k1[u] = __ldg(kv + (3 * t + 1) * nr);
-        k2[u] = __ldg(kv + (3 * t + 2) * nr);
+        nb[u] = t0 + u < cnt ? __ldg(nbp + 1 + t0 + u) : -1;
+        const T* kt = kv + 3 * (nb[u] < 0 ? 0 : nb[u] >> 24) * nr;
+        k0[u] = __ldg(kt);
+        k1[u] = __ldg(kt + nr);
+        k2[u] = __ldg(kt + 2 * nr);
       }
 #pragma unroll
-      for (int u = 0; u < NB; ++u)
+      for (int u = 0; u < NB; ++u) {
+        if (t0 + u >= wcnt) break;
         if (nb[u] >= 0) {
-          const int lb = (int)(nb[u] - S.copy_off);
+          const int lb = nb[u] & 0xffffff;
           s += k0[u] * xs[lb] + k1[u] * xs[lb + 1] + k2[u] * xs[lb + 2];
         }
+      }
     }
-    cbuf[slot] = double(s);
+    if (act) cbuf[slot] = double(s);
   }
 }
 

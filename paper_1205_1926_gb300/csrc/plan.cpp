@@ -302,16 +302,26 @@ int plan_build(const tfeti_problem* prob, Plan& plan) {
       b2 += sh.n_bnd;
     }
     plan.kbb_total = kown;
-    plan.sub_nbr.assign((size_t)(plan.n_copy / 3) * 28, -1);
+    // lumped preconditioner: per subdomain its interface nodes ordered by the number and pattern of the
+    // stencil neighbours on the interface (lump_ord: node at a position), and by position the count
+    // and the neighbours as (t << 24) | first slot less copy_off
+    plan.lump_ord.assign((size_t)(plan.n_copy / 3), 0);
+    plan.lump_nbr.assign((size_t)(plan.n_copy / 3) * 28, 0);
+    struct LumpNode {
+      int32_t ii, cnt, pattern;
+      std::array<int32_t, 27> nbr;
+    };
+    std::vector<LumpNode> nodes;
     for (int p = 0; p < ns; ++p) {
       const auto& s = plan.subs[p];
+      nodes.clear();
       int ln = 0;
       for (int lk = 0; lk < s.nn[2]; ++lk)
         for (int lj = 0; lj < s.nn[1]; ++lj)
           for (int li = 0; li < s.nn[0]; ++li, ++ln) {
             const int ii = iface_index[p][ln];
             if (ii < 0) continue;
-            const int64_t base = (s.copy_off / 3 + ii) * 28;
+            LumpNode v{ii, 0, 0, {}};
             for (int dz = -1; dz <= 1; ++dz)
               for (int dy = -1; dy <= 1; ++dy)
                 for (int dx = -1; dx <= 1; ++dx) {
@@ -319,9 +329,21 @@ int plan_build(const tfeti_problem* prob, Plan& plan) {
                   const int a = li + dx, b = lj + dy, c = lk + dz;
                   if (a < 0 || b < 0 || c < 0 || a >= s.nn[0] || b >= s.nn[1] || c >= s.nn[2]) continue;
                   const int jj = iface_index[p][a + s.nn[0] * (b + s.nn[1] * c)];
-                  if (jj >= 0) plan.sub_nbr[base + t] = (int32_t)(s.copy_off + 3 * jj);
+                  if (jj < 0) continue;
+                  v.nbr[v.cnt++] = (int32_t)((t << 24) | (3 * jj));
+                  v.pattern |= 1 << t;
                 }
+            nodes.push_back(v);
           }
+      std::stable_sort(nodes.begin(), nodes.end(), [](const LumpNode& x, const LumpNode& y) {
+        return x.cnt != y.cnt ? x.cnt > y.cnt : x.pattern < y.pattern;
+      });
+      for (size_t k = 0; k < nodes.size(); ++k) {
+        const size_t pos = (size_t)(s.copy_off / 3) + k;
+        plan.lump_ord[pos] = nodes[k].ii;
+        plan.lump_nbr[28 * pos] = nodes[k].cnt;
+        for (int t = 0; t < nodes[k].cnt; ++t) plan.lump_nbr[28 * pos + 1 + t] = nodes[k].nbr[t];
+      }
     }
     for (int64_t sl = 0; sl < plan.n_copy; ++sl)
       if (plan.slot_bnd[sl] < 0) return bad(plan, "internal: interface node off the box boundary"), TFETI_ERR_ARG;

@@ -77,9 +77,9 @@ struct Plan {
   // Per copy slot: the boundary index of its node.  Blocks of K are stored per
   // boundary node and neighbour as 3x3 (27 x 9 doubles per boundary node).
   std::vector<int32_t> shape_bln, shape_tnbr, sub_b2s, slot_bnd;
-  // per interface node (3 slots): first slot of each of its 27 stencil neighbours
-  // that is an interface node of the same subdomain, or -1; padded to 28 entries
-  std::vector<int32_t> sub_nbr;
+  // per subdomain its interface nodes ordered for the lumped preconditioner, and by position the count of
+  // stencil neighbours that are interface nodes of the same subdomain and those, padded to 28 entries
+  std::vector<int32_t> lump_ord, lump_nbr;
   int64_t kbb_template_total = 0, kbb_total = 0;
   int64_t s_total = 0;       // floats of all shapes' dual Schur blocks
   // coarse matrix pairs (p, q) with p >= q that share at least one group,
