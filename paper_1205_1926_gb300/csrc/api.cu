@@ -508,16 +508,16 @@ void fp64_pass(tfeti_ctx* c, const SolveArgs& a) {
   if (rest && c->fac_pending && c->n_items_el < a.n_items) {
     SolveArgs e = a;
     e.n_items = c->n_items_el;
-    launch_sub_solve(c->M, e, c->solve_smem, sb);
+    launch_sub_solve(c->M, e, sb);
     if (dg) cudaStreamWaitEvent(sb, c->ev_fac_done, 0);   // the context stream joins below, past ev_join
     else join_factorisation(c);
     SolveArgs o = a;
     o.items = a.items + c->n_items_el;
     o.n_items = a.n_items - c->n_items_el;
-    launch_sub_solve(c->M, o, c->solve_smem, sb);
+    launch_sub_solve(c->M, o, sb);
     c->launches += 2;
   } else if (rest) {
-    launch_sub_solve(c->M, a, c->solve_smem, sb);
+    launch_sub_solve(c->M, a, sb);
     c->launches += 1;
   }
   if (dg) {
@@ -569,7 +569,7 @@ void op_F(tfeti_ctx* c, const double* x, double* yv) {
       a.items = c->d_items_pl64;
       a.n_items = c->n_items_pl64;
       set_stat(a, c->is_pl64);
-      launch_sub_solve(c->M, a, c->solve_smem, c->st2);
+      launch_sub_solve(c->M, a, c->st2);
       cudaEventRecord(c->ev_join, c->st2);
       c->launches += 1;
     }
@@ -607,7 +607,7 @@ void op_F32(tfeti_ctx* c, const double* x, double* yv, bool contract = true) {
   a.in_mode = 0;
   a.out_mode = 0;
   if (!c->schur_ready) {
-    launch_sub_solve(c->M, a, c->solve_smem32, c->st);
+    launch_sub_solve(c->M, a, c->st);
     c->launches += 1;
   } else {
     if (c->n_items_pl > 0) {
@@ -616,7 +616,7 @@ void op_F32(tfeti_ctx* c, const double* x, double* yv, bool contract = true) {
       a.items = c->d_items_pl;
       a.n_items = c->n_items_pl;
       set_stat(a, c->is_pl);
-      launch_sub_solve(c->M, a, c->solve_smem32, c->st2);
+      launch_sub_solve(c->M, a, c->st2);
       cudaEventRecord(c->ev_join, c->st2);
       c->launches += 1;
     }
@@ -670,7 +670,7 @@ int form_schur_blocks(tfeti_ctx* c) {
     a.S32 = c->S32;
     a.S64 = c->S64;
     a.s_off = c->s_off_c[sh];
-    launch_sub_solve(c->M, a, c->solve_smem, c->st);
+    launch_sub_solve(c->M, a, c->st);
     launch_schur_tile_S(c->S32 + c->s_off_c[sh], n_bd, false, c->Shi + c->s_tile_off[sh], c->Slo + c->s_tile_off[sh],
                         c->st);
     c->launches += 2;
@@ -834,7 +834,7 @@ int ensure_kinv(tfeti_ctx* c) {
     a.rep_sub = P.shapes[sh].rep_sub;
     a.S64 = kinv;
     a.s_off = off[sh];
-    launch_sub_solve(c->M, a, c->solve_smem, c->st);
+    launch_sub_solve(c->M, a, c->st);
     c->launches += 1;
   }
   sync(c);
@@ -1272,7 +1272,7 @@ void op_precond_dirichlet(tfeti_ctx* c, const double* w, double* out, bool fp32)
   a.dst = c->dx_c;
   a.in_mode = 4;
   a.out_mode = 1;
-  launch_sub_solve(M, a, fp32 ? c->solve_smem32 : c->solve_smem, c->st);   // y = K_ii^-1 v_i, 0 on b
+  launch_sub_solve(M, a, c->st);   // y = K_ii^-1 v_i, 0 on b
   launch_apply_K(M, c->elem_np, c->dKe, c->dx_c, c->dx_a, c->st);    // t = K [0; y]
   launch_slots_diff(M, c->dx_b, c->dx_a, c->cbuf, c->st);            // (v - t)_b
   launch_contract(M, c->cbuf, out, c->st);
@@ -2633,7 +2633,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     for (const SubInfo& s : P.subs) c->rec_max = std::max(c->rec_max, s.rec);
-    c->npad = (P.max_ndof + 1) & ~1;
+    c->npad = (P.max_ndof + 3) & ~3;   // vectors on 16-byte boundaries
     // the cluster form of the solve splits a row block into at least four rows per CTA
     int min_nb = kMaxNB;
     bool cl_ok = true;
@@ -2645,11 +2645,9 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     const long long room = (long long)max_smem - 1024 - 16LL * c->rec_max;   // static smem and barriers
     c->rcap = (int)std::min<long long>(kMaxRHS, room / (8LL * c->npad));
     if (c->rcap < 1) return fail(c, TFETI_ERR_ARG, "subdomain too large for the shared-memory solve");
-    c->solve_smem = sub_solve_smem(c->rec_max, c->npad, c->rcap, 8);
     const long long room32 = (long long)max_smem - 1024 - 8LL * c->rec_max;
     c->rcap32 = (int)std::min<long long>(kMaxRHS, room32 / (4LL * c->npad));
     if (c->rcap32 < 1) c->rcap32 = 1;
-    c->solve_smem32 = sub_solve_smem(c->rec_max, c->npad, c->rcap32, 4);
   }
   c->kbb = dalloc<double>(c, P.kbb_template_total + P.kbb_total);
   c->own_kbb_base = P.kbb_template_total;

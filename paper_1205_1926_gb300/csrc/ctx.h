@@ -54,7 +54,6 @@ struct tfeti_ctx {
   tfeti::SolveItem* d_items32 = nullptr;
   int n_items32 = 0;
   int rcap32 = 1;
-  size_t solve_smem32 = 0;
   int precision = 0;                 // TFETI_PRECISION_*
   double inner_rtol = 1e-3;
   double *dlt = nullptr, *rin = nullptr;
@@ -185,7 +184,6 @@ struct tfeti_ctx {
     int max_count = 0, n_eff = 0;
   };
   ItemStat is64, is32, is_pl, is_pl64, is_d, is_d32;
-  size_t solve_smem = 0;
   int n_sm = 1;
   int* d_list = nullptr;
   long long* d_list_off = nullptr;

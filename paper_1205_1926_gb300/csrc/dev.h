@@ -163,6 +163,7 @@ struct SolveArgs {
   int max_count;               // largest item count of the launch
   int n_eff;                   // its items counted by work: total over the largest item's, rounded up
   int max_bw;                  // largest half bandwidth of any subdomain
+  int stages;                  // panel buffers of the one-CTA form (set by the launch)
   int cl_max;                  // most CTAs that may share an item (cluster form), 1: none
   // in_mode 2 / out_mode 2 (dual Schur block formation of one shape): item.sub[] hold
   // boundary-dof columns j; the geometry is subdomain rep_sub; column j of
@@ -180,8 +181,8 @@ struct SolveArgs {
 };
 int smem_optin_max();
 int dyn_smem_limit(const void* fn);
-void launch_sub_solve(const DevMesh& M, const SolveArgs& a, size_t smem_bytes, cudaStream_t st);
-size_t sub_solve_smem(int rec_max, int npad, int rcap, int elem_bytes);
+void launch_sub_solve(const DevMesh& M, const SolveArgs& a, cudaStream_t st);
+size_t sub_solve_smem(int rec_max, int npad, int rcap, int elem_bytes, int stages);
 // FP64 dual Schur block applied to the elastic subdomains of one shape: X[k][i] =
 // (B^T lam) at boundary dof i of subdomain sub_list[k] (row-major [n_list][n_bd]),
 // then cbuf at the interface slots = (X S)[k][i], S64[j * n_bd + i] = S[i][j].

@@ -13,6 +13,7 @@
 //   L^{-1} x = (I + N)^{-1} D^{-1} x   and   L^{-T} y = D^{-T} (I + N)^{-T} y,
 // so each step of the forward and backward block recurrences is one GEMV with
 // a panel, and the triangular blocks are applied in parallel before and after.
+#include <algorithm>
 #include <cstdint>
 
 #include "async_common.cuh"
@@ -24,6 +25,8 @@ namespace tfeti {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kThreads32 = 512;   // of the FP32 one-CTA solve, whose steps are bound by latency
+constexpr int kSolveStages = 6;   // most panels in flight in the one-CTA solve
 constexpr int kNB1 = kMaxNB + 1;
 
 // ---------------------------------------------------------------------------
@@ -206,9 +209,9 @@ __global__ void __launch_bounds__(kThreads) k_band_chol(DevMesh M, const int* __
 
 // ---------------------------------------------------------------------------
 // Subdomain solve: one CTA applies K^+ to up to kMaxRHS subdomains of one
-// shape that share a factor record.  Shared memory: two panel buffers
-// (nb x bw doubles each) filled one step ahead by bulk copies, the kMaxRHS
-// local vectors, two mbarriers.
+// shape that share a factor record.  Shared memory: a.stages panel buffers
+// (nb x bw entries each) filled ahead by bulk copies, the local vectors, one
+// mbarrier per buffer.
 // ---------------------------------------------------------------------------
 
 // Right-hand sides of an item into vec (stride npad), by all threads of a CTA; ends with a barrier.
@@ -261,13 +264,68 @@ __device__ __forceinline__ void load_rhs(const DevMesh& M, const SolveArgs& a, c
   __syncthreads();
 }
 
-// The sweeps of one item with R right-hand sides, all threads of a CTA; the panels of steps 0 and 1 are
-// on their way.  Returns -1, or the step whose panel copy did not complete.
+// Sums over the warp of NR values per lane: lane / (32 / NR) gets the sum of v[lane / (32 / NR)].
+template <typename T, int NR>
+__device__ __forceinline__ T warp_sum_rows(T (&v)[NR], int lane) {
+  T k;
+  int o;
+  if constexpr (NR == 4) {
+    const bool h = lane & 16, g = lane & 8;
+    T a = h ? v[2] : v[0], b = h ? v[3] : v[1];
+    a += __shfl_xor_sync(0xffffffffu, h ? v[0] : v[2], 16);
+    b += __shfl_xor_sync(0xffffffffu, h ? v[1] : v[3], 16);
+    k = g ? b : a;
+    k += __shfl_xor_sync(0xffffffffu, g ? a : b, 8);
+    o = 4;
+  } else if constexpr (NR == 2) {
+    const bool h = lane & 16;
+    k = h ? v[1] : v[0];
+    k += __shfl_xor_sync(0xffffffffu, h ? v[0] : v[1], 16);
+    o = 8;
+  } else {
+    k = v[0];
+    o = 16;
+  }
+  for (; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+  return k;
+}
+
+// Forward step in FP32, where the shared-memory reads bound it: a warp takes NR whole rows of the block,
+// the lanes the columns, so that a column's x is read once for NR rows and no two lanes share a bank.
+template <int R, int NR>
+__device__ __forceinline__ void forward_rows32(const float* P, int bw, int jlo, int c0, int r0, int jb, float* vec,
+                                               int npad) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const float* prow = P + warp * NR * bw;
+  float acc[R][NR] = {};
+#pragma unroll 4
+  for (int j = jlo + lane; j < bw; j += 32) {
+    float x[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) x[r] = vec[r * npad + c0 + j];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      const float mv = prow[i * bw + j];
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r][i] = fmaf(mv, x[r], acc[r][i]);
+    }
+  }
+  const int t = warp * NR + lane / (32 / NR);
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const float v = warp_sum_rows<float, NR>(acc[r], lane);
+    if (lane % (32 / NR) == 0 && t < jb) vec[r * npad + r0 + t] -= v;
+  }
+}
+
+// The sweeps of one item with R right-hand sides, all threads of a CTA; the panels of the first NS steps
+// (buffers of pstride entries at pan) are on their way.  Returns -1, or the step whose panel copy did not
+// complete.
 template <typename T, int R>
-__device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __restrict__ dinv, T* const* pan, T* vec,
-                     int npad, uint64_t* bar, int* s_fail) {
+__device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __restrict__ dinv, const T* pan, int pstride,
+                     int NS, T* vec, int npad, uint64_t* bar, int* s_fail) {
   const int n = S0.n_dof, bw = S0.bw, nb = S0.nb, nblk = S0.nblk, rec = S0.rec;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, nt = blockDim.x;
   const int nsteps = 2 * nblk;
   const uint32_t pbytes = (uint32_t)rec * (uint32_t)sizeof(T);
   auto step_block = [nblk, nsteps](int k) { return k < nblk ? k : nsteps - 1 - k; };
@@ -293,25 +351,32 @@ __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __res
 
   // ---- block recurrences: forward y_b = x'_b - M_b y[r0-bw, r0), then backward
   //      z'[r0-bw, r0) -= M_b^T z'_b for b = nblk-1 .. 0
-  const int g = lane >> 3, l = lane & 7;
-  int k_fail = -1;
+  // forward rows: 8 lanes each, or 16 where a block has at most 16 rows
+  const int lpr = nb <= 16 ? 16 : 8, frow = tid / lpr, l = tid % lpr;
+  int k_fail = -1, buf = 0;
+  uint32_t phase = 0;
   for (int k = 0; k < nsteps; ++k) {
-    const int buf = k & 1;
-    const bool ok = mbar_wait(&bar[buf], (uint32_t)((k >> 1) & 1));
+    const bool ok = mbar_wait(&bar[buf], phase);
     if (!ok) *s_fail = 1;
-    const T* P = pan[buf];
+    const T* P = pan + buf * pstride;
     const int b = step_block(k);
     const int r0 = b * nb, jb = min(nb, n - r0);
     const int c0 = r0 - bw, jlo = max(0, -c0);
     if (ok) {
-      if (k < nblk) {
-        const int t = 4 * warp + g;                 // 8 warps x 4 rows = 32 rows
+      bool done = false;
+      if constexpr (sizeof(T) == 4) {
+        if (k < nblk && nb == 32) forward_rows32<R, 32 * 32 / kThreads32>(P, bw, jlo, c0, r0, jb, vec, npad), done = true;
+        else if (k < nblk && nb == 16) forward_rows32<R, 16 * 32 / kThreads32>(P, bw, jlo, c0, r0, jb, vec, npad), done = true;
+      }
+      if (done) {
+      } else if (k < nblk) {
+        const int t = frow;
         const bool act = t < jb;
         T acc[R] = {};
         if (act) {
           const T* prow = P + t * bw;
-          for (int j = l; j < bw; j += 8) {
-            if (j < jlo) continue;
+#pragma unroll 8
+          for (int j = jlo + l; j < bw; j += lpr) {
             const T mv = prow[j];
             const int c = c0 + j;
 #pragma unroll
@@ -320,6 +385,7 @@ __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __res
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) {
+          if (lpr == 16) acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 8);
           acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 4);
           acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 2);
           acc[r] += __shfl_xor_sync(0xffffffffu, acc[r], 1);
@@ -335,7 +401,20 @@ __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __res
           const int c = c0 + j;
           const T* zr = vec + r * npad + r0;
           T acc = T(0);
-          for (int t = 0; t < jb; ++t) acc = fma(P[t * bw + j], zr[t], acc);
+          int t = 0;
+          if constexpr (sizeof(T) == 4) {   // z' four at a time (nb a multiple of 4 puts them on 16 bytes)
+            if ((nb & 3) == 0)
+#pragma unroll 4
+              for (; t + 4 <= jb; t += 4) {
+                const float4 z = *reinterpret_cast<const float4*>(zr + t);
+                acc = fmaf(P[t * bw + j], z.x, acc);
+                acc = fmaf(P[(t + 1) * bw + j], z.y, acc);
+                acc = fmaf(P[(t + 2) * bw + j], z.z, acc);
+                acc = fmaf(P[(t + 3) * bw + j], z.w, acc);
+              }
+          }
+#pragma unroll 8
+          for (; t < jb; ++t) acc = fma(P[t * bw + j], zr[t], acc);
           vec[r * npad + c] -= acc;
         }
       }
@@ -345,7 +424,12 @@ __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __res
       k_fail = k;
       break;
     }
-    if (tid == 0 && k + 2 < nsteps) bulk_copy(pan[buf], fac + (long long)step_block(k + 2) * rec, pbytes, &bar[buf]);
+    if (tid == 0 && k + NS < nsteps)
+      bulk_copy(const_cast<T*>(P), fac + (long long)step_block(k + NS) * rec, pbytes, &bar[buf]);
+    if (++buf == NS) {
+      buf = 0;
+      phase ^= 1;
+    }
   }
   if (k_fail >= 0) return k_fail;
 
@@ -373,7 +457,7 @@ __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __res
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs a) {
+__global__ void __launch_bounds__(sizeof(T) == 4 ? kThreads32 : kThreads, 1) k_sub_solve(DevMesh M, SolveArgs a) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
   T* sm = reinterpret_cast<T*>(sm_raw);
   __shared__ int s_fail;
@@ -383,8 +467,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
   const int n = S0.n_dof, bw = S0.bw, nb = S0.nb, nblk = S0.nblk, rec = S0.rec;
   const int R = item.count;
   const int npad = a.npad;                       // vector stride (largest n of the launch, even)
-  T* pan[2] = {sm, sm + a.rec_max};
-  T* vec = sm + 2 * a.rec_max;                   // [rcap][npad]
+  const int NS = a.stages;
+  T* pan = sm;                                   // [NS][rec_max]
+  T* vec = sm + NS * a.rec_max;                  // [rcap][npad]
   uint64_t* bar = reinterpret_cast<uint64_t*>(vec + ((a.rcap * npad + 1) & ~1));
   const bool own = (item.fac & kOwnFac) != 0;
   const T* fac = (sizeof(T) == 8 ? reinterpret_cast<const T*>(own ? a.fac_own : a.fac)
@@ -397,17 +482,15 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
 
   if (tid == 0) {
     s_fail = 0;
-    mbar_init(&bar[0]);
-    mbar_init(&bar[1]);
+    for (int k = 0; k < NS; ++k) mbar_init(&bar[k]);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
   // step k uses the panel of block k (forward, k < nblk) or 2 nblk - 1 - k (backward)
   auto step_block = [nblk, nsteps](int k) { return k < nblk ? k : nsteps - 1 - k; };
-  if (tid == 0) {
-    bulk_copy(pan[0], fac, pbytes, &bar[0]);
-    bulk_copy(pan[1], fac + (long long)step_block(1) * rec, pbytes, &bar[1]);
-  }
+  if (tid == 0)
+    for (int k = 0; k < NS && k < nsteps; ++k)
+      bulk_copy(pan + k * a.rec_max, fac + (long long)step_block(k) * rec, pbytes, &bar[k]);
 
   const int n_bd = 3 * S0.n_bnd;
   load_rhs<T>(M, a, item, S0, vec, npad);
@@ -415,17 +498,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_sub_solve(DevMesh M, SolveArgs 
   // the pipe also where its predicate is off (a single right-hand side took 1200 us of the four's
   // 1600 us for a 2187-dof box when all four were predicated)
   int k_fail;
-  if (R == 1) k_fail = sweep<T, 1>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
-  else if (R == 2) k_fail = sweep<T, 2>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
-  else if (R == 3) k_fail = sweep<T, 3>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
-  else k_fail = sweep<T, 4>(S0, fac, dinv, pan, vec, npad, bar, &s_fail);
+  if (R == 1) k_fail = sweep<T, 1>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
+  else if (R == 2) k_fail = sweep<T, 2>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
+  else if (R == 3) k_fail = sweep<T, 3>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
+  else k_fail = sweep<T, 4>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
   if (k_fail >= 0) {
-    // a panel copy never completed: report, give the copies still in flight (steps
-    // k_fail and k_fail + 1) a bounded time to land, and leave
+    // a panel copy never completed: report, give the copies still in flight (steps k_fail ..
+    // k_fail + NS - 1) a bounded time to land, and leave
     if (tid == 0) {
       atomicOr(a.err, 2);
-      mbar_wait(&bar[k_fail & 1], (uint32_t)((k_fail >> 1) & 1));
-      if (k_fail + 1 < nsteps) mbar_wait(&bar[(k_fail + 1) & 1], (uint32_t)(((k_fail + 1) >> 1) & 1));
+      for (int k = k_fail; k < k_fail + NS && k < nsteps; ++k) mbar_wait(&bar[k % NS], (uint32_t)((k / NS) & 1));
     }
     return;
   }
@@ -502,9 +584,6 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, unsigned rank) {
 __device__ __forceinline__ void st_cluster(const double* p, unsigned rank, double v) {
   asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(cluster_addr(p, rank)), "d"(v) : "memory");
 }
-__device__ __forceinline__ void st_cluster(const float* p, unsigned rank, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "f"(v) : "memory");
-}
 // Remote store of v to p in CTA rank, completing sizeof(v) bytes on bar there.
 __device__ __forceinline__ void st_async(const double* p, const uint64_t* bar, unsigned rank, double v) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];" ::"r"(
@@ -512,43 +591,11 @@ __device__ __forceinline__ void st_async(const double* p, const uint64_t* bar, u
                "l"(__double_as_longlong(v)), "r"(cluster_addr(bar, rank))
                : "memory");
 }
-__device__ __forceinline__ void st_async(const float* p, const uint64_t* bar, unsigned rank, float v) {
-  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(
-                   cluster_addr(p, rank)),
-               "r"(__float_as_uint(v)), "r"(cluster_addr(bar, rank))
-               : "memory");
-}
 __device__ __forceinline__ void cluster_barrier() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// Sums over the warp of NR values per lane: lane / (32 / NR) gets the sum of v[lane / (32 / NR)].
-template <typename T, int NR>
-__device__ __forceinline__ T warp_sum_rows(T (&v)[NR], int lane) {
-  T k;
-  int o;
-  if constexpr (NR == 4) {
-    const bool h = lane & 16, g = lane & 8;
-    T a = h ? v[2] : v[0], b = h ? v[3] : v[1];
-    a += __shfl_xor_sync(0xffffffffu, h ? v[0] : v[2], 16);
-    b += __shfl_xor_sync(0xffffffffu, h ? v[1] : v[3], 16);
-    k = g ? b : a;
-    k += __shfl_xor_sync(0xffffffffu, g ? a : b, 8);
-    o = 4;
-  } else if constexpr (NR == 2) {
-    const bool h = lane & 16;
-    k = h ? v[1] : v[0];
-    k += __shfl_xor_sync(0xffffffffu, h ? v[0] : v[1], 16);
-    o = 8;
-  } else {
-    k = v[0];
-    o = 16;
-  }
-  for (; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
-  return k;
-}
-
-// Shared memory of a cluster CTA in values of T: panel slices, the vectors, the own rows' x', the
+// Shared memory of a cluster CTA in doubles: panel slices, the vectors, the own rows' x', the
 // window of column sums (a power of two above bw + nb), the received sums.
 struct ClLayout {
   int slice, npad, own, win, recv;
@@ -563,9 +610,10 @@ struct ClLayout {
 };
 
 // R right-hand sides, NR own rows of a block per warp (nb / C = 4 NR).
-template <typename T, int R, int NR>
-__device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& item, int C, unsigned q, T* sm,
+template <int R, int NR>
+__device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& item, int C, unsigned q, double* sm,
                          uint64_t* bar, uint64_t* xbar) {
+  using T = double;
   constexpr int rpc = 4 * NR;
   __shared__ T s_z[4][rpc][R];     // backward: z' of the own rows, one copy per warp
   const SubDev& S0 = M.subs[item.sub[0]];
@@ -578,9 +626,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
   T* recv = win + R * lay.win;               // [kClRing][C][rpc][R]
   const int npad = lay.npad, wmask = lay.win - 1;
   const bool own = (item.fac & kOwnFac) != 0;
-  const T* fac = (sizeof(T) == 8 ? reinterpret_cast<const T*>(own ? a.fac_own : a.fac)
-                                 : reinterpret_cast<const T*>(own ? a.fac32_own : a.fac32)) +
-                 (item.fac & ~kOwnFac);
+  const T* fac = (own ? a.fac_own : a.fac) + (item.fac & ~kOwnFac);
   const T* dinv = fac + (long long)nblk * rec;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nsteps = 2 * nblk;
@@ -754,7 +800,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
   }
 }
 
-template <typename T, int R>
+template <int R>
 __global__ void __launch_bounds__(kClThreads) k_solve_cl(DevMesh M, SolveArgs a) {
   extern __shared__ __align__(128) unsigned char sm_raw[];
   __shared__ uint64_t bar[kClStages], xbar[kClRing];
@@ -766,21 +812,21 @@ __global__ void __launch_bounds__(kClThreads) k_solve_cl(DevMesh M, SolveArgs a)
   }
   __syncthreads();
   const SolveItem item = a.items[blockIdx.x / C];
-  T* sm = reinterpret_cast<T*>(sm_raw);
+  double* sm = reinterpret_cast<double*>(sm_raw);
   const int rpc = M.subs[item.sub[0]].nb / C;   // 4, 8 or 16 (the same for the whole cluster)
-  if (rpc == 4) cl_solve<T, R, 1>(M, a, item, C, cluster_rank(), sm, bar, xbar);
-  else if (rpc == 8) cl_solve<T, R, 2>(M, a, item, C, cluster_rank(), sm, bar, xbar);
-  else cl_solve<T, R, 4>(M, a, item, C, cluster_rank(), sm, bar, xbar);
+  if (rpc == 4) cl_solve<R, 1>(M, a, item, C, cluster_rank(), sm, bar, xbar);
+  else if (rpc == 8) cl_solve<R, 2>(M, a, item, C, cluster_rank(), sm, bar, xbar);
+  else cl_solve<R, 4>(M, a, item, C, cluster_rank(), sm, bar, xbar);
 }
 
 // Launches the cluster form with C CTAs per item; false if it cannot run (nothing launched).
-template <typename T, int R>
+template <int R>
 bool launch_cl(const DevMesh& M, const SolveArgs& a, int C, cudaStream_t st) {
   const ClLayout lay(a.rec_max, a.npad, a.max_bw, C);
-  const size_t smem = sizeof(T) * lay.values(R);
-  static const int lim = dyn_smem_limit((const void*)k_solve_cl<T, R>);
+  const size_t smem = sizeof(double) * lay.values(R);
+  static const int lim = dyn_smem_limit((const void*)k_solve_cl<R>);
   if (smem > (size_t)lim) return false;
-  cudaFuncSetAttribute(k_solve_cl<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  cudaFuncSetAttribute(k_solve_cl<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(a.n_items * C));
   cfg.blockDim = dim3(kClThreads);
@@ -793,7 +839,7 @@ bool launch_cl(const DevMesh& M, const SolveArgs& a, int C, cudaStream_t st) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_solve_cl<T, R>, M, a) == cudaSuccess;
+  return cudaLaunchKernelEx(&cfg, k_solve_cl<R>, M, a) == cudaSuccess;
 }
 
 }  // namespace
@@ -870,39 +916,47 @@ void launch_band_chol(const DevMesh& M, const int* sub_list, int n_list, const l
   }
 }
 
-size_t sub_solve_smem(int rec_max, int npad, int rcap, int elem_bytes) {
+size_t sub_solve_smem(int rec_max, int npad, int rcap, int elem_bytes, int stages) {
   const size_t vec = ((size_t)rcap * npad + 1) & ~(size_t)1;
-  return (size_t)elem_bytes * (2 * (size_t)rec_max + vec) + 2 * sizeof(uint64_t);
+  return (size_t)elem_bytes * ((size_t)stages * rec_max + vec) + stages * sizeof(uint64_t);
 }
 
-void launch_sub_solve(const DevMesh& M, const SolveArgs& a, size_t smem_bytes, cudaStream_t st) {
+void launch_sub_solve(const DevMesh& M, const SolveArgs& args, cudaStream_t st) {
+  SolveArgs a = args;
   if (a.n_items <= 0) return;
-  // Cluster form for items of at most two right-hand sides: the most CTAs per item for which the
+  static const int n_sm = sm_count();
+  // Cluster form for FP64 items of at most two right-hand sides: the most CTAs per item for which the
   // launch still has at most two per SM, counting the items by their work (n_eff = total work over
-  // the largest item's; small boxes beside a large one end early).  Measured, FP64 pass of one CTA /
-  // 2 / 4 / 8 CTAs per item: 54 boxes of 8^3 elements 559 / 432 / 354 / 499 us, 3 boxes of 6^3 (with
+  // the largest item's; small boxes beside a large one end early).  Measured, pass of one CTA / 2 /
+  // 4 / 8 CTAs per item: 54 boxes of 8^3 elements 559 / 432 / 354 / 499 us, 3 boxes of 6^3 (with
   // the other boxes' product) - / 167 / 123 / 102 us, 125 uneven boxes of 4..12 elements per edge
-  // 1970 / 1401 / 1042 / - us; FP32, the uneven boxes: 627 / 634 / 603 us.
-  if (a.cl_max > 1 && a.max_count <= 2 && (a.in_mode == 0 || a.in_mode == 1 || a.in_mode == 4) && !a.alpha) {
-    static const int n_sm = sm_count();
+  // 1970 / 1401 / 1042 / - us.
+  const bool plain = a.in_mode == 0 || a.in_mode == 1 || a.in_mode == 4;
+  if (!a.fp32 && a.cl_max > 1 && a.max_count <= 2 && plain && !a.alpha) {
     int C = a.cl_max;
     while (C > 1 && a.n_eff * C > 2 * n_sm) C /= 2;
     if (C > 1) {
-      const bool one = a.max_count == 1;
-      const bool done = a.fp32 ? (one ? launch_cl<float, 1>(M, a, C, st) : launch_cl<float, 2>(M, a, C, st))
-                               : (one ? launch_cl<double, 1>(M, a, C, st) : launch_cl<double, 2>(M, a, C, st));
-      if (done) return;
+      if (a.max_count == 1 ? launch_cl<1>(M, a, C, st) : launch_cl<2>(M, a, C, st)) return;
       cudaGetLastError();
     }
   }
+  // One CTA per item.  A step's panel (35 KB in FP32 for an 8^3 box) takes about a microsecond from
+  // L2 and a step a third of that, so as many panels are kept in flight as shared memory holds: of the
+  // whole SM when the items fit one per SM, else of half of it.
+  static const int lim64 = dyn_smem_limit((const void*)k_sub_solve<double>);
+  static const int lim32 = dyn_smem_limit((const void*)k_sub_solve<float>);
+  const int lim = a.fp32 ? lim32 : lim64, eb = a.fp32 ? 4 : 8;
+  if (plain) a.rcap = std::max(1, std::min(a.rcap, a.max_count));
+  const size_t room = a.n_items <= n_sm ? (size_t)lim : (size_t)lim / 2 - 1024;
+  a.stages = 2;
+  while (a.stages < kSolveStages && sub_solve_smem(a.rec_max, a.npad, a.rcap, eb, a.stages + 1) <= room) ++a.stages;
+  const size_t smem = sub_solve_smem(a.rec_max, a.npad, a.rcap, eb, a.stages);
   if (a.fp32) {
-    static const int lim = dyn_smem_limit((const void*)k_sub_solve<float>);
     cudaFuncSetAttribute(k_sub_solve<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    k_sub_solve<float><<<a.n_items, kThreads, smem_bytes, st>>>(M, a);
+    k_sub_solve<float><<<a.n_items, kThreads32, smem, st>>>(M, a);
   } else {
-    static const int lim = dyn_smem_limit((const void*)k_sub_solve<double>);
     cudaFuncSetAttribute(k_sub_solve<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    k_sub_solve<double><<<a.n_items, kThreads, smem_bytes, st>>>(M, a);
+    k_sub_solve<double><<<a.n_items, kThreads, smem, st>>>(M, a);
   }
 }
 
