@@ -31,25 +31,32 @@ __device__ double block_reduce_sum(double v, double* red) {
   return s;   // valid in thread 0
 }
 
-// Six block sums at once, in the order of block_reduce_sum (shuffle tree within each
-// warp, then a shuffle tree over the warps' partials), with one barrier; red holds
-// 6 x 32 doubles.  The sums are valid in thread 0.
+// Six block sums at once: within a warp the lanes halve the values they carry at each of the first
+// exchanges (9 additions per lane instead of 30: the FP64 pipe is narrow), then one lane per value adds
+// the warps' partials in warp order.  red holds 6 x 32 doubles.  The sum of value c is valid in thread c
+// (as v[0]).
 __device__ void block_reduce_sum6(double v[6], double* red) {
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const unsigned all = 0xffffffffu;
+  const bool h4 = l & 16, h2 = l & 8, h1 = l & 4;
+  double a[4], b[2], c;
 #pragma unroll
-  for (int c = 0; c < 6; ++c)
-    for (int o = 16; o > 0; o >>= 1) v[c] += __shfl_down_sync(0xffffffffu, v[c], o);
-  if (l == 0)
+  for (int k = 0; k < 4; ++k) {   // values 0..3 stay in the low half, 4 and 5 go to the high half
+    const double hi = k < 2 ? v[4 + k] : 0.0;
+    a[k] = (h4 ? hi : v[k]) + __shfl_xor_sync(all, h4 ? v[k] : hi, 16);
+  }
 #pragma unroll
-    for (int c = 0; c < 6; ++c) red[c * 32 + w] = v[c];
+  for (int k = 0; k < 2; ++k) b[k] = (h2 ? a[2 + k] : a[k]) + __shfl_xor_sync(all, h2 ? a[k] : a[2 + k], 8);
+  c = (h1 ? b[1] : b[0]) + __shfl_xor_sync(all, h1 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(all, c, 2);
+  c += __shfl_xor_sync(all, c, 1);
+  const int idx = (h4 ? 4 : 0) + (h2 ? 2 : 0) + (h1 ? 1 : 0);
+  if ((l & 3) == 0 && idx < 6) red[idx * 32 + w] = c;
   __syncthreads();
-  if (threadIdx.x < 32) {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      double s = threadIdx.x < nw ? red[c * 32 + threadIdx.x] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-      v[c] = s;
-    }
+  if (threadIdx.x < 6) {
+    double s = 0.0;
+    for (int k = 0; k < nw; ++k) s += red[threadIdx.x * 32 + k];
+    v[0] = s;
   }
 }
 
@@ -145,24 +152,23 @@ __global__ void __launch_bounds__(256, 4) k_G_csr(DevMesh M, const T* __restrict
 #pragma unroll
         for (int c = 0; c < 6; ++c) acc[c] += g[k][c] * v[k];
   }
-  double s[6];
   if constexpr (sizeof(T) == 4) {
-    // the FP32 instance sums its block in FP32 (the FP64 pipe is narrow), in the order of
-    // block_reduce_sum6, and rounds the sums to FP64 at the end
+    // the FP32 instance sums its block in FP32 (the FP64 pipe is narrow) and rounds the sums to FP64 at
+    // the end
     block_reduce_sum6f(acc, reinterpret_cast<float*>(red));
+    if (threadIdx.x == 0)
 #pragma unroll
-    for (int c = 0; c < 6; ++c) s[c] = double(acc[c]);
+      for (int c = 0; c < 6; ++c) {
+        gx[6 * (long long)p + c] = scale * double(acc[c]);
+        if (gx32) gx32[6 * (long long)p + c] = (float)(scale * double(acc[c]));
+      }
   } else {
-#pragma unroll
-    for (int c = 0; c < 6; ++c) s[c] = double(acc[c]);
-    block_reduce_sum6(s, red);
-  }
-  if (threadIdx.x == 0)
-#pragma unroll
-    for (int c = 0; c < 6; ++c) {
-      gx[6 * (long long)p + c] = scale * s[c];
-      if (gx32) gx32[6 * (long long)p + c] = (float)(scale * s[c]);
+    block_reduce_sum6(acc, red);
+    if (threadIdx.x < 6) {
+      gx[6 * (long long)p + threadIdx.x] = scale * acc[0];
+      if (gx32) gx32[6 * (long long)p + threadIdx.x] = (float)(scale * acc[0]);
     }
+  }
 }
 
 // out[row] = ax * x[row] + bh * (G^T h)[row]   (x nullable); T as in k_G_csr.
