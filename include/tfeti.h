@@ -108,7 +108,7 @@ typedef struct tfeti_problem {
  * doubles, 4.8 GB at 4096 subdomains) applied by one GEMV.  PLANES: G G^T is block
  * tridiagonal over the planes of subdomains with equal z index (a subdomain couples
  * only to the boxes around it); its block LDL^T with explicit inverses of the pivot
- * blocks is applied by 2 nz - 1 dependent GEMVs of (6 nx ny)^2, nz planes of nx x ny
+ * blocks, eliminated from both ends, is applied by nz + 1 dependent GEMVs of (6 nx ny)^2, nz planes of nx x ny
  * subdomains (3 x 16 x 1536^2 doubles = 0.9 GB at 16^3 subdomains).  Both give H g to
  * rounding. */
 #define TFETI_COARSE_AUTO   0

@@ -337,7 +337,8 @@ void launch_lumped(const DevMesh& M, const double* w, const double* kbb, const l
 // G G^T is block tridiagonal over the planes of subdomains with equal z index (a subdomain
 // couples only to the 26 boxes around it), n_planes blocks of n_pl = 6 x (subdomains per
 // plane); a block LDL^T with explicit inverses W_k of the pivots and the products V_k, U_k
-// turns the solve into 2 n_planes - 1 dependent GEMVs of n_pl x n_pl (coarse_planes_factor).
+// eliminating from both ends at once, turns the solve into n_planes + 1 dependent launches of n_pl x n_pl
+// GEMVs (coarse_planes_factor).
 constexpr int kCoarseDense = 0, kCoarsePlanes = 1;
 constexpr long long kCoarseDenseMax = 6144;   // TFETI_COARSE_AUTO: dense H up to this n_coarse
 struct CoarseOp {

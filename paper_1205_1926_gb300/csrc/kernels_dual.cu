@@ -2,6 +2,8 @@
 // coarse operators G = R^T B^T and G^T, the projector pieces, the lumped
 // preconditioner B K B^T, deterministic reductions and the PCGP updates, and
 // the one-time coarse set-up (G G^T assembly, dense Cholesky, explicit inverse).
+#include <algorithm>
+
 #include "dev.h"
 #include "dual_common.cuh"
 
@@ -860,9 +862,12 @@ __global__ void k_coarse_assemble_planes(DevMesh M, const int* __restrict__ pair
   }
 }
 
-// Apply of the plane solver (H = (G G^T)^-1 by block LDL^T over the planes):
-// first y_k = alpha W_k x_k for every plane (blockIdx.y = k), then the forward steps
-// y_k -= V_k y_{k-1}, k = 1..np-1, and the backward steps y_k -= U_k y_{k+1}, k = np-2..0.
+// Apply of the plane solver (H = (G G^T)^-1 by a block LDL^T over the planes that eliminates from both
+// ends towards the middle plane m, so that the two ends' steps run side by side: n_planes + 1 dependent
+// launches instead of 2 n_planes - 1 from one end): first y_k = alpha W_k x_k for every plane (blockIdx.y =
+// k), then y_k -= V_k y_{k-1} for k = 1..m-1 beside y_k -= U_k y_{k+1} for k = n_planes-2..m+1, the middle
+// plane y_m -= V_m y_{m-1} + U_m y_{m+1}, and back out, y_k -= U_k y_{k+1} for k = m-1..0 beside y_k -=
+// V_k y_{k-1} for k = m+1..n_planes-1.
 // Two warps per row, the other plane's segment staged in shared memory.  T: FP64 blocks, or
 // their FP32 copies (FP32 products and sums); y8 (nullable): the padded FP32 copy of the final
 // y written by the last step that touches a plane (final != 0).
@@ -939,18 +944,32 @@ __global__ void __launch_bounds__(256) k_plane_first(const T* __restrict__ W, in
   }
 }
 
+// Up to two planes (blockIdx.y) in one launch, each with one or two neighbours: y -= M[0] from[0] (+ M[1] from[1]).
 template <typename T>
-__global__ void __launch_bounds__(256) k_plane_step(const T* __restrict__ Mk, int n, const double* __restrict__ y_other,
-                                                    double* y_k, long long row0, float* y8, int final) {
+struct PlaneStep {
+  const T* M[2][2];
+  const double* from[2][2];
+  double* y[2];
+  long long row0[2];
+};
+template <typename T>
+__global__ void __launch_bounds__(256) k_plane_step(PlaneStep<T> P, int n, float* y8, int final) {
   extern __shared__ __align__(16) unsigned char plane_xs[];
   __shared__ double red[kPlaneRows];
-  plane_stage<T>(y_other, n, plane_xs);
-  const int r = blockIdx.x * kPlaneRows + (threadIdx.x >> 6);
-  const double d = plane_row_dot<T>(r < n ? Mk + (long long)r * n : nullptr, plane_xs, n, red);
+  const int t = blockIdx.y, r = blockIdx.x * kPlaneRows + (threadIdx.x >> 6);
+  double d = 0.0;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const T* Mk = P.M[t][k];
+    if (!Mk) continue;
+    if (k) __syncthreads();   // the first neighbour's segment has been read
+    plane_stage<T>(P.from[t][k], n, plane_xs);
+    d += plane_row_dot<T>(r < n ? Mk + (long long)r * n : nullptr, plane_xs, n, red);
+  }
   if ((threadIdx.x & 63) == 0 && r < n) {
-    const double v = y_k[r] - d;
-    y_k[r] = v;
-    if (final) plane_y8(y8, row0 + r, v);
+    const double v = P.y[t][r] - d;
+    P.y[t][r] = v;
+    if (final) plane_y8(y8, P.row0[t] + r, v);
   }
 }
 
@@ -1293,21 +1312,34 @@ void launch_coarse_assemble_planes(const DevMesh& M, const int* pair_p, const in
                                                                 trip_j, n_pairs, Adiag, Aoff, per_plane, n_pl);
 }
 
-// Block LDL^T of the block-tridiagonal G G^T over the planes, with explicit inverses:
-// D_0 = A_00, D_k = A_kk - A_{k,k-1} W_{k-1} A_{k,k-1}^T, W_k = D_k^-1 (in place of Adiag),
+// Block LDL^T of the block-tridiagonal G G^T over the planes, eliminated from both ends to the middle plane m,
+// with explicit inverses: D_0 = A_00 and D_k = A_kk - A_{k,k-1} W_{k-1} A_{k,k-1}^T below m, D_{np-1} and D_k =
+// A_kk - A_{k+1,k}^T W_{k+1} A_{k+1,k} above it, D_m with both; W_k = D_k^-1 (in place of Adiag),
 // V_k = W_k A_{k,k-1} (k >= 1), U_k = W_k A_{k+1,k}^T (k <= np-2).  T: n_pl^2 doubles,
-// work: dense_inverse_work(n_pl) doubles.  A non-positive pivot sets *err (device).
+// work: dense_inverse_work(n_pl).
 void coarse_planes_factor(double* W, const double* Aoff, double* V, double* U, int n, int np, double* T,
                           double* work, int* err, cudaStream_t st) {
   const long long blk = (long long)n * n;
-  for (int k = 0; k < np; ++k) {
-    double* Wk = W + k * blk;
-    if (k > 0) {
-      const double* Ak = Aoff + k * blk;
-      dgemm(n, n, 0, n, 1.0, Ak, n, 1, W + (k - 1) * blk, n, 1, 0.0, T, n, 0, 0, st);   // T = A_{k,k-1} W_{k-1}
-      dgemm(n, n, 0, n, -1.0, T, n, 1, Ak, 1, n, 1.0, Wk, n, 0, 0, st);                // D_k = A_kk - T A^T
-    }
-    dense_cholesky_inverse(Wk, work, n, err, st);
+  const int m = np / 2;
+  // Aoff[k]: rows of plane k, columns of plane k - 1
+  auto from_below = [&](int k) {
+    const double* Ak = Aoff + k * blk;
+    dgemm(n, n, 0, n, 1.0, Ak, n, 1, W + (k - 1) * blk, n, 1, 0.0, T, n, 0, 0, st);   // T = A_{k,k-1} W_{k-1}
+    dgemm(n, n, 0, n, -1.0, T, n, 1, Ak, 1, n, 1.0, W + k * blk, n, 0, 0, st);        // D_k -= T A_{k,k-1}^T
+  };
+  auto from_above = [&](int k) {
+    const double* Ak = Aoff + (k + 1) * blk;
+    dgemm(n, n, 0, n, 1.0, Ak, 1, n, W + (k + 1) * blk, n, 1, 0.0, T, n, 0, 0, st);   // T = A_{k+1,k}^T W_{k+1}
+    dgemm(n, n, 0, n, -1.0, T, n, 1, Ak, n, 1, 1.0, W + k * blk, n, 0, 0, st);        // D_k -= T A_{k+1,k}
+  };
+  for (int k = 0; k < m; ++k) {
+    if (k > 0) from_below(k);
+    dense_cholesky_inverse(W + k * blk, work, n, err, st);
+  }
+  for (int k = np - 1; k >= m; --k) {
+    if (k == m && m > 0) from_below(k);
+    if (k + 1 < np) from_above(k);
+    dense_cholesky_inverse(W + k * blk, work, n, err, st);
   }
   for (int k = 0; k < np; ++k) {
     const double* Wk = W + k * blk;
@@ -1327,12 +1359,35 @@ static void plane_apply(const T* W, const T* V, const T* U, int n, int np, const
     cudaFuncSetAttribute(k_plane_step<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   }
   k_plane_first<T><<<dim3(rb, (unsigned)np), 256, smem, st>>>(W, n, x, alpha, y, y8, np == 1 ? 1 : 0);
-  for (int k = 1; k < np; ++k)
-    k_plane_step<T><<<rb, 256, smem, st>>>(V + k * blk, n, y + (long long)(k - 1) * n, y + (long long)k * n,
-                                           (long long)k * n, y8, k == np - 1 ? 1 : 0);
-  for (int k = np - 2; k >= 0; --k)
-    k_plane_step<T><<<rb, 256, smem, st>>>(U + k * blk, n, y + (long long)(k + 1) * n, y + (long long)k * n,
-                                           (long long)k * n, y8, 1);
+  const int m = np / 2;
+  PlaneStep<T> P;
+  int cnt = 0;
+  auto add = [&](int k, bool below, bool above) {   // plane k from its neighbours below (k - 1) and above
+    P.M[cnt][0] = below ? V + k * blk : above ? U + k * blk : nullptr;
+    P.from[cnt][0] = y + (long long)(below ? k - 1 : k + 1) * n;
+    P.M[cnt][1] = below && above ? U + k * blk : nullptr;
+    P.from[cnt][1] = y + (long long)(k + 1) * n;
+    P.y[cnt] = y + (long long)k * n;
+    P.row0[cnt++] = (long long)k * n;
+  };
+  auto step = [&](int final) {
+    if (cnt) k_plane_step<T><<<dim3(rb, (unsigned)cnt), 256, smem, st>>>(P, n, y8, final);
+    cnt = 0;
+  };
+  for (int s = 1; s < m || np - 1 - s > m; ++s) {
+    if (s < m) add(s, true, false);
+    if (np - 1 - s > m) add(np - 1 - s, false, true);
+    step(0);
+  }
+  if (np > 1) {
+    add(m, m > 0, m + 1 < np);
+    step(1);
+  }
+  for (int s = 1; m - s >= 0 || m + s < np; ++s) {
+    if (m - s >= 0) add(m - s, false, true);
+    if (m + s < np) add(m + s, true, false);
+    step(1);
+  }
 }
 
 void coarse_apply(const CoarseOp& C, const double* x, double alpha, double* y, cudaStream_t st) {
@@ -1354,6 +1409,10 @@ void coarse_apply32(const CoarseOp& C, const double* x, const float* x32, double
   }
 }
 
-int coarse_launches(const CoarseOp& C) { return C.mode == kCoarseDense ? 1 : 2 * C.n_planes - 1; }
+int coarse_launches(const CoarseOp& C) {
+  if (C.mode == kCoarseDense) return 1;
+  const int np = C.n_planes, m = np / 2;
+  return 1 + std::max(0, std::max(m - 1, np - 2 - m)) + (np > 1 ? 1 : 0) + std::max(m, np - 1 - m);
+}
 
 }  // namespace tfeti
