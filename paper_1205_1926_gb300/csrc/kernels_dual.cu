@@ -173,30 +173,20 @@ __global__ void __launch_bounds__(256, 4) k_G_csr(DevMesh M, const T* __restrict
   }
 }
 
-// out[row] = ax * x[row] + bh * (G^T h)[row]   (x nullable); T as in k_G_csr.
-template <typename T>
-__global__ void k_GT_csr(DevMesh M, const T* __restrict__ GTv, const double* __restrict__ x, double ax,
+// out[row] = ax * x[row] + bh * (G^T h)[row]   (x nullable).
+__global__ void k_GT_csr(DevMesh M, const double* __restrict__ GTv, const double* __restrict__ x, double ax,
                          const double* __restrict__ h, double bh, double* out) {
   const long long row = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (row >= M.n_mult) return;
   double s = 0.0;
   for (long long e = M.gt_ptr[row]; e < M.gt_ptr[row + 1]; ++e) {
-    const double* hq = h + 6 * (long long)M.gt_p[e];
-    T g[6];
-    g_entry<T>(GTv, e, g);
-    double hv[6];
-    if (sizeof(T) == 8) {
-      const double2* h2 = reinterpret_cast<const double2*>(hq);
-      const double2 a = __ldg(h2), b = __ldg(h2 + 1), c = __ldg(h2 + 2);
-      hv[0] = a.x; hv[1] = a.y; hv[2] = b.x; hv[3] = b.y; hv[4] = c.x; hv[5] = c.y;
-    } else {
+    const double2* h2 = reinterpret_cast<const double2*>(h + 6 * (long long)M.gt_p[e]);
+    double g[6];
+    g_entry<double>(GTv, e, g);
+    const double2 a = __ldg(h2), b = __ldg(h2 + 1), c = __ldg(h2 + 2);
+    const double hv[6] = {a.x, a.y, b.x, b.y, c.x, c.y};
 #pragma unroll
-      for (int c = 0; c < 6; ++c) hv[c] = hq[c];
-    }
-    T t = T(0);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) t += g[c] * T(hv[c]);
-    s += double(t);
+    for (int k = 0; k < 6; ++k) s = fma(g[k], hv[k], s);
   }
   out[row] = (x ? ax * x[row] : 0.0) + bh * s;
 }
@@ -336,7 +326,8 @@ __global__ void __launch_bounds__(512, 3) k_gemv64(const double* __restrict__ A,
         const long long j = j0 + 64 * u;
         if (j < n2) {
           const double2 v = __ldg(x2 + j);
-          acc += a[u].x * v.x + a[u].y * v.y;
+          acc = fma(a[u].x, v.x, acc);   // one operation per product: the FP64 pipe bounds the sum
+          acc = fma(a[u].y, v.y, acc);
         }
       }
     }
@@ -409,7 +400,9 @@ __global__ void __launch_bounds__(256, 4) k_lumped(DevMesh M, const double* __re
         if (t0 + u >= wcnt) break;
         if (nb[u] >= 0) {
           const int lb = nb[u] & 0xffffff;
-          s += k0[u] * xs[lb] + k1[u] * xs[lb + 1] + k2[u] * xs[lb + 2];
+          s = fma(k0[u], xs[lb], s);
+          s = fma(k1[u], xs[lb + 1], s);
+          s = fma(k2[u], xs[lb + 2], s);
         }
       }
     }
@@ -886,7 +879,8 @@ __device__ __forceinline__ double plane_part_dot<double>(const double* __restric
 #pragma unroll 4
   for (int j = sub; j < (n >> 1); j += 64) {
     const double2 a = __ldg(r2 + j), v = x2[j];
-    acc += a.x * v.x + a.y * v.y;
+    acc = fma(a.x, v.x, acc);
+    acc = fma(a.y, v.y, acc);
   }
   return acc;
 }
@@ -1117,7 +1111,7 @@ void launch_G_apply(const DevMesh& M, const double* x_lam, const double* x_full,
 
 void launch_GT_update(const DevMesh& M, const double* x, double ax, const double* h, double bh, double* out,
                       cudaStream_t st) {
-  if (M.n_mult > 0) k_GT_csr<double><<<blocks_for(M.n_mult, 256), 256, 0, st>>>(M, M.GTv, x, ax, h, bh, out);
+  if (M.n_mult > 0) k_GT_csr<<<blocks_for(M.n_mult, 256), 256, 0, st>>>(M, M.GTv, x, ax, h, bh, out);
 }
 
 void launch_fill_G(const DevMesh& M, const int* gp_slot, const double* gp_coef, const int* gt_e, double* Gv,
