@@ -302,7 +302,7 @@ void build_dir_item_list(tfeti_ctx* c, const std::vector<int>& plastic_count, in
     SolveItem it{};
     it.fac = c->dtmpl_off[k];
     for (int p = 0; p < ns; ++p) {
-      if (plastic_count[p] > 0 || c->dclass[p] != (int)k) continue;
+      if (plastic_count[p] > 0 || c->dclass[p] != (int)k || c->h_isubs[p].n_dof == 0) continue;
       it.sub[it.count++] = p;
       if (it.count == R) {
         items.push_back(it);
@@ -312,7 +312,7 @@ void build_dir_item_list(tfeti_ctx* c, const std::vector<int>& plastic_count, in
     if (it.count) items.push_back(it);
   }
   for (int p = 0; p < ns; ++p)
-    if (plastic_count[p] > 0) {
+    if (plastic_count[p] > 0 && c->h_isubs[p].n_dof > 0) {
       SolveItem it{};
       it.fac = kOwnFac | own_off(c, p);
       it.count = 1;
@@ -1267,12 +1267,15 @@ void op_precond_dirichlet(tfeti_ctx* c, const double* w, double* out, bool fp32)
   a.n_items = fp32 ? c->n_items_d32 : c->n_items_d;
   set_stat(a, fp32 ? c->is_d32 : c->is_d);
   a.src = c->dx_b;
-  a.bmask = c->d_bmask;
+  a.rec_max = c->i_rec_max;
+  a.npad = c->i_npad;
+  a.max_bw = c->i_max_bw;
+  a.cl_max = c->i_cl_max;
   a.no_fix = 1;
   a.dst = c->dx_c;
   a.in_mode = 4;
   a.out_mode = 1;
-  launch_sub_solve(M, a, c->st);   // y = K_ii^-1 v_i, 0 on b
+  launch_sub_solve(c->Mi, a, c->st);   // y = K_ii^-1 v_i; dx_c stays 0 on b
   launch_apply_K(M, c->elem_np, c->dKe, c->dx_c, c->dx_a, c->st);    // t = K [0; y]
   launch_slots_diff(M, c->dx_b, c->dx_a, c->cbuf, c->st);            // (v - t)_b
   launch_contract(M, c->cbuf, out, c->st);
@@ -1461,10 +1464,10 @@ int assemble(tfeti_ctx* c, const double* du, const double* df, double* f_out, bo
     }
     if (c->dirichlet) {
       // K_ii factors of the plastic subdomains (same slots), on the same band workspaces
-      launch_band_fill(M, c->d_list, (int)list.size(), c->elem_np, c->dKe, c->band_ws, c->d_list_off, 0, max_rows,
-                       c->plan.max_bw, c->st, c->d_bmask);
+      launch_band_fill(c->Mi, c->d_list, (int)list.size(), c->elem_np, c->dKe, c->band_ws, c->d_list_off, 0, max_rows,
+                       c->plan.max_bw, c->st, true);
       cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-      launch_band_chol(M, c->d_list, (int)list.size(), c->d_list_off, c->band_ws, c->d_list_fac, c->dfac_own,
+      launch_band_chol(c->Mi, c->d_list, (int)list.size(), c->d_list_off, c->band_ws, c->d_list_fac, c->dfac_own,
                        c->d_err, c->plan.max_bw, c->n_sm, c->st);
       c->launches += 2;
       c->factor_launches += 1;
@@ -2399,6 +2402,8 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
       d.origin[k] = s.origin[k];
       d.dims[k] = s.dims[k];
       d.nn[k] = s.nn[k];
+      d.ilo[k] = 0;
+      d.inn[k] = s.nn[k];
     }
     d.n_dof = s.n_dof;
     d.n_elem = s.n_elem;
@@ -2751,7 +2756,13 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   // Dirichlet preconditioner: constrained-dof mask, template classes, factor pools
   if (P.prob.precond == TFETI_PRECOND_DIRICHLET && base) {
     c->dirichlet = true;
-    c->d_bmask = base->d_bmask;
+    c->h_isubs = base->h_isubs;
+    c->Mi = c->M;
+    c->Mi.subs = base->Mi.subs;
+    c->i_rec_max = base->i_rec_max;
+    c->i_npad = base->i_npad;
+    c->i_max_bw = base->i_max_bw;
+    c->i_cl_max = base->i_cl_max;
     c->dclass = base->dclass;
     c->dclass_rep = base->dclass_rep;
     c->dtmpl_off = base->dtmpl_off;
@@ -2762,11 +2773,50 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     c->dx_a = dalloc<double>(c, P.n_dof);
     c->dx_b = dalloc<double>(c, P.n_dof);
     c->dx_c = dalloc<double>(c, P.n_dof);
+    cudaMemsetAsync(c->dx_c, 0, sizeof(double) * P.n_dof, c->st);   // the solves write the unconstrained dofs only
   } else if (P.prob.precond == TFETI_PRECOND_DIRICHLET) {
     c->dirichlet = true;
     std::vector<uint8_t> mask(P.n_dof, 0);
     for (long long sl = 0; sl < P.n_copy; ++sl) mask[P.subs[P.slot_sub[sl]].dof_off + P.slot_ldof[sl]] = 1;
-    c->d_bmask = upload(c, mask);
+    // node boxes without constraint rows: faces of a box are glued, fixed or free as a whole, so the nodes
+    // that carry no rows form a box
+    c->h_isubs = c->h_subs;
+    int min_nb = kMaxNB;
+    bool cl_ok = true;
+    for (int p = 0; p < ns; ++p) {
+      SubDev& d = c->h_isubs[p];
+      int lo[3] = {d.nn[0], d.nn[1], d.nn[2]}, hi[3] = {-1, -1, -1}, cnt = 0;
+      for (int ln = 0; ln < d.n_dof / 3; ++ln) {
+        const long long b = d.dof_off + 3LL * ln;
+        if (mask[b] || mask[b + 1] || mask[b + 2]) continue;
+        const int l[3] = {ln % d.nn[0], (ln / d.nn[0]) % d.nn[1], ln / (d.nn[0] * d.nn[1])};
+        for (int k = 0; k < 3; ++k) {
+          lo[k] = std::min(lo[k], l[k]);
+          hi[k] = std::max(hi[k], l[k]);
+        }
+        ++cnt;
+      }
+      int box = 1;
+      for (int k = 0; k < 3; ++k) {
+        d.ilo[k] = cnt ? lo[k] : 0;
+        d.inn[k] = cnt ? hi[k] - lo[k] + 1 : 1;
+        box *= d.inn[k];
+      }
+      if (cnt && box != cnt) return fail(c, TFETI_ERR_ARG, "internal: unconstrained nodes do not form a box");
+      d.n_dof = 3 * cnt;
+      d.bw = 3 * (d.inn[0] * d.inn[1] + d.inn[0] + 1) + 2;
+      d.nb = std::min(P.subs[p].nb, d.bw + 1);
+      d.nblk = (d.n_dof + d.nb - 1) / d.nb;
+      d.rec = (d.nb * d.bw + 3) & ~3;
+      c->i_rec_max = std::max(c->i_rec_max, d.rec);
+      c->i_npad = std::max(c->i_npad, (d.n_dof + 3) & ~3);
+      c->i_max_bw = std::max(c->i_max_bw, d.bw);
+      min_nb = std::min(min_nb, d.nb);
+      cl_ok = cl_ok && (d.nb == 16 || d.nb == 32);
+    }
+    c->i_cl_max = cl_ok ? std::min(8, min_nb / 4) : 1;
+    c->Mi = c->M;
+    c->Mi.subs = upload(c, c->h_isubs);
     std::map<std::pair<int, std::vector<int>>, int> classes;
     c->dclass.assign(ns, 0);
     long long tmpl = 0;
@@ -2778,7 +2828,8 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
         it = classes.emplace(std::make_pair(sb.shape, std::move(key)), (int)c->dclass_rep.size()).first;
         c->dclass_rep.push_back(p);
         c->dtmpl_off.push_back(tmpl);
-        tmpl += (sb.fac_size + 3) & ~3LL;     // 16-byte aligned records (bulk copies)
+        const SubDev& d = c->h_isubs[p];      // 16-byte aligned records (bulk copies)
+        tmpl += ((long long)d.nblk * d.rec + (long long)d.nblk * d.nb * d.nb + 3) & ~3LL;
       }
       c->dclass[p] = it->second;
     }
@@ -2791,6 +2842,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     c->dx_a = dalloc<double>(c, P.n_dof);
     c->dx_b = dalloc<double>(c, P.n_dof);
     c->dx_c = dalloc<double>(c, P.n_dof);
+    cudaMemsetAsync(c->dx_c, 0, sizeof(double) * P.n_dof, c->st);   // the solves write the unconstrained dofs only
     // template factors on the representatives' own band workspaces (unused at set-up)
     std::vector<long long> boffs = band_workspace(c, c->dclass_rep), foffs;
     int max_rows = 0;
@@ -2802,10 +2854,10 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     int* dl = upload(c, c->dclass_rep);
     long long* dbo = upload(c, boffs);
     long long* dfo = upload(c, foffs);
-    launch_band_fill(M, dl, (int)boffs.size(), c->elem_np, c->dKe, c->band_ws, dbo, 1, max_rows, P.max_bw, c->st,
-                     c->d_bmask);
+    launch_band_fill(c->Mi, dl, (int)boffs.size(), c->elem_np, c->dKe, c->band_ws, dbo, 1, max_rows, P.max_bw, c->st,
+                     true);
     cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-    launch_band_chol(M, dl, (int)boffs.size(), dbo, c->band_ws, dfo, c->dfac, c->d_err, P.max_bw, c->n_sm, c->st);
+    launch_band_chol(c->Mi, dl, (int)boffs.size(), dbo, c->band_ws, dfo, c->dfac, c->d_err, P.max_bw, c->n_sm, c->st);
     int herr = 0;
     cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
     sync(c);

@@ -205,7 +205,11 @@ struct tfeti_ctx {
   // replaced by identity rows and columns (K_ii), one template per (shape, pattern of
   // constrained dofs) class for elastic subdomains, own ones for plastic subdomains
   bool dirichlet = false;
-  uint8_t* d_bmask = nullptr;               // 1 at the local dofs of constrained nodes, [n_dof]
+  // descriptors of the subdomains' node boxes without constraint rows (K_ii: n_dof, bw, nb, ... of those
+  // boxes), and the largest of them
+  std::vector<tfeti::SubDev> h_isubs;
+  tfeti::DevMesh Mi{};
+  int i_rec_max = 0, i_npad = 0, i_max_bw = 0, i_cl_max = 1;
   std::vector<int> dclass, dclass_rep;      // class of each subdomain; a representative of each class
   std::vector<long long> dtmpl_off;         // per class: offset of its factor in dfac
   double* dfac = nullptr;

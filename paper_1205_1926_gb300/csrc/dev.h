@@ -19,7 +19,18 @@ struct SubDev {
   long long dof_off, elem_off, band_off, copy_off, r_off;
   long long bnd_off;          // its shape's boundary tables (shape_bln, 27 x for shape_tnbr)
   long long b2s_off;          // its boundary index -> first copy slot table
+  // node box of the dofs that n_dof counts: the whole box (ilo = 0, inn = nn), or in the Dirichlet
+  // preconditioner's descriptors the nodes without constraint rows (K_ii)
+  int ilo[3], inn[3];
 };
+
+// Local dof of the box for dof i of the descriptor's node box (the same for the whole box).
+__host__ __device__ inline int box_dof(const SubDev& S, int i) {
+  const int node = i / 3;
+  const int a = node % S.inn[0] + S.ilo[0], b = (node / S.inn[0]) % S.inn[1] + S.ilo[1],
+            c = node / (S.inn[0] * S.inn[1]) + S.ilo[2];
+  return 3 * (a + S.nn[0] * (b + S.nn[1] * c)) + i % 3;
+}
 
 constexpr int kMaxRHS = 4;     // right-hand sides one solve CTA carries
 constexpr int kSchurMinCount = 4;   // shapes with fewer subdomains never form their dual Schur block
@@ -119,8 +130,7 @@ void launch_return_map(const DevMesh& M, const double* du, const double* sig_k, 
 void launch_elem_correction(const DevMesh& M, GPData gp, int* elem_np, int* sub_np, double* dKe, cudaStream_t st);
 void launch_band_fill(const DevMesh& M, const int* sub_list, int n_list, const int* elem_np, const double* dKe,
                       double* band, const long long* band_off_list, int elastic_only, int max_rows, int max_bw,
-                      cudaStream_t st,
-                      const uint8_t* bmask = nullptr);
+                      cudaStream_t st, bool interior = false);
 // Boundary 3x3 blocks of K for the listed subdomains (elastic_only: the shape's elastic template);
 // also rounded to FP32 into kbb32 at the same offsets when kbb32 != null.  Per subdomain the
 // 27 x 9 values of its n_bnd boundary nodes are stored [t][cc][3 b + a]: K[3 node_b + a][3 nbr_t + cc].
@@ -140,7 +150,7 @@ void launch_band_chol(const DevMesh& M, const int* sub_list, int n_list, const l
                       int n_sm, cudaStream_t st);
 
 // Subdomain K^+ solve.  in_mode 0: x = B^T lam at the interface slots (zero
-// elsewhere); 1: x = src - B^T lam (lam nullable); 4: see bmask.  out_mode 0: interface slots
+// elsewhere); 1: x = src - B^T lam (lam nullable); 4: see no_fix.  out_mode 0: interface slots
 // to cbuf; 1: full local vector to dst (+ R alpha if alpha != null); 3: both.
 struct SolveArgs {
   const double* lam;
@@ -174,9 +184,9 @@ struct SolveArgs {
   float* S32;
   double* S64;                 // nullable: the same columns in FP64
   long long s_off;
-  // in_mode 4 (Dirichlet preconditioner): x = src with the dofs marked in bmask zeroed;
+  // in_mode 4 (Dirichlet preconditioner): the descriptors' node boxes are the nodes without constraint
+  // rows; x = src there, and out_mode 1 writes dst there only;
   // no_fix: the factor has no fixing dofs (they are not zeroed before and after)
-  const uint8_t* bmask;
   int no_fix;
 };
 int smem_optin_max();

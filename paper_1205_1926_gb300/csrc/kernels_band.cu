@@ -235,7 +235,7 @@ __device__ __forceinline__ void load_rhs(const DevMesh& M, const SolveArgs& a, c
     if (a.in_mode == 0)
       for (int i = tid; i < n; i += nt) x[i] = T(0);
     else if (a.in_mode == 4)
-      for (int i = tid; i < n; i += nt) x[i] = a.bmask[S.dof_off + i] ? T(0) : T(a.src[S.dof_off + i]);
+      for (int i = tid; i < n; i += nt) x[i] = T(a.src[S.dof_off + box_dof(S, i)]);
     else
       for (int i = tid; i < n; i += nt) x[i] = a.src ? T(a.src[S.dof_off + i]) : T(0);
   }
@@ -552,7 +552,7 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kThreads32 : kThreads, 1) k_s
           const double* al = a.alpha + 6 * (long long)p;
           for (int c = 0; c < 6; ++c) v += Rb[(long long)i * 6 + c] * al[c];
         }
-        a.dst[S.dof_off + i] = v;
+        a.dst[S.dof_off + (a.in_mode == 4 ? box_dof(S, i) : i)] = v;
       }
     }
   }
@@ -796,7 +796,10 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
       }
     if (a.out_mode == 1 || a.out_mode == 3)
       for (int b = (int)q; b < nblk; b += C)
-        for (int t = tid; t < nb && b * nb + t < n; t += kClThreads) a.dst[S.dof_off + b * nb + t] = double(x[b * nb + t]);
+        for (int t = tid; t < nb && b * nb + t < n; t += kClThreads) {
+          const int i = b * nb + t;
+          a.dst[S.dof_off + (a.in_mode == 4 ? box_dof(S, i) : i)] = x[i];
+        }
   }
 }
 

@@ -515,9 +515,9 @@ __device__ double stiffness_entry(const DevMesh& M, const SubDev& S, const int* 
 
 // Band storage of subdomain K_p with the fixing dofs replaced by identity rows:
 // band[r*(bw+1) + k] = K[r][r - bw + k] (lower band, row-major).
-// With bmask == null the six fixing dofs of Remark 1 get identity rows and columns
-// (K_rr of the generalised inverse); with bmask the dofs marked in it do (K_ii of the
-// Dirichlet preconditioner: the constrained nodes eliminated, Sec. 4.2).  The band is cleared first;
+// interior = 0: the six fixing dofs of Remark 1 get identity rows and columns (K_rr of the generalised
+// inverse); interior = 1: the descriptors' node boxes are the nodes without constraint rows and the band is
+// K_ii of the Dirichlet preconditioner (Sec. 4.2), numbered within that box.  The band is cleared first;
 // then one thread per (node, neighbour not after it, component pair) writes the stencil's entries: 126
 // per node instead of an index decode for every of the 3 (bw + 1) band entries.
 __global__ void k_band_clear(DevMesh M, const int* __restrict__ sub_list, double* band,
@@ -531,24 +531,23 @@ __global__ void k_band_clear(DevMesh M, const int* __restrict__ sub_list, double
 
 __global__ void k_band_fill(DevMesh M, const int* __restrict__ sub_list, const int* elem_np, const double* dKe,
                             double* band, const long long* __restrict__ band_off_list, int elastic_only,
-                            const uint8_t* __restrict__ bmask) {
+                            int interior) {
   const int item = blockIdx.y;
   const int p = sub_list[item];
   const SubDev& S = M.subs[p];
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const int node = idx / 126, m = (idx / 9) % 14, k = idx % 9;   // neighbours 0..13: those not after the node
   if (node >= S.n_dof / 3) return;
-  const int r[3] = {node % S.nn[0], (node / S.nn[0]) % S.nn[1], node / (S.nn[0] * S.nn[1])};
+  const int r[3] = {S.ilo[0] + node % S.inn[0], S.ilo[1] + (node / S.inn[0]) % S.inn[1],
+                    S.ilo[2] + node / (S.inn[0] * S.inn[1])};
   const int d[3] = {m % 3 - 1, (m / 3) % 3 - 1, m / 9 - 1};
 #pragma unroll
   for (int x = 0; x < 3; ++x)
-    if (r[x] + d[x] < 0 || r[x] + d[x] >= S.nn[x]) return;
-  const int row = 3 * node + k / 3, col = 3 * (node + d[0] + S.nn[0] * (d[1] + S.nn[1] * d[2])) + k % 3;
+    if (r[x] + d[x] < S.ilo[x] || r[x] + d[x] >= S.ilo[x] + S.inn[x]) return;
+  const int row = 3 * node + k / 3, col = 3 * (node + d[0] + S.inn[0] * (d[1] + S.inn[1] * d[2])) + k % 3;
   if (col > row) return;
   bool fixed = false;
-  if (bmask) {
-    fixed = bmask[S.dof_off + row] | bmask[S.dof_off + col];
-  } else {
+  if (!interior) {
 #pragma unroll
     for (int t = 0; t < 6; ++t) fixed |= (S.fix[t] == row) | (S.fix[t] == col);
   }
@@ -766,12 +765,13 @@ void launch_elem_correction(const DevMesh& M, GPData gp, int* elem_np, int* sub_
 
 void launch_band_fill(const DevMesh& M, const int* sub_list, int n_list, const int* elem_np, const double* dKe,
                       double* band, const long long* band_off_list, int elastic_only, int max_rows, int max_bw,
-                      cudaStream_t st, const uint8_t* bmask) {
+                      cudaStream_t st, bool interior) {
   if (n_list <= 0) return;
   k_band_clear<<<dim3(blocks_for((long long)max_rows * (max_bw + 1), 256 * 16), n_list), 256, 0, st>>>(M, sub_list, band,
                                                                                                 band_off_list);
   dim3 grid(blocks_for((long long)max_rows / 3 * 126, 256), n_list);
-  k_band_fill<<<grid, 256, 0, st>>>(M, sub_list, elem_np, dKe, band, band_off_list, elastic_only, bmask);
+  k_band_fill<<<grid, 256, 0, st>>>(M, sub_list, elem_np, dKe, band, band_off_list, elastic_only,
+                                       interior ? 1 : 0);
 }
 
 void launch_kbb_fill(const DevMesh& M, const int* sub_list, const long long* dst_off, int n_list, int max_bnd,

@@ -43,3 +43,32 @@ def test_apply_K(nel, cuts, hot):
     ref = np.concatenate([FixingNodeInverse(K, s.fixing_dofs()).apply(x[m.dec.dof_off[p]:m.dec.dof_off[p + 1]])
                           for p, (K, s) in enumerate(zip(Kb, m.dec.subs))])
     assert np.linalg.norm(y.cpu().numpy() - ref) <= 1e-10 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("nel,cuts", [
+    ((4, 4, 4), ((0, 2, 4), (0, 2, 4), (0, 4))),      # free faces: node boxes with and without them
+    ((3, 5, 4), ((0, 1, 3), (0, 5), (0, 1, 2, 4))),   # boxes one element thick: no unconstrained node in some
+    ((8, 8, 4), ((0, 8), (0, 4, 8), (0, 4))),
+])
+@pytest.mark.parametrize("hot", [0, 1])
+def test_dirichlet_preconditioner_on_node_boxes(nel, cuts, hot):
+    """Bbar Sbar Bbar^T x through the K_ii of the unconstrained nodes, elastic and partly yielding (1e-11 of the
+    largest entry)."""
+    from oracle.tfeti import TFETISolver
+    w = W.Workload(name="di", nel=nel, cuts=cuts)
+    m = ElastoplasticModel(w)
+    du, _ = W.seeded_partly_plastic_increment(w, 9, hot)
+    if not hot:
+        du = 0.0 * du
+    ctx = T.Context(w, precond=T.PRECOND_DIRICHLET)
+    n, nm = ctx.sizes["n_dof"], ctx.sizes["n_mult"]
+    dev = lambda a: torch.as_tensor(np.ascontiguousarray(a), device="cuda")  # noqa: E731
+    ctx.assemble_tangent(dev(du), dev(np.zeros(n)))
+    Kb, _, _ = m.assemble(du, np.zeros(n))
+    sol = TFETISolver(m.dec, Kb, [FixingNodeInverse(K, s.fixing_dofs()) for K, s in zip(Kb, m.dec.subs)],
+                      precond="dirichlet")
+    x = W.seeded_vector(nm, 8)
+    y = torch.zeros(nm, dtype=torch.float64, device="cuda")
+    ctx.apply("precond", dev(x), y)
+    ref = sol.apply_precond(x)
+    assert np.abs(y.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max()
