@@ -2533,31 +2533,34 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   {
     // explicit G = R^T B^T: entries (row, slot, B coefficient) in subdomain order, and
     // the permutation into row order (a counting sort; subdomain order within a row)
-    std::vector<long long> gp_ptr(ns + 1, 0);
+    std::vector<long long> gp_ptr(ns + 1, 0), gp_ptr3(3 * (size_t)ns + 1, 0);
     std::vector<int> gp_row, gp_slot;
     std::vector<double> gp_coef;
     for (int p = 0; p < ns; ++p) {
       gp_ptr[p] = (long long)gp_row.size();
       const SubInfo& sb = P.subs[p];
-      for (long long sl = sb.copy_off; sl < sb.copy_off + sb.n_copy; ++sl) {
-        const Group& g = P.groups[P.slot_group[sl]];
-        const int j = P.slot_j[sl];
-        if (g.nrows == 0) continue;
-        if (g.dirichlet) {
-          gp_row.push_back((int)(g.row0 + j));
-          gp_slot.push_back((int)sl);
-          gp_coef.push_back(1.0);
-        } else {
-          for (int r = std::max(j, 1); r < g.k; ++r) {
-            gp_row.push_back((int)(g.row0 + r - 1));
+      for (int cc = 0; cc < 3; ++cc) {
+        gp_ptr3[3 * (size_t)p + cc] = (long long)gp_row.size();
+        for (long long sl = sb.copy_off + cc; sl < sb.copy_off + sb.n_copy; sl += 3) {
+          const Group& g = P.groups[P.slot_group[sl]];
+          const int j = P.slot_j[sl];
+          if (g.nrows == 0) continue;
+          if (g.dirichlet) {
+            gp_row.push_back((int)(g.row0 + j));
             gp_slot.push_back((int)sl);
-            gp_coef.push_back(helmert_coef(r, j));
+            gp_coef.push_back(1.0);
+          } else {
+            for (int r = std::max(j, 1); r < g.k; ++r) {
+              gp_row.push_back((int)(g.row0 + r - 1));
+              gp_slot.push_back((int)sl);
+              gp_coef.push_back(helmert_coef(r, j));
+            }
           }
         }
       }
     }
     const long long ne = (long long)gp_row.size();
-    gp_ptr[ns] = ne;
+    gp_ptr[ns] = gp_ptr3[3 * (size_t)ns] = ne;
     std::vector<long long> gt_ptr(P.n_mult + 1, 0);
     for (long long e = 0; e < ne; ++e) ++gt_ptr[gp_row[e] + 1];
     for (long long r = 0; r < P.n_mult; ++r) gt_ptr[r + 1] += gt_ptr[r];
@@ -2573,18 +2576,23 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     M.gp_row = upload(c, gp_row);
     M.gt_ptr = upload(c, gt_ptr);
     M.gt_p = upload(c, gt_p);
-    double* Gv = dalloc<double>(c, (size_t)std::max(1LL, 6 * ne));
-    double* GTv = dalloc<double>(c, (size_t)std::max(1LL, 6 * ne));
+    M.gp_ptr3 = upload(c, gp_ptr3);
+    double* G3 = dalloc<double>(c, (size_t)std::max(1LL, 4 * ne));
+    double* GT3 = dalloc<double>(c, (size_t)std::max(1LL, 4 * ne));
+    float4* G3f = dalloc<float4>(c, (size_t)std::max(1LL, ne));
+    float4* GT3f = dalloc<float4>(c, (size_t)std::max(1LL, ne));
     float* Gv32 = dalloc<float>(c, (size_t)std::max(1LL, 8 * ne));
     float* GTv32 = dalloc<float>(c, (size_t)std::max(1LL, 8 * ne));
-    M.Gv = Gv;
-    M.GTv = GTv;
+    M.G3 = G3;
+    M.GT3 = GT3;
+    M.G3f = G3f;
+    M.GT3f = GT3f;
     M.Gv32 = Gv32;
     M.GTv32 = GTv32;
     int* d_slot = upload(c, gp_slot);
     double* d_coef = upload(c, gp_coef);
     int* d_gte = upload(c, gt_e);
-    launch_fill_G(M, d_slot, d_coef, d_gte, Gv, Gv32, GTv, GTv32, c->st);
+    launch_fill_G(M, d_slot, d_coef, d_gte, G3, G3f, Gv32, GT3, GT3f, GTv32, c->st);
     c->launches += 1;
     sync(c);
   }

@@ -83,17 +83,23 @@ struct DevMesh {
   const double* Kst;       // [27 node types][27 neighbours][9] assembled elastic stencils (kernels_fem.cu)
   const double* helm;      // [8 r][8 j] Helmert coefficients (row r = 1..7, copy j)
   // G = R^T B^T explicitly (it depends only on B and R): one entry per (multiplier
-  // row, copy slot) with B[row][slot] != 0, value B[row][slot] * R[slot dof][0..5].
-  // Subdomain order: entries gp_ptr[p]..gp_ptr[p+1] of subdomain p, their rows gp_row,
-  // values Gv / Gv32 [entry][6].  Row order: entries gt_ptr[row]..gt_ptr[row+1],
-  // subdomain gt_p, values GTv / GTv32 [entry][6].
-  const long long* gp_ptr;
+  // row, copy slot) with B[row][slot] != 0, value B[row][slot] * R[slot dof][0..5].  Of the six
+  // values of a dof of component c only three differ from zero: the translation c and the two
+  // rotations about other axes than c (on a box's regular nodes the modes about its centroid are
+  // orthogonal as they stand).
+  // Subdomain order: entries gp_ptr[p]..gp_ptr[p+1] of subdomain p, component by component from
+  // gp_ptr3[3p + c], their rows gp_row; G3 / G3f [entry][4] = translation, the two rotations in order,
+  // the row (as an integer).  Row order: entries gt_ptr[row]..gt_ptr[row+1], subdomain gt_p; GT3 / GT3f
+  // with (subdomain << 2) | component.  Gv32, GTv32: all values in FP32, [entry][8].
+  const long long *gp_ptr, *gp_ptr3;
   const int* gp_row;
-  const double* Gv;
+  const double* G3;
+  const float4* G3f;
   const float* Gv32;
   const long long* gt_ptr;
   const int* gt_p;
-  const double* GTv;
+  const double* GT3;
+  const float4* GT3f;
   const float* GTv32;
   long long n_gpairs;
   double wdet;
@@ -384,8 +390,8 @@ void launch_project32(const DevMesh& M, const CoarseOp& C, const double* x, doub
 inline long long h32_ld(long long l) { return (l + 3) & ~3LL; }
 void launch_h_to_f32(const double* H, long long l, float* H32, cudaStream_t st);
 // Values of the explicit G from R and the (row, slot, coefficient) entries (set-up).
-void launch_fill_G(const DevMesh& M, const int* gp_slot, const double* gp_coef, const int* gt_e, double* Gv,
-                   float* Gv32, double* GTv, float* GTv32, cudaStream_t st);
+void launch_fill_G(const DevMesh& M, const int* gp_slot, const double* gp_coef, const int* gt_e, double* G3, float4* G3f,
+                   float* Gv32, double* GT3, float4* GT3f, float* GTv32, cudaStream_t st);
 // Dirichlet preconditioner pieces: xfull = B^T w on the copy-slot dofs, 0 elsewhere
 // (xfull zeroed by the caller); cbuf[slot] = v[dof] - t[dof] on the copy slots.
 void launch_slots_to_full(const DevMesh& M, const double* w, double* xfull, cudaStream_t st);

@@ -105,54 +105,68 @@ __global__ void k_G_full(DevMesh M, const double* __restrict__ x_full, double* g
 // gx[6p+c] = scale * (G x)[6p+c] = scale * sum over the entries of subdomain p of G[entry][c] x[row]
 // (and, with gx32, its FP32 rounding for the FP32 coarse GEMV).  One CTA per subdomain.  T: FP64
 // values, or their FP32 copy (products, per-thread and block sums in T) for the inner iterations of
-// the mixed mode.  FP64 values: 6 per entry; FP32 values: 8 per entry (6 and two zeros), read as two
-// float4.
+// the mixed mode.  An entry is its three non-zero values and its row in one or two 16-byte loads; the
+// entries of the three components are taken side by side, so that the sums an entry adds to are known
+// and three chains of loads (the row, then x there) overlap.
 template <typename T>
-__device__ __forceinline__ void g_entry(const T* __restrict__ Gv, long long e, T g[6]);
-template <>
-__device__ __forceinline__ void g_entry<double>(const double* __restrict__ Gv, long long e, double g[6]) {
-  // 6 doubles = 48 bytes per entry: every entry starts on a 16-byte boundary
-  const double2* v = reinterpret_cast<const double2*>(Gv + e * 6);
-  const double2 a = __ldg(v), b = __ldg(v + 1), c = __ldg(v + 2);
-  g[0] = a.x; g[1] = a.y; g[2] = b.x; g[3] = b.y; g[4] = c.x; g[5] = c.y;
-}
-template <>
-__device__ __forceinline__ void g_entry<float>(const float* __restrict__ Gv, long long e, float g[6]) {
-  const float4 a = __ldg(reinterpret_cast<const float4*>(Gv) + 2 * e);
-  const float4 b = __ldg(reinterpret_cast<const float4*>(Gv) + 2 * e + 1);
-  g[0] = a.x; g[1] = a.y; g[2] = a.z; g[3] = a.w; g[4] = b.x; g[5] = b.y;
+struct GEntry {
+  T t, a, b;   // translation c; rotations about the first and second other axis
+  int id;      // row (G), or (subdomain << 2) | component (G^T)
+};
+template <typename T>
+__device__ __forceinline__ GEntry<T> g_entry(const void* __restrict__ G, long long e) {
+  GEntry<T> g;
+  if constexpr (sizeof(T) == 8) {
+    const double2* v = reinterpret_cast<const double2*>(G) + 2 * e;
+    const double2 u = __ldg(v), w = __ldg(v + 1);
+    g = {u.x, u.y, w.x, (int)__double_as_longlong(w.y)};
+  } else {
+    const float4 v = __ldg(reinterpret_cast<const float4*>(G) + e);
+    g = {v.x, v.y, v.z, __float_as_int(v.w)};
+  }
+  return g;
 }
 
-// entries per thread with their loads in flight together (FP32 / FP64 values)
 template <typename T>
-constexpr int g_batch() { return sizeof(T) == 4 ? 4 : 2; }
-template <typename T>
-__global__ void __launch_bounds__(256, 4) k_G_csr(DevMesh M, const T* __restrict__ Gv, const double* __restrict__ x,
+__global__ void __launch_bounds__(256, 4) k_G_csr(DevMesh M, const void* __restrict__ G, const double* __restrict__ x,
                                                   double* gx, double scale, float* gx32 = nullptr) {
   __shared__ double red[6 * 32];
   const int p = blockIdx.x;
-  const long long e0 = M.gp_ptr[p], e1 = M.gp_ptr[p + 1];
+  long long e0[3], n[3], most = 0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    e0[c] = M.gp_ptr3[3 * p + c];
+    n[c] = M.gp_ptr3[3 * p + c + 1] - e0[c];
+    most = n[c] > most ? n[c] : most;
+  }
   T acc[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-  // a thread's entries e0 + tid + k blockDim in k order, g_batch<T>() of them with all their
-  // loads in flight together (the row index, then x at the row, is a chain of two dependent loads)
-  constexpr int kGU = g_batch<T>();
-  const long long bd = blockDim.x;
-  for (long long eb = e0 + threadIdx.x; eb < e1; eb += kGU * bd) {
-    int row[kGU];
+  constexpr int U = sizeof(T) == 4 ? 2 : 1;
+  for (long long i0 = threadIdx.x; i0 < most; i0 += U * blockDim.x) {
+    GEntry<T> g[U][3];
+    T v[U][3];
 #pragma unroll
-    for (int k = 0; k < kGU; ++k) row[k] = eb + k * bd < e1 ? __ldg(M.gp_row + eb + k * bd) : -1;
-    T g[kGU][6];
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int k = 0; k < kGU; ++k)
-      if (row[k] >= 0) g_entry<T>(Gv, eb + k * bd, g[k]);
-    T v[kGU];
+      for (int c = 0; c < 3; ++c) {
+        const long long i = i0 + u * blockDim.x;
+        g[u][c] = {T(0), T(0), T(0), -1};
+        if (i < n[c]) g[u][c] = g_entry<T>(G, e0[c] + i);
+      }
 #pragma unroll
-    for (int k = 0; k < kGU; ++k) v[k] = row[k] >= 0 ? T(__ldg(x + row[k])) : T(0);
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int k = 0; k < kGU; ++k)
-      if (row[k] >= 0)
+      for (int c = 0; c < 3; ++c) v[u][c] = g[u][c].id >= 0 ? T(__ldg(x + g[u][c].id)) : T(0);
 #pragma unroll
-        for (int c = 0; c < 6; ++c) acc[c] += g[k][c] * v[k];
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const GEntry<T>& q = g[u][c];
+        if (q.id >= 0) {
+          acc[c] = fma(q.t, v[u][c], acc[c]);
+          acc[3 + (c == 0 ? 1 : 0)] = fma(q.a, v[u][c], acc[3 + (c == 0 ? 1 : 0)]);
+          acc[3 + (c == 2 ? 1 : 2)] = fma(q.b, v[u][c], acc[3 + (c == 2 ? 1 : 2)]);
+        }
+      }
   }
   if constexpr (sizeof(T) == 4) {
     // the FP32 instance sums its block in FP32 (the FP64 pipe is narrow) and rounds the sums to FP64 at
@@ -173,41 +187,36 @@ __global__ void __launch_bounds__(256, 4) k_G_csr(DevMesh M, const T* __restrict
   }
 }
 
+// (G^T h) of one entry in FP32: h8 padded to 8 values per subdomain.
+__device__ __forceinline__ float gt_entry32(const GEntry<float>& g, const float* __restrict__ h8) {
+  const int c = g.id & 3;
+  const float* h = h8 + 8 * (long long)(g.id >> 2);
+  return g.t * __ldg(h + c) + g.a * __ldg(h + 3 + (c == 0 ? 1 : 0)) + g.b * __ldg(h + 3 + (c == 2 ? 1 : 2));
+}
+
 // out[row] = ax * x[row] + bh * (G^T h)[row]   (x nullable).
-__global__ void k_GT_csr(DevMesh M, const double* __restrict__ GTv, const double* __restrict__ x, double ax,
-                         const double* __restrict__ h, double bh, double* out) {
+__global__ void k_GT_csr(DevMesh M, const double* __restrict__ x, double ax, const double* __restrict__ h, double bh,
+                         double* out) {
   const long long row = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (row >= M.n_mult) return;
   double s = 0.0;
   for (long long e = M.gt_ptr[row]; e < M.gt_ptr[row + 1]; ++e) {
-    const double2* h2 = reinterpret_cast<const double2*>(h + 6 * (long long)M.gt_p[e]);
-    double g[6];
-    g_entry<double>(GTv, e, g);
-    const double2 a = __ldg(h2), b = __ldg(h2 + 1), c = __ldg(h2 + 2);
-    const double hv[6] = {a.x, a.y, b.x, b.y, c.x, c.y};
-#pragma unroll
-    for (int k = 0; k < 6; ++k) s = fma(g[k], hv[k], s);
+    const GEntry<double> g = g_entry<double>(M.GT3, e);
+    const int c = g.id & 3;
+    const double* hp = h + 6 * (long long)(g.id >> 2);
+    s = fma(g.t, __ldg(hp + c), s);
+    s = fma(g.a, __ldg(hp + 3 + (c == 0 ? 1 : 0)), s);
+    s = fma(g.b, __ldg(hp + 3 + (c == 2 ? 1 : 2)), s);
   }
   out[row] = (x ? ax * x[row] : 0.0) + bh * s;
 }
 
-// FP32: out[row] = x[row] - (G^T h)[row] with the padded FP32 values and h8, the FP32
-// copy of h padded to 8 per subdomain (two float4 per entry and subdomain).
-__global__ void k_GT_csr32(DevMesh M, const float* __restrict__ GTv8, const double* __restrict__ x,
-                           const float* __restrict__ h8, double* out) {
+// FP32: out[row] = x[row] - (G^T h)[row], h8 the FP32 copy of h padded to 8 per subdomain.
+__global__ void k_GT_csr32(DevMesh M, const double* __restrict__ x, const float* __restrict__ h8, double* out) {
   const long long row = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (row >= M.n_mult) return;
-  const long long e0 = M.gt_ptr[row], e1 = M.gt_ptr[row + 1];
-  const float4* g4 = reinterpret_cast<const float4*>(GTv8);
-  const float4* h4 = reinterpret_cast<const float4*>(h8);
   double s = 0.0;
-  for (long long e = e0; e < e1; ++e) {
-    const int q = __ldg(M.gt_p + e);
-    const float4 a = __ldg(g4 + 2 * e), b = __ldg(g4 + 2 * e + 1);
-    const float4 u = __ldg(h4 + 2 * q), v = __ldg(h4 + 2 * q + 1);
-    const float t = a.x * u.x + a.y * u.y + a.z * u.z + a.w * u.w + b.x * v.x + b.y * v.y;
-    s += double(t);
-  }
+  for (long long e = M.gt_ptr[row]; e < M.gt_ptr[row + 1]; ++e) s += double(gt_entry32(g_entry<float>(M.GT3f, e), h8));
   out[row] = x[row] - s;
 }
 
@@ -262,26 +271,34 @@ __global__ void __launch_bounds__(512, 3) k_gemv32(const float* __restrict__ A, 
   }
 }
 
-// Entry values of G: e' runs over the row-ordered entries, e = gt_e[e'] is the same
+// Entry values of G: et runs over the row-ordered entries, e = gt_e[et] is the same
 // entry in subdomain order (a permutation), v = coef * R_p[slot dof][c].
 __global__ void k_fill_G(DevMesh M, const int* __restrict__ gp_slot, const double* __restrict__ gp_coef,
-                         const int* __restrict__ gt_e, double* Gv, float* Gv32, double* GTv, float* GTv32) {
+                         const int* __restrict__ gt_e, double* G3, float4* G3f, float* Gv32, double* GT3, float4* GT3f,
+                         float* GTv32) {
   const long long et = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (et >= M.n_gpairs) return;
   const long long e = gt_e[et];
   const long long slot = gp_slot[e];
-  const SubDev& S = M.subs[M.slot_sub[slot]];
+  const int p = M.slot_sub[slot], comp = M.slot_ldof[slot] % 3;
+  const SubDev& S = M.subs[p];
   const double* r = M.R + S.r_off + (long long)M.slot_ldof[slot] * 6;
   const double cf = gp_coef[e];
   for (int c = 0; c < 8; ++c) {
     const double v = c < 6 ? cf * r[c] : 0.0;
-    if (c < 6) {
-      Gv[e * 6 + c] = v;
-      GTv[et * 6 + c] = v;
-    }
     Gv32[e * 8 + c] = (float)v;
     GTv32[et * 8 + c] = (float)v;
   }
+  const double t = cf * r[comp], a = cf * r[3 + (comp == 0 ? 1 : 0)], b = cf * r[3 + (comp == 2 ? 1 : 2)];
+  const int row = M.gp_row[e], id = (p << 2) | comp;
+  double2* g = reinterpret_cast<double2*>(G3) + 2 * e;
+  g[0] = make_double2(t, a);
+  g[1] = make_double2(b, __longlong_as_double((long long)row));
+  g = reinterpret_cast<double2*>(GT3) + 2 * et;
+  g[0] = make_double2(t, a);
+  g[1] = make_double2(b, __longlong_as_double((long long)id));
+  G3f[e] = make_float4((float)t, (float)a, (float)b, __int_as_float(row));
+  GT3f[et] = make_float4((float)t, (float)a, (float)b, __int_as_float(id));
 }
 
 // out = v + R_p alpha_p on the dofs of subdomain p = blockIdx.y.
@@ -579,13 +596,11 @@ __device__ bool grid_sum_last(double s, double* partial, int* ctr, double* red, 
 // partial[j * gridDim.x + block].  kDefl: the instance that carries the deflation sums (AW given).
 template <bool kDefl>
 __global__ void __launch_bounds__(256, 4)
-    k_GT32_dot(DevMesh M, const float* __restrict__ GTv8, const double* __restrict__ x, const float* __restrict__ h8,
+    k_GT32_dot(DevMesh M, const double* __restrict__ x, const float* __restrict__ h8,
                double* out, const double* __restrict__ v, int mode, double* sc, double* partial, int* ctr,
                const double* __restrict__ AW, const double* __restrict__ Einv) {
   __shared__ double red[32];
   __shared__ int is_last;
-  const float4* g4 = reinterpret_cast<const float4*>(GTv8);
-  const float4* h4 = reinterpret_cast<const float4*>(h8);
   const int kd = (kDefl && mode == 1 && AW) ? (int)sc[kDeflK] : 0;
   const long long m = M.n_mult;
   constexpr int KD = kDefl ? kDeflMax : 1;
@@ -605,26 +620,11 @@ __global__ void __launch_bounds__(256, 4)
     float s0 = 0.f, s1 = 0.f;   // a row's few FP32 products summed in FP32
     for (long long k = 0; e0 + k < e1 || f0 + k < f1; ++k) {
       const bool a0 = e0 + k < e1, a1 = f0 + k < f1;
-      int q0 = 0, q1 = 0;
-      float4 ga0, gb0, ga1, gb1;
-      if (a0) {
-        q0 = __ldg(M.gt_p + e0 + k);
-        ga0 = __ldg(g4 + 2 * (e0 + k));
-        gb0 = __ldg(g4 + 2 * (e0 + k) + 1);
-      }
-      if (a1) {
-        q1 = __ldg(M.gt_p + f0 + k);
-        ga1 = __ldg(g4 + 2 * (f0 + k));
-        gb1 = __ldg(g4 + 2 * (f0 + k) + 1);
-      }
-      if (a0) {
-        const float4 u = __ldg(h4 + 2 * q0), w = __ldg(h4 + 2 * q0 + 1);
-        s0 += ga0.x * u.x + ga0.y * u.y + ga0.z * u.z + ga0.w * u.w + gb0.x * w.x + gb0.y * w.y;
-      }
-      if (a1) {
-        const float4 u = __ldg(h4 + 2 * q1), w = __ldg(h4 + 2 * q1 + 1);
-        s1 += ga1.x * u.x + ga1.y * u.y + ga1.z * u.z + ga1.w * u.w + gb1.x * w.x + gb1.y * w.y;
-      }
+      GEntry<float> g0 = {0.f, 0.f, 0.f, 0}, g1 = {0.f, 0.f, 0.f, 0};
+      if (a0) g0 = g_entry<float>(M.GT3f, e0 + k);
+      if (a1) g1 = g_entry<float>(M.GT3f, f0 + k);
+      if (a0) s0 += gt_entry32(g0, h8);
+      if (a1) s1 += gt_entry32(g1, h8);
     }
     const double o0 = x0 - double(s0);
     out[row0] = o0;
@@ -1105,19 +1105,19 @@ void launch_contract(const DevMesh& M, const double* cbuf, double* y, cudaStream
 
 void launch_G_apply(const DevMesh& M, const double* x_lam, const double* x_full, double* gx, double scale,
                     cudaStream_t st) {
-  if (x_lam) k_G_csr<double><<<M.n_sub, 256, 0, st>>>(M, M.Gv, x_lam, gx, scale);
+  if (x_lam) k_G_csr<double><<<M.n_sub, 256, 0, st>>>(M, M.G3, x_lam, gx, scale);
   else k_G_full<<<M.n_sub, 256, 0, st>>>(M, x_full, gx, scale);
 }
 
 void launch_GT_update(const DevMesh& M, const double* x, double ax, const double* h, double bh, double* out,
                       cudaStream_t st) {
-  if (M.n_mult > 0) k_GT_csr<<<blocks_for(M.n_mult, 256), 256, 0, st>>>(M, M.GTv, x, ax, h, bh, out);
+  if (M.n_mult > 0) k_GT_csr<<<blocks_for(M.n_mult, 256), 256, 0, st>>>(M, x, ax, h, bh, out);
 }
 
-void launch_fill_G(const DevMesh& M, const int* gp_slot, const double* gp_coef, const int* gt_e, double* Gv,
-                   float* Gv32, double* GTv, float* GTv32, cudaStream_t st) {
+void launch_fill_G(const DevMesh& M, const int* gp_slot, const double* gp_coef, const int* gt_e, double* G3, float4* G3f,
+                   float* Gv32, double* GT3, float4* GT3f, float* GTv32, cudaStream_t st) {
   if (M.n_gpairs > 0)
-    k_fill_G<<<blocks_for(M.n_gpairs, 256), 256, 0, st>>>(M, gp_slot, gp_coef, gt_e, Gv, Gv32, GTv, GTv32);
+    k_fill_G<<<blocks_for(M.n_gpairs, 256), 256, 0, st>>>(M, gp_slot, gp_coef, gt_e, G3, G3f, Gv32, GT3, GT3f, GTv32);
 }
 
 void launch_gemv(const double* A, long long n, const double* x, double alpha, double* y, cudaStream_t st) {
@@ -1140,7 +1140,7 @@ void launch_h_to_f32(const double* H, long long l, float* H32, cudaStream_t st) 
 void launch_project32(const DevMesh& M, const CoarseOp& C, const double* x, double* gx, float* gx32, double* hx,
                       float* hx8, double* out, cudaStream_t st) {
   launch_G32_coarse32(M, C, x, gx, gx32, hx, hx8, st);
-  if (M.n_mult > 0) k_GT_csr32<<<blocks_for(M.n_mult, 256), 256, 0, st>>>(M, M.GTv32, x, hx8, out);
+  if (M.n_mult > 0) k_GT_csr32<<<blocks_for(M.n_mult, 256), 256, 0, st>>>(M, x, hx8, out);
 }
 
 void launch_add_R_alpha(const DevMesh& M, const double* v, const double* alpha, double* out, int max_ndof,
@@ -1204,13 +1204,13 @@ void launch_dot2(const double* x1, const double* y1, const double* x2, const dou
 
 void launch_GT32_dot(const DevMesh& M, const double* x, const float* h8, double* out, const double* v, int mode,
                      double* sc, double* partial, int* ctr, cudaStream_t st, const double* AW, const double* Einv) {
-  if (AW) k_GT32_dot<true><<<kFusedBlocks, 256, 0, st>>>(M, M.GTv32, x, h8, out, v, mode, sc, partial, ctr, AW, Einv);
-  else k_GT32_dot<false><<<kFusedBlocks, 256, 0, st>>>(M, M.GTv32, x, h8, out, v, mode, sc, partial, ctr, AW, Einv);
+  if (AW) k_GT32_dot<true><<<kFusedBlocks, 256, 0, st>>>(M, x, h8, out, v, mode, sc, partial, ctr, AW, Einv);
+  else k_GT32_dot<false><<<kFusedBlocks, 256, 0, st>>>(M, x, h8, out, v, mode, sc, partial, ctr, AW, Einv);
 }
 
 void launch_G32_coarse32(const DevMesh& M, const CoarseOp& C, const double* x, double* gx, float* gx32, double* hx,
                          float* hx8, cudaStream_t st) {
-  k_G_csr<float><<<M.n_sub, 256, 0, st>>>(M, M.Gv32, x, gx, 1.0, gx32);
+  k_G_csr<float><<<M.n_sub, 256, 0, st>>>(M, M.G3f, x, gx, 1.0, gx32);
   coarse_apply32(C, gx, gx32, hx, hx8, st);
 }
 
