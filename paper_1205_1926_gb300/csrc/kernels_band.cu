@@ -18,6 +18,7 @@
 
 #include "async_common.cuh"
 #include "dev.h"
+#include "diag_chol.cuh"
 #include "dual_common.cuh"
 
 namespace tfeti {
@@ -54,61 +55,6 @@ __device__ __forceinline__ unsigned cluster_size() {
   return r;
 }
 
-// Cholesky of the jb x jb block D (lower, in shared memory) and its inverse X, all threads.
-// The pivot's square root and reciprocal come from y = 1/sqrt(d) by Newton-Raphson,
-// y <- y (3 - d y^2) / 2, two steps from an FP32 rsqrtf guess (2^-23 -> below FP64
-// rounding): on this part every FP64 instruction of a lone thread occupies the
-// sub-partition's FP64 pipe for a whole warp's worth of cycles, so the library
-// square root and division sequences dominated the column step.  A pivot that is
-// not positive sets bit 1 of err and is replaced by 1.
-__device__ void diag_factor_invert(double* D, double* X, int jb, int* err) {
-  const int tid = threadIdx.x, nt = blockDim.x;
-  __shared__ double s_rdiag[kMaxNB];
-  // X = I; column c of the factor and row c of X = L^{-1} advance together: after the
-  // pivot, column c of L and row c of X are scaled by 1/L[c][c]; then the trailing lower
-  // triangle of D and the rows r > c of X (X[r][:] -= L[r][c] X[c][:]) are updated in the
-  // same phase, three barriers per column
-  for (int e = tid; e < jb * jb; e += nt) X[(e / jb) * kNB1 + e % jb] = (e / jb == e % jb) ? 1.0 : 0.0;
-  for (int c = 0; c < jb; ++c) {
-    if (tid == 0) {
-      double d = D[c * kNB1 + c];
-      if (!(d > 0.0)) {
-        atomicOr(err, 1);
-        d = 1.0;
-      }
-      double y = (double)rsqrtf((float)d);
-      y = y * (1.5 - 0.5 * d * y * y);
-      y = y * (1.5 - 0.5 * d * y * y);
-      D[c * kNB1 + c] = d * y;
-      s_rdiag[c] = y;
-    }
-    __syncthreads();
-    const double inv = s_rdiag[c];
-    const int m = jb - c - 1;
-    for (int e = tid; e < jb; e += nt) {
-      if (e < m) D[(c + 1 + e) * kNB1 + c] *= inv;
-      else X[c * kNB1 + (e - m)] *= inv;
-    }
-    __syncthreads();
-    // trailing lower triangle, enumerated densely so that every lane of a warp has an entry,
-    // followed by the m x (c + 1) update of X
-    const int ntri = m * (m + 1) / 2;
-    for (int e = tid; e < ntri + m * (c + 1); e += nt) {
-      if (e < ntri) {
-        int t = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-        while (t * (t + 1) / 2 > e) --t;
-        while ((t + 1) * (t + 2) / 2 <= e) ++t;
-        const int r = c + 1 + t, q = c + 1 + (e - t * (t + 1) / 2);
-        D[r * kNB1 + q] -= D[r * kNB1 + c] * D[q * kNB1 + c];
-      } else {
-        const int f = e - ntri, r = c + 1 + f / (c + 1), q = f % (c + 1);
-        X[r * kNB1 + q] -= D[r * kNB1 + c] * X[c * kNB1 + q];
-      }
-    }
-    __syncthreads();
-  }
-}
-
 __global__ void __launch_bounds__(kThreads) k_band_chol(DevMesh M, const int* __restrict__ sub_list,
                                                          const long long* __restrict__ off_list, double* band,
                                                          const long long* __restrict__ fac_list, double* fac_pool,
@@ -134,7 +80,7 @@ __global__ void __launch_bounds__(kThreads) k_band_chol(DevMesh M, const int* __
       Dm[r * kNB1 + c] = (c <= r) ? A[(long long)(j0 + r) * W + c - r + bw] : 0.0;
     }
     __syncthreads();
-    diag_factor_invert(Dm, Di, jb, err);
+    diag_factor_invert(Dm, Di, jb, err, 1);
     // factor record of block row b (split over the cluster): dinv and M_b = Di * L[b rows][j0-bw .. j0)
     if (q == 0)
       for (int idx = tid; idx < NB * NB; idx += nt) {
@@ -890,7 +836,8 @@ void launch_band_chol(const DevMesh& M, const int* sub_list, int n_list, const l
                    cudaSuccess;
   cudaGetLastError();
   // cluster size: the largest power of two with n_list * C <= 2 * n_sm (at most 16, or 8 if
-  // non-portable cluster sizes are unavailable)
+  // non-portable cluster sizes are unavailable); 54 boxes of 8^3 elements take 17.4 ms with 4 CTAs each,
+  // 19.8 ms with 8
   int C = 1;
   const int cmax = big ? 16 : 8;
   while (C < cmax && (long long)n_list * C * 2 <= 2LL * n_sm) C *= 2;

@@ -26,6 +26,7 @@
 // and backward substitution with L, k_wood_y64 y = Z s on all dofs, k_wood_cb64 y at the copy
 // slots.
 #include "dev.h"
+#include "diag_chol.cuh"
 #include "dual_common.cuh"
 
 namespace tfeti {
@@ -186,37 +187,13 @@ __global__ void __launch_bounds__(256) k_wood_chol_diag(WoodArgs a, int p) {
   for (int e = threadIdx.x; e < kBlk * kBlk; e += blockDim.x) {
     const int i = e / kBlk, j = e % kBlk;
     A[i][j] = (i < jb && j < jb) ? C[(long long)(k0 + i) * r + k0 + j] : (i == j ? 1.0 : 0.0);
-    Li[i][j] = i == j ? 1.0 : 0.0;
   }
   __syncthreads();
-  for (int k = 0; k < kBlk; ++k) {   // right-looking in shared memory
-    if (threadIdx.x == 0) {
-      if (!(A[k][k] > 0.0)) atomicOr(a.err, 8);
-      A[k][k] = sqrt(fmax(A[k][k], 1e-300));
-    }
-    __syncthreads();
-    for (int i = k + 1 + threadIdx.x; i < kBlk; i += blockDim.x) A[i][k] /= A[k][k];
-    __syncthreads();
-    for (int e = threadIdx.x; e < kBlk * kBlk; e += blockDim.x) {
-      const int i = e / kBlk, j = e % kBlk;
-      if (i > k && j > k && j <= i) A[i][j] -= A[i][k] * A[j][k];
-    }
-    __syncthreads();
-  }
-  // inverse of the lower factor, one column per thread (forward substitution of unit vectors)
-  if (threadIdx.x < kBlk) {
-    const int c = threadIdx.x;
-    for (int i = 0; i < kBlk; ++i) {
-      double v = i == c ? 1.0 : 0.0;
-      for (int q = c; q < i; ++q) v -= A[i][q] * Li[q][c];
-      Li[i][c] = i >= c ? v / A[i][i] : 0.0;
-    }
-  }
-  __syncthreads();
+  diag_factor_invert(&A[0][0], &Li[0][0], kBlk, a.err, 8);   // one third the time of a divide and root per column
   double* D = a.d_pool + a.d_off[w] + (long long)p * kBlk * kBlk;
   for (int e = threadIdx.x; e < kBlk * kBlk; e += blockDim.x) {
     const int i = e / kBlk, j = e % kBlk;
-    D[e] = Li[i][j];
+    D[e] = j <= i ? Li[i][j] : 0.0;
     if (i < jb && j < jb && j <= i) C[(long long)(k0 + i) * r + k0 + j] = A[i][j];
   }
 }
@@ -311,31 +288,47 @@ __global__ void __launch_bounds__(256) k_wood_subst(const SubDev* __restrict__ s
     for (int s = 0; s < nbk; ++s) {
       const int b = pass == 0 ? s : nbk - 1 - s;
       const int b0 = b * kBlk, bb = min(kBlk, r - b0);
-      // T = Y_b - sum over the solved blocks (forward: a < b, L_ba; backward: a > b, L_ab^T)
-      for (int e = threadIdx.x; e < kBlk * kBlk; e += blockDim.x) {
-        const int i = e / kBlk, j = e % kBlk;
-        float v = i < bb ? ys[(b0 + i) * kBlk + j] : 0.f;
-        if (i < bb) {
-          if (pass == 0) {
-            for (int q = 0; q < b0; ++q) v -= C[(long long)(b0 + i) * r + q] * ys[q * kBlk + j];
-          } else {
-            for (int q = b0 + bb; q < r; ++q) v -= C[(long long)q * r + b0 + i] * ys[q * kBlk + j];
-          }
+      // T = Y_b - sum over the solved blocks (forward: a < b, L_ba; backward: a > b, L_ab^T): four rows
+      // per thread side by side, sharing the column's y
+      const int j = threadIdx.x & 31, i0 = threadIdx.x >> 5;
+      int row[4];
+      float v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        row[k] = min(i0 + 8 * k, bb - 1);
+        v[k] = ys[(b0 + row[k]) * kBlk + j];
+      }
+      if (pass == 0) {
+#pragma unroll 4
+        for (int q = 0; q < b0; ++q) {
+          const float y = ys[q * kBlk + j];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] -= __ldg(C + (long long)(b0 + row[k]) * r + q) * y;
         }
-        T[i][j] = v;
+      } else {
+#pragma unroll 4
+        for (int q = b0 + bb; q < r; ++q) {
+          const float y = ys[q * kBlk + j];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) v[k] -= __ldg(C + (long long)q * r + b0 + row[k]) * y;
+        }
       }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) T[i0 + 8 * k][j] = i0 + 8 * k < bb ? v[k] : 0.f;
       __syncthreads();
+      // Y_b = Li T or Li^T T (Li is zero above its diagonal)
       const float* Li = D + (long long)b * kBlk * kBlk;
-      for (int e = threadIdx.x; e < kBlk * kBlk; e += blockDim.x) {
-        const int i = e / kBlk, j = e % kBlk;
-        if (i >= bb) continue;
-        float v = 0.f;
-        if (pass == 0)
-          for (int q = 0; q <= i; ++q) v += Li[i * kBlk + q] * T[q][j];
-        else
-          for (int q = i; q < bb; ++q) v += Li[q * kBlk + i] * T[q][j];
-        ys[(b0 + i) * kBlk + j] = v;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) v[k] = 0.f;
+#pragma unroll 4
+      for (int q = 0; q < bb; ++q) {
+        const float y = T[q][j];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] += __ldg(Li + (pass == 0 ? row[k] * kBlk + q : q * kBlk + row[k])) * y;
       }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (i0 + 8 * k < bb) ys[(b0 + row[k]) * kBlk + j] = v[k];
       __syncthreads();
     }
   }
@@ -469,20 +462,23 @@ __global__ void __launch_bounds__(256) k_wood_s64(WoodArgs a) {
   const int nbk = wood_nblk(r);
   for (int b = 0; b < nbk; ++b) {
     const int b0 = b * kBlk, bb = min(kBlk, r - b0);
-    for (int i = warp; i < bb; i += 8) {
+    // eight lanes per row, for the block's rows of L and for its inverted diagonal block alike
+    const int i = tid >> 3, l = tid & 7;
+    double v = 0.0;
+    if (i < bb) {
       const double* row = L + (long long)(b0 + i) * r;
-      double v = 0.0;
-      for (int q = lane; q < b0; q += 32) v = fma(row[q], s[q], v);
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-      if (lane == 0) T[i] = s[b0 + i] - v;
+#pragma unroll 4
+      for (int q = l; q < b0; q += 8) v = fma(row[q], s[q], v);
     }
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (l == 0) T[i] = i < bb ? s[b0 + i] - v : 0.0;
     __syncthreads();
-    if (tid < bb) {
-      const double* Li = D + (long long)b * kBlk * kBlk + tid * kBlk;
-      double v = 0.0;
-      for (int q = 0; q <= tid; ++q) v = fma(Li[q], T[q], v);
-      s[b0 + tid] = v;
-    }
+    const double* Li = D + (long long)b * kBlk * kBlk + i * kBlk;
+    v = 0.0;
+#pragma unroll
+    for (int q = 0; q < kBlk; q += 8) v = fma(Li[q + l], T[q + l], v);
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (l == 0 && i < bb) s[b0 + i] = v;
     __syncthreads();
   }
   for (int b = nbk - 1; b >= 0; --b) {
@@ -492,18 +488,17 @@ __global__ void __launch_bounds__(256) k_wood_s64(WoodArgs a) {
       for (int q = b0 + bb + warp; q < r; q += 8) v = fma(L[(long long)q * r + b0 + lane], s[q], v);
     part[warp][lane] = v;
     __syncthreads();
-    if (tid < bb) {
-      double acc = 0.0;
-      for (int k = 0; k < 8; ++k) acc += part[k][tid];
-      T[tid] = s[b0 + tid] - acc;
-    }
+    const int i = tid >> 3, l = tid & 7;
+    v = part[l][i];
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (l == 0) T[i] = i < bb ? s[b0 + i] - v : 0.0;
     __syncthreads();
-    if (tid < bb) {
-      const double* Li = D + (long long)b * kBlk * kBlk;
-      double x = 0.0;
-      for (int q = tid; q < bb; ++q) x = fma(Li[q * kBlk + tid], T[q], x);
-      s[b0 + tid] = x;
-    }
+    const double* Li = D + (long long)b * kBlk * kBlk + i;
+    v = 0.0;
+#pragma unroll
+    for (int q = 0; q < kBlk; q += 8) v = fma(Li[(q + l) * kBlk], T[q + l], v);
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (l == 0 && i < bb) s[b0 + i] = v;
     __syncthreads();
   }
   for (int c = tid; c < r; c += blockDim.x) t[c] = s[c];
