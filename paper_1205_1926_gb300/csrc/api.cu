@@ -138,8 +138,8 @@ std::vector<long long> band_workspace(tfeti_ctx* c, const std::vector<int>& list
 }
 
 double dot_host(tfeti_ctx* c, const double* x, const double* y, long long n) {
-  launch_dot(x, y, n, c->partial, c->sc + 8, c->st);
-  c->launches += 2;
+  launch_dot(x, y, n, c->partial, c->d_dot_ctr, c->sc + 8, c->st);
+  c->launches += 1;
   double v = 0.0;
   cudaMemcpyAsync(&v, c->sc + 8, sizeof(double), cudaMemcpyDeviceToHost, c->st);
   sync(c);
@@ -1509,17 +1509,17 @@ PcgOut pcg_core(tfeti_ctx* c, double* x, double* r, double tol_abs, int maxit, b
   for (int j = 1; j <= maxit; ++j) {
     if (fp32) {                                      // inner iterations of the mixed mode
       op_project32(c, r, c->w);
-      launch_dot(c->w, c->w, m, c->partial, c->sc + 3, c->st);
+      launch_dot(c->w, c->w, m, c->partial, c->d_dot_ctr, c->sc + 3, c->st);
       op_precond32(c, c->w, c->z);
       op_project32(c, c->z, c->y);
     } else {
       op_project(c, r, c->w);                        // w = P r
-      launch_dot(c->w, c->w, m, c->partial, c->sc + 3, c->st);
+      launch_dot(c->w, c->w, m, c->partial, c->d_dot_ctr, c->sc + 3, c->st);
       op_precond(c, c->w, c->z);                     // z = F^-1 w
       op_project(c, c->z, c->y);                     // y = P z
     }
-    launch_dot(c->y, c->w, m, c->partial, c->sc + 0, c->st);
-    c->launches += 4;
+    launch_dot(c->y, c->w, m, c->partial, c->d_dot_ctr, c->sc + 0, c->st);
+    c->launches += 2;
     cudaMemcpyAsync(c->h_sc, c->sc, sizeof(double) * 8, cudaMemcpyDeviceToHost, c->st);
     cudaEvent_t ready = nullptr;
     if (j == 1) {
@@ -1536,10 +1536,10 @@ PcgOut pcg_core(tfeti_ctx* c, double* x, double* r, double tol_abs, int maxit, b
     launch_p_update(m, c->y, c->pdir, c->sc, j == 1, c->st);   // p = y + beta p
     if (fp32) op_F32(c, c->pdir, c->Fp);
     else op_F(c, c->pdir, c->Fp);                              // F p
-    launch_dot(c->pdir, c->Fp, m, c->partial, c->sc + 2, c->st);
+    launch_dot(c->pdir, c->Fp, m, c->partial, c->d_dot_ctr, c->sc + 2, c->st);
     launch_lam_r_update(m, c->pdir, c->Fp, x, r, c->sc, c->st);
     cudaMemcpyAsync(c->sc + 1, c->sc + 0, sizeof(double), cudaMemcpyDeviceToDevice, c->st);
-    c->launches += 5;
+    c->launches += 4;
     if (ready) {
       cudaEventSynchronize(ready);
       cudaEventDestroy(ready);
@@ -2690,8 +2690,9 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   c->tn = dalloc<double>(c, P.n_dof);
   c->tn2 = dalloc<double>(c, P.n_dof);
   c->partial = dalloc<double>(c, std::max(2 * kRedBlocks, (1 + kDeflMax) * kFusedBlocks));   // dot2, fused kernels
-  c->d_ctr = dalloc<int>(c, 4);                                              // arrival counters of the fused kernels
-  cudaMemsetAsync(c->d_ctr, 0, sizeof(int) * 4, c->st);
+  c->d_ctr = dalloc<int>(c, 5);                                              // arrival counters of the fused kernels
+  cudaMemsetAsync(c->d_ctr, 0, sizeof(int) * 5, c->st);
+  c->d_dot_ctr = c->d_ctr + 4;
   c->sc = dalloc<double>(c, kNumScalars);
   c->d_err = dalloc<int>(c, 1);
   cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);

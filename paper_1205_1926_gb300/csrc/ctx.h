@@ -280,6 +280,7 @@ struct tfeti_ctx {
   float *cW32 = nullptr, *cV32 = nullptr, *cU32 = nullptr;
   double *partial = nullptr, *sc = nullptr, *h_sc = nullptr;
   int* d_ctr = nullptr;                      // arrival counters of the fused inner-iteration kernels
+  int* d_dot_ctr = nullptr;                  // and of the dot products
   int* d_err = nullptr;
   int max_copy = 0;
   // timing

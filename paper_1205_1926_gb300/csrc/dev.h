@@ -503,7 +503,7 @@ void launch_p_update_g(long long n, const double* y, double* p, const double* sc
                        const double* W = nullptr);
 void launch_lam_r_update_g(long long n, const double* p, const double* Fp, double* lam, double* r, const double* sc,
                            cudaStream_t st);
-void launch_dot(const double* x, const double* y, long long n, double* partial, double* out, cudaStream_t st);
+void launch_dot(const double* x, const double* y, long long n, double* partial, int* ctr, double* out, cudaStream_t st);
 void launch_axpby(long long n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st);
 void launch_p_update(long long n, const double* y, double* p, const double* sc, int first, cudaStream_t st);
 void launch_lam_r_update(long long n, const double* p, const double* Fp, double* lam, double* r, double* sc,

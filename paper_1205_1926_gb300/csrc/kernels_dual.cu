@@ -442,23 +442,18 @@ __global__ void k_slots_diff(DevMesh M, const double* __restrict__ v, const doub
   cbuf[sl] = v[d] - t[d];
 }
 
-// Deterministic dot product: fixed grid, fixed per-block order, fixed final order.
-__global__ void k_dot_partial(const double* __restrict__ x, const double* __restrict__ y, long long n,
-                              double* partial) {
+// Deterministic dot product: fixed grid, fixed per-block order; the block that arrives last sums the
+// partials in block order (one launch; ctr: an int, zero between launches).
+__device__ bool grid_sum_last(double s, double* partial, int* ctr, double* red, double* total);
+__global__ void k_dot(const double* __restrict__ x, const double* __restrict__ y, long long n, double* partial, int* ctr,
+                      double* out) {
   __shared__ double red[32];
   double s = 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    s += x[i] * y[i];
+    s = fma(x[i], y[i], s);
   s = block_reduce_sum(s, red);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
-}
-
-__global__ void k_dot_final(const double* partial, int nparts, double* out) {
-  __shared__ double red[32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nparts; i += blockDim.x) s += partial[i];
-  s = block_reduce_sum(s, red);
-  if (threadIdx.x == 0) *out = s;
+  double tot = 0.0;
+  if (grid_sum_last(s, partial, ctr, red, &tot) && threadIdx.x == 0) *out = tot;
 }
 
 __global__ void k_axpby(long long n, double a, const double* __restrict__ x, double b, const double* __restrict__ y,
@@ -470,17 +465,22 @@ __global__ void k_axpby(long long n, double a, const double* __restrict__ x, dou
 // Scalars: sc[0] = y.w (current), sc[1] = y.w (previous), sc[2] = p.Fp, sc[3] = w.w,
 // sc[4] = beta, sc[5] = gamma, sc[6] = breakdown flag.
 __global__ void k_p_update(long long n, const double* __restrict__ y, double* p, const double* sc, int first) {
+  __shared__ double s_beta;   // one FP64 division per block (the FP64 pipe is narrow)
+  if (threadIdx.x == 0) s_beta = first ? 0.0 : sc[0] / sc[1];
+  __syncthreads();
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double beta = first ? 0.0 : sc[0] / sc[1];
-  p[i] = first ? y[i] : y[i] + beta * p[i];
+  p[i] = first ? y[i] : y[i] + s_beta * p[i];
 }
 
 __global__ void k_lam_r_update(long long n, const double* __restrict__ p, const double* __restrict__ Fp, double* lam,
                                double* r, const double* sc) {
+  __shared__ double s_gamma;
+  if (threadIdx.x == 0) s_gamma = sc[0] / sc[2];
+  __syncthreads();
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const double gamma = sc[0] / sc[2];
+  const double gamma = s_gamma;
   lam[i] += gamma * p[i];
   r[i] -= gamma * Fp[i];
 }
@@ -1173,9 +1173,8 @@ void launch_lumped32(const DevMesh& M, const double* w, const float* kbb32, cons
   k_lumped<float><<<M.n_sub, 256, smem, st>>>(M, w, kbb32, kbb_off, cbuf);
 }
 
-void launch_dot(const double* x, const double* y, long long n, double* partial, double* out, cudaStream_t st) {
-  k_dot_partial<<<kRedBlocks, 256, 0, st>>>(x, y, n, partial);
-  k_dot_final<<<1, 256, 0, st>>>(partial, kRedBlocks, out);
+void launch_dot(const double* x, const double* y, long long n, double* partial, int* ctr, double* out, cudaStream_t st) {
+  k_dot<<<kRedBlocks, 256, 0, st>>>(x, y, n, partial, ctr, out);
 }
 
 void launch_axpby(long long n, double a, const double* x, double b, const double* y, double* out, cudaStream_t st) {
