@@ -24,7 +24,6 @@ scaling; the solver itself runs on one GPU).
 from __future__ import annotations
 
 import argparse
-import hashlib
 import json
 import os
 import statistics
@@ -43,25 +42,26 @@ UNIT = "s/load_step"
 FP64_NOMINAL_TFLOPS = 1.25    # GB300 FP64 rate as published; the roofline uses the rate measured in the run
 
 
-# DRAM traffic per launch of the banded F-apply kernel at the 64^3 benchmark size, from one ncu capture
-# (dram__bytes_read.sum + dram__bytes_write.sum; the launch-list summary under profiles/ gives the
-# command).  Valid only while the kernel source is the one measured.
-MEASURED_TRAFFIC = {"k_sub_solve": {"workload": "cube64_8x8x8", "bytes": 34.37e6,
-                                    "src": "paper_1205_1926_gb300/csrc/kernels_band.cu",
-                                    "sha256": "5f8f884233206d10cad9c65b326615a3ce4106e7bd603f2808adf1301e97fb6d"}}
-
-
-def measured_traffic(kernel, workload):
-    rec = MEASURED_TRAFFIC.get(kernel)
-    if rec is None or rec["workload"] != workload:
-        return None
-    try:
-        with open(os.path.join(ROOT, rec["src"]), "rb") as fh:
-            if hashlib.sha256(fh.read()).hexdigest() != rec["sha256"]:
-                return None
-    except OSError:
-        return None
-    return rec["bytes"]
+def digit_product(w, boundary):
+    """Tensor-core work of one FP64 K^+ pass by the digit product (28 BF16 digit products of every box with
+    its shape's dense K^+, on all dofs or on the boundary dofs; shapes with at least 4 boxes and at most 3072
+    dofs), and whether every box takes it."""
+    count = {}
+    for k in range(len(w.cuts[2]) - 1):
+        for j in range(len(w.cuts[1]) - 1):
+            for i in range(len(w.cuts[0]) - 1):
+                a = tuple(w.cuts[d][q + 1] - w.cuts[d][q] for d, q in enumerate((i, j, k)))
+                count[a] = count.get(a, 0) + 1
+    flops, every = 0.0, True
+    for a, c in count.items():
+        n = 3 * (a[0] + 1) * (a[1] + 1) * (a[2] + 1)
+        inner = 3 * max(0, a[0] - 1) * max(0, a[1] - 1) * max(0, a[2] - 1)
+        if c < 4 or n > 3072:
+            every = False
+            continue
+        m = n - inner if boundary else n
+        flops += 28.0 * 2.0 * c * m * m
+    return flops, every
 
 
 def algorithmic_fapply(w):
@@ -324,7 +324,7 @@ def replica_value(elapsed_max, steps, world):
 ARMS = ("fp64", "mixed", "mixed_history", "mixed_learned")
 EXTRA_ARMS = ("mixed_learned_deflated", "mixed_history_bf16")   # measured variants that lose (--extra-arms)
 ARM_NOTES = {
-    "fp64": "Algorithm 3 in FP64 (banded K^+ applies), the paper's method",
+    "fp64": "Algorithm 3 in FP64 (K^+ by digit products and banded sweeps), the paper's method",
     "mixed": "FP64-refined PCGP: FP32 dual Schur blocks on the tensor cores (elastic) and FP32 banded solves "
              "(plastic), FP32 projector and preconditioner inside; FP64 residual and stopping test",
     "mixed_history": "the mixed arm with each dual solve started from the Galerkin-optimal combination of the "
@@ -518,30 +518,34 @@ def run_gpu(args, rank, world, local_rank):
     units = args.steps * world
     pk, pk_kind = peaks()
     tm = main["tm"]
-    # F-apply kernels: the banded K^+ solves (k_sub_solve: every F-apply of the FP64 arm, the residual
-    # solves of the mixed arms) and, with --fapply schur, the FP64 dual-Schur DGEMM.  The roofline object
-    # describes the one with the larger share of the headline arm's device time; the other sits beside it.
-    # Both are FP64-FMA-bound on this GPU (0.25 flop/B against a ridge of fp64 / hbm ~ 0.18 flop/B), so the
-    # peak is the FP64 FMA rate measured in this run.
+    # F-apply passes: K^+ of every box (the F-applies of the FP64 arm, the residual solves of the mixed
+    # arms) and, with --fapply schur, the FP64 dual-Schur DGEMM.  The roofline object describes the one with
+    # the larger share of the headline arm's device time; the other sits beside it.  Where every box's shape
+    # takes the digit product (kernels_digits.cu) a pass is tensor-core work: its peak is the BF16 rate, and
+    # the method's FP64 flops over its time are given beside it.  Otherwise the banded sweeps set the time,
+    # bound by the FP64 FMA rate measured in this run.
     algo = algorithmic_fapply(w)
     avg_f_ms = tm["f_apply_ms_total"] / max(tm["f_apply_launches"], 1)
     achieved_tf = algo["flops"] / (avg_f_ms * 1e-3) / 1e12 if avg_f_ms > 0 else None
-    traffic = measured_traffic("k_sub_solve", w.name)
-    dram_gbs = traffic / (avg_f_ms * 1e-3) / 1e9 if (traffic and avg_f_ms > 0) else None
     peak_kind = (f"FP64 FMA rate measured in this run (tfeti_measure_fp64_fma); nominal {FP64_NOMINAL_TFLOPS}")
-    banded = {"bound": "alu", "achieved": achieved_tf, "peak": fp64_peak, "unit": "TFLOP/s",
-              "frac": achieved_tf / fp64_peak if achieved_tf else None,
-              "traffic": traffic,
-              "kernel": "k_sub_solve (banded forward/backward substitution with the factor records, FP64)",
-              "peak_kind": peak_kind,
-              "algorithmic": algo | {"note": "per launch: every subdomain's banded factor n (bw + 1) entries, "
-                                             "2 flops per entry and right-hand side, forward and backward sweep"},
-              "total_ms": tm["f_apply_ms_total"], "launches": tm["f_apply_launches"], "avg_launch_ms": avg_f_ms,
-              "executed_flops_per_launch": tm["f_apply_flops"],
-              "hbm": {"dram_gbs": dram_gbs, "peak_gbs": pk["hbm_gbs"],
-                      "frac": dram_gbs / pk["hbm_gbs"] if dram_gbs else None,
-                      "of": f"{pk_kind} hbm_gbs; DRAM bytes per launch from the ncu capture (traffic): the "
-                            "shared elastic factor record stays in L2, so HBM does not bound this kernel"}}
+    method = {"achieved": achieved_tf, "peak": fp64_peak, "unit": "TFLOP/s", "peak_kind": peak_kind}
+    digit_flops, all_digits = digit_product(w, boundary=main_arm == "fp64")
+    if all_digits:
+        d_tf = digit_flops / (avg_f_ms * 1e-3) / 1e12 if avg_f_ms > 0 else None
+        banded = {"bound": "tensor", "achieved": d_tf, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
+                  "frac": d_tf / pk["bf16_tflops"] if d_tf else None, "traffic": None,
+                  "kernel": "k_dg_split_x + k_dg_gemm + k_dg_scatter (FP64 K^+ by BF16 digit products, tcgen05)",
+                  "peak_kind": f"{pk_kind} bf16_tflops", "fp64_method": method}
+    else:
+        banded = {"bound": "alu", "achieved": achieved_tf, "peak": fp64_peak, "unit": "TFLOP/s",
+                  "frac": achieved_tf / fp64_peak if achieved_tf else None, "traffic": None,
+                  "kernel": "k_solve_cl / k_sub_solve (banded sweeps, FP64) beside the digit product of the shapes "
+                            "with at least 4 boxes",
+                  "peak_kind": peak_kind}
+    banded |= {"algorithmic": algo | {"note": "per pass: every subdomain's banded factor n (bw + 1) entries, "
+                                              "2 flops per entry and right-hand side, forward and backward sweep"},
+               "total_ms": tm["f_apply_ms_total"], "launches": tm["f_apply_launches"], "avg_launch_ms": avg_f_ms,
+               "executed_flops_per_launch": digit_flops if all_digits else tm["f_apply_flops"]}
     schur = None
     if tm["schur_launches"] > 0 and tm["schur_ms_total"] > 0:
         s_tf = tm["schur_flops_total"] / (tm["schur_ms_total"] * 1e-3) / 1e12

@@ -112,11 +112,12 @@ __device__ __forceinline__ void store_digits8(const double* v, int emax, uint4* 
   for (int i = 0; i < kS; ++i) dst[i * digit_stride16] = make_uint4(w[i][0], w[i][1], w[i][2], w[i][3]);
 }
 
-// 2^(e - 23) for the biased exponent field emax of a row's largest entry (the integer product
-// in units of 2^-32 times the two rows' scales is the result); NaN for a non-finite row.
+// 2^(e - 7) with 2^e the power of two above a row's largest entry, emax its biased exponent
+// field (the integer product in units of 2^-kUnit times the two rows' scales is the result);
+// NaN for a non-finite row.
 __device__ __forceinline__ double row_scale(int emax) {
   if (emax >= 0x7ff) return __longlong_as_double(0x7ff8000000000000LL);
-  return scalbn(1.0, emax - 1022 - 7) ;
+  return scalbn(1.0, emax - 1022 - 7);
 }
 
 __device__ __forceinline__ int exp_field(double v) {
