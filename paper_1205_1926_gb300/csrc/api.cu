@@ -2464,10 +2464,15 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   for (size_t i = 0; i < (size_t)P.n_copy; ++i) bt_ptr[i + 1] += bt_ptr[i];
   bt_row.resize((size_t)bt_ptr[(size_t)P.n_copy]);
   bt_val.resize(bt_row.size());
+  std::vector<SlotRow> slot_row((size_t)P.n_copy, SlotRow{-1, 0, 0.0});
   for (const Group& g : P.groups)
     for (int j = 0; j < g.k; ++j) {
       int e = bt_ptr[(size_t)g.slot[j]];
       if (g.nrows == 0) continue;
+      const int r0 = std::max(j, 1);
+      if (g.dirichlet) slot_row[(size_t)g.slot[j]] = {(int)g.row0 + j, 0, 1.0};
+      else if (r0 < g.k)
+        slot_row[(size_t)g.slot[j]] = {(int)g.row0 + r0 - 1, g.k << 16 | r0 << 8 | j, helmert_coef(r0, j)};
       if (g.dirichlet) {
         bt_row[e] = (int)g.row0 + j;
         bt_val[e] = 1.0;
@@ -2478,14 +2483,21 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
         bt_val[e] = helmert_coef(r, j);
       }
     }
+  std::vector<RowSlots> row_slots((size_t)P.n_mult);
+  for (long long row = 0; row < P.n_mult; ++row) {
+    const Group& g = P.groups[P.row_group[row]];
+    const int rr = P.row_r[row];
+    if (g.dirichlet) row_slots[row] = {(int)g.slot[rr], -1, 0, P.row_group[row]};
+    else row_slots[row] = {(int)g.slot[0], (int)g.slot[1], rr + 1, P.row_group[row]};
+  }
   M.subs = c->d_subs;
   M.n_sub = ns;
   M.groups = upload(c, gd);
   M.bt_ptr = upload(c, bt_ptr);
   M.bt_row = upload(c, bt_row);
   M.bt_val = upload(c, bt_val);
-  M.slot_group = upload(c, P.slot_group);
-  M.slot_j = upload(c, P.slot_j);
+  M.slot_row = upload(c, slot_row);
+  M.row_slots = upload(c, row_slots);
   M.slot_ldof = upload(c, P.slot_ldof);
   M.slot_sub = upload(c, P.slot_sub);
   M.row_group = upload(c, P.row_group);

@@ -55,13 +55,31 @@ struct GroupDev {
 // kernels read the header (row0, k, nrows, dirichlet) of a group as one 16-byte load
 static_assert(sizeof(GroupDev) % 16 == 0 && offsetof(GroupDev, dirichlet) == 12, "GroupDev header layout");
 
+// Column of B at one copy slot, i.e. one row of B^T: its first multiplier row (-1: none) and that entry, and the
+// Helmert rows that follow it, r = r0 + 1 .. k - 1 of a free group (rest = k << 16 | r0 << 8 | j; 0 for a Dirichlet
+// row).  Almost every slot has one entry (copies shared by two subdomains, Dirichlet rows), so (B^T x) costs one
+// coalesced 16-byte load and one gather of x instead of the chain slot -> group number -> header of an 80-byte group
+// record -> x and the Helmert table.  Latency and load sectors bound these gathers: 1728 boxes of 8^3, splitting of
+// B^T lambda 59 -> 45 us; 512 boxes, FP32 lumped preconditioner 29.4 -> 26.7 us, operand gather 13.2 -> 10.1 us.
+struct alignas(16) SlotRow {
+  int row, rest;
+  double c;
+};
+
+// Row of B: its first two copy slots (s1 = -1: a Dirichlet row, one slot), its Helmert number r and its group, whose
+// record holds the further slots of a row with r > 1.  (B v)[row] of the usual two-slot row is one coalesced load and
+// two gathers: B v over 1728 boxes of 8^3 22.1 -> 14.0 us, over 512 boxes 8.0 -> 6.8 us.
+struct alignas(16) RowSlots {
+  int s0, s1, r, group;
+};
+
 // Everything a kernel needs to know about the mesh and the decomposition.
 struct DevMesh {
   const SubDev* subs;
   int n_sub;
   const GroupDev* groups;
-  const int* slot_group;
-  const int* slot_j;
+  const SlotRow* slot_row;
+  const RowSlots* row_slots;
   const int* slot_ldof;
   const int* slot_sub;
   const int* row_group;

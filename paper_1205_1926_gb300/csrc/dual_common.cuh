@@ -5,70 +5,43 @@
 
 namespace tfeti {
 
-// (B^T x) at one copy slot: Dirichlet groups carry one identity row per copy;
-// free groups carry Helmert rows r = 1..k-1, whose coefficient for copy j is
-// helm[r][j] (non-zero for j <= r).
-__device__ __forceinline__ double bt_at_slot(const DevMesh& M, const double* __restrict__ x, long long slot) {
-  const GroupDev& g = M.groups[M.slot_group[slot]];
-  const int j = M.slot_j[slot];
-  if (g.nrows == 0) return 0.0;
-  if (g.dirichlet) return x[g.row0 + j];
-  double s = 0.0;
-  for (int r = (j > 1 ? j : 1); r < g.k; ++r) s += M.helm[r * 8 + j] * x[g.row0 + r - 1];
+// Adds the entries of a B^T row after its first one (copies shared by more than two subdomains).
+__device__ __forceinline__ double bt_rest(const DevMesh& M, const double* __restrict__ x, int row, int rest, double s) {
+  const int r0 = (rest >> 8) & 0xff, j = rest & 0xff;
+  for (int r = r0 + 1; r < (rest >> 16); ++r) s += __ldg(M.helm + r * 8 + j) * x[row + r - r0];
   return s;
 }
 
-// (B^T x) at U copy slots at once (slot < 0 gives 0), each value summed as bt_at_slot sums it.
-// The loads run stage by stage over the U slots (their groups, the groups' headers, then each
-// value's first Helmert term), so that the U chains of dependent loads overlap; the further
-// terms (copies shared by more than two subdomains) follow in a loop.
+// (B^T x) at U copy slots at once (slot < 0 gives 0): the slots' records, then their first entries'
+// gathers, so that the U chains of dependent loads overlap.
 template <int U>
 __device__ __forceinline__ void bt_at_slots(const DevMesh& M, const double* __restrict__ x, const long long* slot,
                                             double* out) {
-  int g[U], j[U];
-#pragma unroll
-  for (int k = 0; k < U; ++k) {
-    g[k] = slot[k] >= 0 ? __ldg(M.slot_group + slot[k]) : -1;
-    j[k] = slot[k] >= 0 ? __ldg(M.slot_j + slot[k]) : 0;
-  }
-  int4 hd[U];   // GroupDev header: row0, k, nrows, dirichlet
+  int4 rec[U];   // SlotRow
 #pragma unroll
   for (int k = 0; k < U; ++k)
-    hd[k] = g[k] >= 0 ? __ldg(reinterpret_cast<const int4*>(M.groups + g[k])) : make_int4(0, 0, 0, 0);
-  double xv[U], hv[U];
-  int r0[U];
+    rec[k] = slot[k] >= 0 ? __ldg(reinterpret_cast<const int4*>(M.slot_row + slot[k])) : make_int4(-1, 0, 0, 0);
+  double xv[U];
 #pragma unroll
-  for (int k = 0; k < U; ++k) {
-    r0[k] = hd[k].w ? j[k] : (j[k] > 1 ? j[k] : 1);
-    const bool any = hd[k].z != 0 && (hd[k].w || r0[k] < hd[k].y);
-    xv[k] = any ? x[hd[k].x + r0[k] - (hd[k].w ? 0 : 1)] : 0.0;
-    hv[k] = any && !hd[k].w ? __ldg(M.helm + r0[k] * 8 + j[k]) : 0.0;
-  }
+  for (int k = 0; k < U; ++k) xv[k] = rec[k].x >= 0 ? x[rec[k].x] : 0.0;
 #pragma unroll
-  for (int k = 0; k < U; ++k) {
-    if (hd[k].z == 0) {
-      out[k] = 0.0;
-    } else if (hd[k].w) {
-      out[k] = xv[k];
-    } else {
-      double s = 0.0;
-      if (r0[k] < hd[k].y) {
-        s += hv[k] * xv[k];
-        for (int r = r0[k] + 1; r < hd[k].y; ++r) s += M.helm[r * 8 + j[k]] * x[hd[k].x + r - 1];
-      }
-      out[k] = s;
-    }
-  }
+  for (int k = 0; k < U; ++k)
+    out[k] = bt_rest(M, x, rec[k].x, rec[k].y, __hiloint2double(rec[k].w, rec[k].z) * xv[k]);
+}
+
+__device__ __forceinline__ double bt_at_slot(const DevMesh& M, const double* __restrict__ x, long long slot) {
+  double v;
+  bt_at_slots<1>(M, x, &slot, &v);
+  return v;
 }
 
 // (B v)[row] for copy-slot values v.
 __device__ __forceinline__ double b_at_row(const DevMesh& M, const double* __restrict__ v, long long row) {
-  const GroupDev& g = M.groups[M.row_group[row]];
-  const int rr = M.row_r[row];
-  if (g.dirichlet) return v[g.slot[rr]];
-  const int r = rr + 1;
-  double s = 0.0;
-  for (int j = 0; j <= r; ++j) s += M.helm[r * 8 + j] * v[g.slot[j]];
+  const int4 q = __ldg(reinterpret_cast<const int4*>(M.row_slots + row));   // RowSlots
+  const double v0 = v[q.x];
+  if (q.y < 0) return v0;
+  double s = __ldg(M.helm + q.z * 8) * v0 + __ldg(M.helm + q.z * 8 + 1) * v[q.y];
+  for (int j = 2; j <= q.z; ++j) s += M.helm[q.z * 8 + j] * v[M.groups[q.w].slot[j]];
   return s;
 }
 

@@ -167,6 +167,9 @@ __global__ void __launch_bounds__(256) k_dg_split_x(DevMesh M, const DgBlock* __
     __syncthreads();
     if (tid < 6) xs[S.fix[tid]] = 0.0;
   } else {
+    int fix[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) fix[q] = S.fix[q];
     for (int j0 = tid; j0 < kcols; j0 += U * nt) {
       long long sl[U];
       double v[U];
@@ -174,19 +177,16 @@ __global__ void __launch_bounds__(256) k_dg_split_x(DevMesh M, const DgBlock* __
       for (int k = 0; k < U; ++k) {
         const int j = j0 + k * nt;
         const int b = j < n ? __ldg(M.sub_b2s + S.b2s_off + j / 3) : -1;
-        sl[k] = b >= 0 ? (long long)b + j % 3 : -1;
+        const int ld = j < n ? 3 * __ldg(M.shape_bln + S.bnd_off + j / 3) + j % 3 : -1;
+        bool fixed = false;   // fixing dofs are boundary dofs; their rows and columns of S are zero
+#pragma unroll
+        for (int q = 0; q < 6; ++q) fixed |= ld == fix[q];
+        sl[k] = b >= 0 && !fixed ? (long long)b + j % 3 : -1;
       }
       bt_at_slots<U>(M, lam, sl, v);
 #pragma unroll
       for (int k = 0; k < U; ++k)
         if (j0 + k * nt < kcols) xs[j0 + k * nt] = sl[k] >= 0 ? v[k] : 0.0;
-    }
-    __syncthreads();
-    // fixing dofs are boundary dofs; their rows and columns of S are zero
-    for (int j = tid; j < n; j += nt) {
-      const int ld = 3 * M.shape_bln[S.bnd_off + j / 3] + j % 3;
-      if (ld == S.fix[0] || ld == S.fix[1] || ld == S.fix[2] || ld == S.fix[3] || ld == S.fix[4] || ld == S.fix[5])
-        xs[j] = 0.0;
     }
   }
   __syncthreads();
