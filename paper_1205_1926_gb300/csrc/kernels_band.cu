@@ -537,8 +537,11 @@ __device__ __forceinline__ void st_async(const double* p, const uint64_t* bar, u
                "l"(__double_as_longlong(v)), "r"(cluster_addr(bar, rank))
                : "memory");
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 
 // Shared memory of a cluster CTA in doubles: panel slices, the vectors, the own rows' x', the
@@ -641,6 +644,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
     __syncthreads();
     if (tid == 0 && ok && issued < nsteps) fetch(issued++);
   }
+  cluster_arrive();   // every y has arrived in this CTA's vectors
   // backward: column c belongs to lane c % 32 of warp (c / 32) % 4 from its first step to its last
   for (int k = nblk; k < nsteps; ++k) {
     const int b = nsteps - 1 - k, r0 = b * nb, lo = max(0, r0 - bw), nxt = r0 - nb;
@@ -692,7 +696,9 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
     }
     __syncthreads();
     // z' to CTA b % C, which applies the block's D^-T below (only now: until here every warp of that CTA
-    // may still read the y of its own rows from the same entries)
+    // may still read the y of its own rows from the same entries; and in the first step a y sent there must
+    // not arrive after the z' that replaces it: the sums received before the later steps tell that it has)
+    if (k == nblk) cluster_wait();
     if (warp == 0 && lane < rpc && r0 + (int)q * rpc + lane < n)
 #pragma unroll
       for (int r = 0; r < R; ++r) st_cluster(vec + r * npad + r0 + (int)q * rpc + lane, (unsigned)(b % C), zv[r]);
