@@ -181,49 +181,18 @@ int plan_build(const tfeti_problem* prob, Plan& plan) {
   };
   auto has_rows = [&](int64_t g) { return ncopy[g] >= 2 || node_mask(g) != 0; };
 
-  // ---- box-boundary nodes of every shape, grouped by the pattern of their stencil neighbours on the box
-  // boundary (the faces' inner nodes, the rows beside an edge, the edges, ...; lexicographic within a group): the
-  // kernels that walk boundary nodes or copy slots then find equal work and adjacent table entries in
-  // adjacent threads, on the x and y faces as on the z faces
-  std::vector<std::vector<int32_t>> shape_order(plan.shapes.size());
-  for (size_t k = 0; k < plan.shapes.size(); ++k) {
-    const auto& sh = plan.shapes[k];
-    const int m[3] = {sh.dims[0] + 1, sh.dims[1] + 1, sh.dims[2] + 1};
-    auto on = [&m](int i, int j, int l) {
-      return i >= 0 && j >= 0 && l >= 0 && i < m[0] && j < m[1] && l < m[2] &&
-             (i == 0 || j == 0 || l == 0 || i == m[0] - 1 || j == m[1] - 1 || l == m[2] - 1);
-    };
-    std::vector<std::pair<std::pair<int, int>, int32_t>> nodes;   // ((-neighbours, pattern), local node)
-    int ln = 0;
-    for (int lk = 0; lk < m[2]; ++lk)
-      for (int lj = 0; lj < m[1]; ++lj)
-        for (int li = 0; li < m[0]; ++li, ++ln) {
-          if (!on(li, lj, lk)) continue;
-          int cnt = 0, pattern = 0;
-          for (int t = 0; t < 27; ++t)
-            if (on(li + t % 3 - 1, lj + (t / 3) % 3 - 1, lk + t / 9 - 1)) {
-              ++cnt;
-              pattern |= 1 << t;
-            }
-          nodes.push_back({{-cnt, pattern}, ln});
-        }
-    std::sort(nodes.begin(), nodes.end());
-    for (const auto& v : nodes) shape_order[k].push_back(v.second);
-  }
-
-  // ---- interface nodes and copy slots per subdomain (in its shape's order)
+  // ---- interface nodes and copy slots per subdomain (local node order)
   std::vector<std::vector<int32_t>> iface_index(ns);   // local node -> interface index or -1
   int64_t slot_off = 0;
   for (int p = 0; p < ns; ++p) {
     auto& s = plan.subs[p];
     auto& ix = iface_index[p];
     ix.assign(s.n_nodes, -1);
-    int cnt = 0;
-    for (int32_t ln : shape_order[s.shape])
-      if (has_rows(gnode_of(s, ln % s.nn[0], (ln / s.nn[0]) % s.nn[1], ln / (s.nn[0] * s.nn[1])))) ix[ln] = cnt++;
-    for (int ln = 0; ln < s.n_nodes; ++ln)
-      if (ix[ln] < 0 && has_rows(gnode_of(s, ln % s.nn[0], (ln / s.nn[0]) % s.nn[1], ln / (s.nn[0] * s.nn[1]))))
-        return bad(plan, "internal: interface node off the box boundary"), TFETI_ERR_ARG;
+    int cnt = 0, ln = 0;
+    for (int lk = 0; lk < s.nn[2]; ++lk)
+      for (int lj = 0; lj < s.nn[1]; ++lj)
+        for (int li = 0; li < s.nn[0]; ++li, ++ln)
+          if (has_rows(gnode_of(s, li, lj, lk))) ix[ln] = cnt++;
     s.copy_off = slot_off;
     s.n_copy = 3 * cnt;
     slot_off += s.n_copy;
@@ -287,10 +256,15 @@ int plan_build(const tfeti_problem* prob, Plan& plan) {
       std::vector<int32_t> ln2b(nx_ * ny_ * nz_, -1);
       sh.bnd_off = boff;
       sh.n_bnd = 0;
-      for (int32_t ln : shape_order[&sh - plan.shapes.data()]) {
-        ln2b[ln] = sh.n_bnd++;
-        plan.shape_bln.push_back(ln);
-      }
+      for (int lk = 0; lk < nz_; ++lk)
+        for (int lj = 0; lj < ny_; ++lj)
+          for (int li = 0; li < nx_; ++li) {
+            const bool on = li == 0 || lj == 0 || lk == 0 || li == nx_ - 1 || lj == ny_ - 1 || lk == nz_ - 1;
+            if (!on) continue;
+            const int ln = li + nx_ * (lj + ny_ * lk);
+            ln2b[ln] = sh.n_bnd++;
+            plan.shape_bln.push_back(ln);
+          }
       for (int b = 0; b < sh.n_bnd; ++b) {
         const int ln = plan.shape_bln[boff + b];
         const int li = ln % nx_, lj = (ln / nx_) % ny_, lk = ln / (nx_ * ny_);
