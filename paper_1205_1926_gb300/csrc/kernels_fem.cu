@@ -302,26 +302,12 @@ struct RmConst {
   double cs, kd, a0;           // sqrt(2/3) c, 1 / (3 mu + H), 2 mu c, c = 3 mu / (3 mu + H)
 };
 
-// 1/sqrt(d) and sqrt(d) for normal d of moderate exponent: the hardware's approximation (relative
-// error below 2^-19), one step of the third-order iteration y (1 + e (1/2 + 3/8 e)), e = 1 - d y^2,
-// and a Newton correction of the root.
-__device__ __forceinline__ void root_pair(double d, double& root, double& inv) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
-  const double e = fma(-(d * y), y, 1.0);
-  y = fma(y * e, fma(0.375, e, 0.5), y);
-  const double r = d * y;
-  const double hy = __hiloint2double(__double2hiint(y) - 0x100000, __double2loint(y));   // y / 2
-  root = fma(fma(-r, r, d), hy, r);
-  inv = y;
-}
-
 // One thread per Gauss point, the 8 points of an element in 8 consecutive lanes (blockDim and n_gp
 // multiples of 8); lanes past n_gp compute on the last element and store nothing.
-// Bound by the FP64 pipe: about 52 operations per elastic point and 20 more at a yielding one (74
-// and 56 with a square root, three divisions and derivatives formed one by one): at 96^3, half of the
-// points yielding, 968 us for 7.1 million points where that form took 1714.  The material constants
-// come from the host; the root of |dev tau|^2 and its inverse share one iteration.  kOut: 0 = increments only, 1 = also a, b, n, 2 = also T.
+// Bound by the FP64 pipe: about 52 operations per elastic point and, at a point past the test below, a square
+// root, a division and 11 more (74 per elastic point, two further divisions and the derivatives formed one by one in
+// the form before): at 96^3, half of the points yielding, 1028 us for 7.1 million points where that form took
+// 1714.  The material constants come from the host.  kOut: 0 = increments only, 1 = also a, b, n, 2 = also T.
 template <int kOut>
 __global__ void __launch_bounds__(128) k_return_map(DevMesh M, RmConst K, const double* __restrict__ du,
                                                     const double* __restrict__ sig_k, const double* __restrict__ kap_k,
@@ -367,14 +353,8 @@ __global__ void __launch_bounds__(128) k_return_map(DevMesh M, RmConst K, const 
   double phi = 0.0, inv = 0.0;
   bool pl = false;
   if (__double_as_longlong(1.5 * nrm2) > __double_as_longlong(yield * yield)) {
-    double nrm;
-    const unsigned ef = ((unsigned)__double2hiint(nrm2) >> 20) & 0x7ffu;
-    if (ef - 0x100u < 0x600u) {
-      root_pair(nrm2, nrm, inv);
-    } else {   // extreme magnitudes, infinities and NaN
-      nrm = sqrt(nrm2);
-      inv = 1.0 / nrm;
-    }
+    const double nrm = sqrt(nrm2);
+    inv = 1.0 / nrm;
     phi = fma(kSqrt32, nrm, -yield);
     pl = phi > kTie * yield;
   }
