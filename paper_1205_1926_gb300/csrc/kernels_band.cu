@@ -585,7 +585,9 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
     bulk_copy(pan + (k % kClStages) * lay.slice, fac + (long long)step_block(k) * rec + (long long)q * rpc * bw, pbytes,
               &bar[k % kClStages]);
   };
-  bool ok = true;   // after a wait that gave up, the remaining steps run through without waiting
+  // after a wait that gave up, the remaining steps run through without waiting; thread 0 then neither fetches
+  // panels nor opens exchange phases any more (a phase may be opened once the one before it has completed)
+  bool ok = true;
   auto wait_panel = [&](int k) {
     if (ok) ok = mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1));
   };
@@ -618,7 +620,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
   // forward: a warp's NR rows, columns across the lanes
   for (int k = 0; k < nblk; ++k) {
     const int r0 = k * nb, c0 = r0 - bw, jlo = max(0, -c0);
-    if (tid == 0) mbar_expect_tx(&xbar[k % kClRing], (uint32_t)(min(nb, n - r0) * R * (int)sizeof(T)));
+    if (tid == 0 && ok) mbar_expect_tx(&xbar[k % kClRing], (uint32_t)(min(nb, n - r0) * R * (int)sizeof(T)));
     wait_panel(k);
     const T* P = pan + (k % kClStages) * lay.slice + warp * NR * bw;
     T acc[R][NR] = {};
@@ -648,7 +650,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
   // backward: column c belongs to lane c % 32 of warp (c / 32) % 4 from its first step to its last
   for (int k = nblk; k < nsteps; ++k) {
     const int b = nsteps - 1 - k, r0 = b * nb, lo = max(0, r0 - bw), nxt = r0 - nb;
-    if (tid == 0 && b > 0) mbar_expect_tx(&xbar[k % kClRing], (uint32_t)(nb * R * (int)sizeof(T)));
+    if (tid == 0 && ok && b > 0) mbar_expect_tx(&xbar[k % kClRing], (uint32_t)(nb * R * (int)sizeof(T)));
     // z' of the own rows: y less the CTAs' sums (lane = CTA x row), in every warp
     if (k > nblk) wait_exchange(k - 1);
     T zv[R];
@@ -709,6 +711,11 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
     for (int k = max(0, issued - kClStages); k < issued; ++k)   // copies still in flight land first
       mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1));
   cluster_barrier();   // the z' of the blocks below have arrived
+  if (!ok) {           // the other CTAs' last asynchronous stores, which were not waited for, land before this CTA ends
+    const long long t0 = clock64();
+    while (clock64() - t0 < (1LL << 17)) {
+    }
+  }
 
   // z = D^-T z' on the blocks b % C == q
   __shared__ T s_col[kClThreads][R];

@@ -435,7 +435,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
       __syncwarp();
       if (lane == 0) mbar_arrive(drained_bar);
     }
-    if (ok) ok = mbar_wait(done_bar, 0u);
+    // also where a wait gave up: no MMA may be in flight when TMEM is freed and the CTA ends
+    if (!mbar_wait(done_bar, 0u)) ok = false;
     ok = __all_sync(0xffffffffu, ok);
     if (!ok && lane == 0) atomicOr(s_fail, 1);
     if (ok) {
