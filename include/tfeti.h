@@ -441,6 +441,13 @@ int tfeti_get_tuning(tfeti_ctx* ctx, int32_t* schur_threshold, int32_t* n_schur_
  * results (profilers that do not see into conditional graph bodies need this). */
 int tfeti_set_graphs(tfeti_ctx* ctx, int32_t enable);
 
+/* Limit of the bounded device waits of the banded solves and of the digit product, in SM
+ * cycles: 2^31 (default, about a second) at most.  A wait that gives up ends its kernel, after
+ * its own copies have landed, and the call that launched it returns TFETI_ERR_TIMEOUT; its
+ * outputs hold nothing to be used, and the context stays usable.  0: every such wait gives up
+ * without a look (a check of that way out). */
+int tfeti_set_wait_limit(tfeti_ctx* ctx, int64_t cycles);
+
 /* Load magnitude of the workloads: t_y = sigma_y / max_g sqrt(3/2) ||dev sigma_g||
  * for the elastic response to the unit traction `dir` (host double[3]) on the
  * traction face, solved with tfeti_dual_pcg at rtol.  Requires the zero

@@ -92,6 +92,7 @@ SIGNATURES = {
     "tfeti_first_yield_traction": (C.c_int, [_P, _P, _D, C.POINTER(_D)]),
     "tfeti_set_precision": (C.c_int, [_P, _I, _D]),
     "tfeti_set_graphs": (C.c_int, [_P, _I]),
+    "tfeti_set_wait_limit": (C.c_int, [_P, C.c_int64]),
     "tfeti_set_fapply": (C.c_int, [_P, _I]),
     "tfeti_set_schur_format": (C.c_int, [_P, _I]),
     "tfeti_set_schur_threshold": (C.c_int, [_P, _I]),
@@ -395,6 +396,10 @@ class Context:
     def set_graphs(self, enable: bool):
         """Inner PCGP of the mixed mode as one CUDA graph launch (default) or kernel by kernel."""
         return self._check(self.lib.tfeti_set_graphs(self.h, 1 if enable else 0), "tfeti_set_graphs")
+
+    def set_wait_limit(self, cycles: int = 1 << 31):
+        """Limit of the bounded device waits in SM cycles (default 2^31; 0: each gives up at once)."""
+        return self._check(self.lib.tfeti_set_wait_limit(self.h, int(cycles)), "tfeti_set_wait_limit")
 
     def first_yield_traction(self, direction, rtol=1e-12) -> float:
         arr = (C.c_double * 3)(*direction)

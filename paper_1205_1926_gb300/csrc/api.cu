@@ -137,6 +137,24 @@ std::vector<long long> band_workspace(tfeti_ctx* c, const std::vector<int>& list
   return offs;
 }
 
+// Bounded waits that gave up since the last check: read_waits queues the copy of the wait word, check_waits
+// looks at it after the context stream has been synchronised.  Every entry point that runs kernels with
+// such waits does both, so that a call whose result is not to be used says so itself.
+void read_waits(tfeti_ctx* c) { cudaMemcpyAsync(c->h_err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st); }
+
+int check_waits(tfeti_ctx* c) {
+  const int e = *c->h_err & kErrWaits;
+  if (!e) return TFETI_OK;
+  cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+  if (e & kErrGrid) cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->st);   // the barrier restarts at zero
+  sync(c);
+  return fail(c, TFETI_ERR_TIMEOUT,
+              (e & kErrPanel)    ? "a factor-panel copy did not complete within its time limit"
+              : (e & kErrDigits) ? "a copy or MMA of the digit product did not complete within its time limit"
+              : (e & kErrSchur)  ? "a Schur-tile copy or MMA did not complete within its time limit"
+                                 : "a grid-barrier wait of the fused inner iteration gave up");
+}
+
 double dot_host(tfeti_ctx* c, const double* x, const double* y, long long n) {
   launch_dot(x, y, n, c->partial, c->d_dot_ctr, c->sc + 8, c->st);
   c->launches += 1;
@@ -419,6 +437,7 @@ SolveArgs solve_args(tfeti_ctx* c, bool fp32 = false) {
   set_stat(a, fp32 ? c->is32 : c->is64);
   a.max_bw = c->plan.max_bw;
   a.cl_max = c->cl_max;
+  a.wait_limit = c->wait_limit;
   return a;
 }
 
@@ -536,6 +555,7 @@ void fp64_pass(tfeti_ctx* c, const SolveArgs& a) {
     d.sB = c->dg_sB;
     d.out = c->dg_out;
     d.err = c->d_err;
+    d.wait_limit = c->wait_limit;
     const bool to_c = a.out_mode == 0 || a.out_mode == 3, to_d = a.out_mode == 1 || a.out_mode == 3;
     c->launches += launch_dg_product(c->M, d, a.in_mode == 1 ? a.src : nullptr, a.lam, a.in_mode == 0 ? 1.0 : -1.0,
                                      to_c ? a.cbuf : nullptr, to_d ? a.dst : nullptr, c->st);
@@ -674,7 +694,10 @@ int form_schur_blocks(tfeti_ctx* c) {
     launch_schur_tile_S(c->S32 + c->s_off_c[sh], n_bd, false, c->Shi + c->s_tile_off[sh], c->Slo + c->s_tile_off[sh],
                         c->st);
     c->launches += 2;
+    read_waits(c);
     sync(c);
+    const int wst = check_waits(c);
+    if (wst != TFETI_OK) return wst;
   }
   c->schur_ready = true;
   return cuda_check(c, "forming dual Schur blocks");
@@ -837,8 +860,14 @@ int ensure_kinv(tfeti_ctx* c) {
     launch_sub_solve(c->M, a, c->st);
     c->launches += 1;
   }
+  read_waits(c);
   sync(c);
   dfree(c, d_items, items.size());
+  const int wst = check_waits(c);
+  if (wst != TFETI_OK) {
+    dfree(c, kinv, (size_t)std::max(1LL, tot));
+    return wst;
+  }
   c->kinv = kinv;
   c->kinv_off = off;
   return cuda_check(c, "forming dense K^+ blocks");
@@ -1076,15 +1105,15 @@ int wood_setup(tfeti_ctx* c, const std::vector<int>& np, bool fp64, bool async =
     if (fp64) c->wood_fac_saved += w.n;
     return cuda_check(c, "Woodbury set-up");
   }
-  w.err = c->d_err;
-  cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+  w.err = c->d_piv;
+  cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
   launch_wood_setup(c->M, w, c->st);
   c->launches += wood_setup_launches(w);
   int herr = 0;
-  cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+  cudaMemcpyAsync(&herr, c->d_piv, sizeof(int), cudaMemcpyDeviceToHost, c->st);
   sync(c);
   if (herr & 8) {   // keep the refactorisation and the banded solves for this assembly
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+    cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
     std::fill(c->h_wood.begin(), c->h_wood.end(), 0);
     c->wood.n = 0;
     c->wood_fallbacks += 1;
@@ -1143,14 +1172,14 @@ int wood_materialize(tfeti_ctx* c) {
   cudaMemcpyAsync(c->d_list_fac, facs.data(), sizeof(long long) * facs.size(), cudaMemcpyHostToDevice, c->st);
   launch_band_fill(M, c->d_list, (int)list.size(), c->elem_np, c->dKe, c->band_ws, c->d_list_off, 0, max_rows,
                    c->plan.max_bw, c->st);
-  cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-  launch_band_chol(M, c->d_list, (int)list.size(), c->d_list_off, c->band_ws, c->d_list_fac, c->fac_own, c->d_err,
+  cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
+  launch_band_chol(M, c->d_list, (int)list.size(), c->d_list_off, c->band_ws, c->d_list_fac, c->fac_own, c->d_piv,
                    c->plan.max_bw, c->n_sm, c->st);
   launch_fac_to_f32(c->fac_own, c->fac32_own, c->d_list_fac, (int)list.size(), len, c->st);
   c->launches += 3;
   c->factor_launches += 1;
   int herr = 0;
-  cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+  cudaMemcpyAsync(&herr, c->d_piv, sizeof(int), cudaMemcpyDeviceToHost, c->st);
   sync(c);
   if (herr) return fail(c, TFETI_ERR_NUMERIC, "non-positive pivot in a subdomain factorisation");
   c->wood.fp64 = false;
@@ -1439,16 +1468,16 @@ int assemble(tfeti_ctx* c, const double* du, const double* df, double* f_out, bo
         cudaMemcpyAsync(f_out, c->f_full, sizeof(double) * M.n_dof, cudaMemcpyDeviceToDevice, c->st);
       return cuda_check(c, "assemble");
     }
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+    cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
     cudaEvent_t e0 = c->events ? c->fac_e0 : nullptr, e1 = c->events ? c->fac_e1 : nullptr;
     if (e0) cudaEventRecord(e0, c->st);
     launch_band_chol(M, c->d_list, (int)list.size(), c->d_list_off, c->band_ws, c->d_list_fac, c->fac_own,
-                     c->d_err, c->plan.max_bw, c->n_sm, c->st);
+                     c->d_piv, c->plan.max_bw, c->n_sm, c->st);
     if (e1) cudaEventRecord(e1, c->st);
     c->launches += 2;
     c->factor_launches += 1;
     int herr = 0;
-    cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+    cudaMemcpyAsync(&herr, c->d_piv, sizeof(int), cudaMemcpyDeviceToHost, c->st);
     sync(c);
     if (e0) {
       float ms = 0.f;
@@ -1466,9 +1495,9 @@ int assemble(tfeti_ctx* c, const double* du, const double* df, double* f_out, bo
       // K_ii factors of the plastic subdomains (same slots), on the same band workspaces
       launch_band_fill(c->Mi, c->d_list, (int)list.size(), c->elem_np, c->dKe, c->band_ws, c->d_list_off, 0, max_rows,
                        c->plan.max_bw, c->st, true);
-      cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+      cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
       launch_band_chol(c->Mi, c->d_list, (int)list.size(), c->d_list_off, c->band_ws, c->d_list_fac, c->dfac_own,
-                       c->d_err, c->plan.max_bw, c->n_sm, c->st);
+                       c->d_piv, c->plan.max_bw, c->n_sm, c->st);
       c->launches += 2;
       c->factor_launches += 1;
       if (c->precision == TFETI_PRECISION_MIXED) {
@@ -1478,7 +1507,7 @@ int assemble(tfeti_ctx* c, const double* du, const double* df, double* f_out, bo
         c->launches += 1;
       }
       int derr = 0;
-      cudaMemcpyAsync(&derr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+      cudaMemcpyAsync(&derr, c->d_piv, sizeof(int), cudaMemcpyDeviceToHost, c->st);
       sync(c);
       if (derr) return fail(c, TFETI_ERR_NUMERIC, "non-positive pivot in a Dirichlet-preconditioner factorisation");
     }
@@ -2219,11 +2248,15 @@ int dual_pcg(tfeti_ctx* c, const double* f, double* u_out, double* lambda_out, c
   wood_join(c);   // the inner solves read the set-up's FP32 part
   double r0 = std::sqrt(std::max(0.0, dot_host(c, c->r, c->r, m)));
   {
-    const int fst = check_factorisation(c);   // pivots of a deferred refactorisation
-    if (fst != TFETI_OK) return fst;
     int redo = 0;
-    const int wst = wood_check(c, &redo);      // pivots of an asynchronous Woodbury set-up
-    if (wst != TFETI_OK) return wst;
+    int fst = check_factorisation(c);          // pivots of a deferred refactorisation
+    if (fst == TFETI_OK) fst = wood_check(c, &redo);   // pivots of an asynchronous Woodbury set-up
+    if (fst != TFETI_OK) {
+      read_waits(c);
+      sync(c);
+      const int wst = check_waits(c);          // of the residual solve: not left for a later call
+      return wst != TFETI_OK ? wst : fst;
+    }
     if (redo) {
       residual_solve(c, f, c->lam_im, c->r);
       r0 = std::sqrt(std::max(0.0, dot_host(c, c->r, c->r, m)));
@@ -2342,19 +2375,12 @@ int dual_pcg(tfeti_ctx* c, const double* f, double* u_out, double* lambda_out, c
   }
   if (lambda_out) cudaMemcpyAsync(lambda_out, c->lam, sizeof(double) * m, cudaMemcpyDeviceToDevice, c->st);
   cudaMemsetAsync(c->sc + 6, 0, sizeof(double), c->st);
-  int herr = 0;
-  cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+  read_waits(c);
   sync(c);
   collect_events(c);
   int cst = cuda_check(c, "tfeti_dual_pcg");
+  if (cst == TFETI_OK) cst = check_waits(c);
   if (cst != TFETI_OK) return cst;
-  if (herr & 38) {
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-    if (herr & 32) cudaMemsetAsync(c->d_bar, 0, 2 * sizeof(unsigned), c->st);   // the barrier restarts at zero
-    return fail(c, TFETI_ERR_TIMEOUT, (herr & 2)    ? "a factor-panel copy did not complete within its time limit"
-                                      : (herr & 4) ? "a Schur-tile copy or MMA did not complete within its time limit"
-                                                   : "a grid-barrier wait of the fused inner iteration gave up");
-  }
   if (status == TFETI_OK && !converged) status = fail(c, TFETI_ERR_NOT_CONVERGED, "PCGP iteration limit reached");
   if (info) {
     info->iterations = it;
@@ -2707,7 +2733,10 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
   c->d_dot_ctr = c->d_ctr + 4;
   c->sc = dalloc<double>(c, kNumScalars);
   c->d_err = dalloc<int>(c, 1);
+  c->d_piv = dalloc<int>(c, 1);
   cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+  if (cudaMallocHost(&c->h_err, sizeof(int)) != cudaSuccess) throw std::bad_alloc();
+  *c->h_err = 0;
   if (cudaMallocHost(&c->h_sc, kNumScalars * sizeof(double)) != cudaSuccess) throw std::bad_alloc();
   cudaMemsetAsync(c->u, 0, sizeof(double) * P.n_dof, c->st);
   cudaMemsetAsync(c->sig, 0, sizeof(double) * 6 * P.n_gp, c->st);
@@ -2734,7 +2763,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     int* ti = upload(c, P.trip_i);
     int* tj = upload(c, P.trip_j);
     double* work = nullptr;
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
+    cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
     c->coarse = CoarseOp{};
     c->coarse.mode = mode;
     c->coarse.l = c->l;
@@ -2745,7 +2774,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
         cudaGetLastError();
         throw std::bad_alloc();
       }
-      dense_cholesky_inverse(c->H, work, c->l, c->d_err, c->st);
+      dense_cholesky_inverse(c->H, work, c->l, c->d_piv, c->st);
       c->coarse.H = c->H;
     } else {
       const int n_pl = 6 * per_plane;
@@ -2761,7 +2790,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
         throw std::bad_alloc();
       }
       coarse_planes_factor(c->cW, c->cAoff, c->cV, c->cU, n_pl, n_planes, work + dense_inverse_work(n_pl), work,
-                           c->d_err, c->st);
+                           c->d_piv, c->st);
       c->coarse.n_pl = n_pl;
       c->coarse.n_planes = n_planes;
       c->coarse.W = c->cW;
@@ -2769,7 +2798,7 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
       c->coarse.U = c->cU;
     }
     int herr = 0;
-    cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+    cudaMemcpyAsync(&herr, c->d_piv, sizeof(int), cudaMemcpyDeviceToHost, c->st);
     sync(c);
     cudaFree(work);
     if (herr) return fail(c, TFETI_ERR_SINGULAR, "coarse matrix G G^T is not positive definite");
@@ -2877,10 +2906,10 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     long long* dfo = upload(c, foffs);
     launch_band_fill(c->Mi, dl, (int)boffs.size(), c->elem_np, c->dKe, c->band_ws, dbo, 1, max_rows, P.max_bw, c->st,
                      true);
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-    launch_band_chol(c->Mi, dl, (int)boffs.size(), dbo, c->band_ws, dfo, c->dfac, c->d_err, P.max_bw, c->n_sm, c->st);
+    cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
+    launch_band_chol(c->Mi, dl, (int)boffs.size(), dbo, c->band_ws, dfo, c->dfac, c->d_piv, P.max_bw, c->n_sm, c->st);
     int herr = 0;
-    cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+    cudaMemcpyAsync(&herr, c->d_piv, sizeof(int), cudaMemcpyDeviceToHost, c->st);
     sync(c);
     if (herr) return fail(c, TFETI_ERR_NUMERIC, "non-positive pivot in a Dirichlet-preconditioner factorisation");
     long long len = 0;
@@ -2906,10 +2935,10 @@ int setup_impl(tfeti_ctx* c, tfeti_ctx* base = nullptr) {
     long long* dof = upload(c, offs);
     long long* dfac = upload(c, facs);
     launch_band_fill(M, dl, (int)reps.size(), c->elem_np, c->dKe, c->band, dof, 1, max_rows, P.max_bw, c->st);
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-    launch_band_chol(M, dl, (int)reps.size(), dof, c->band, dfac, c->fac, c->d_err, P.max_bw, c->n_sm, c->st);
+    cudaMemsetAsync(c->d_piv, 0, sizeof(int), c->st);
+    launch_band_chol(M, dl, (int)reps.size(), dof, c->band, dfac, c->fac, c->d_piv, P.max_bw, c->n_sm, c->st);
     int herr = 0;
-    cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+    cudaMemcpyAsync(&herr, c->d_piv, sizeof(int), cudaMemcpyDeviceToHost, c->st);
     sync(c);
     if (herr) return fail(c, TFETI_ERR_NUMERIC, "non-positive pivot in an elastic template factorisation");
     long long len = 0;
@@ -3101,6 +3130,7 @@ int tfeti_destroy(tfeti_ctx* c) {
   if (c->ev_fac_fork) cudaEventDestroy(c->ev_fac_fork);
   if (c->ev_fac_done) cudaEventDestroy(c->ev_fac_done);
   if (c->h_err_fac) cudaFreeHost(c->h_err_fac);
+  if (c->h_err) cudaFreeHost(c->h_err);
   if (c->st2) cudaStreamDestroy(c->st2);
   if (c->st_mlp) cudaStreamDestroy(c->st_mlp);
   if (c->st_wood) cudaStreamDestroy(c->st_wood);
@@ -3393,6 +3423,13 @@ int tfeti_set_graphs(tfeti_ctx* c, int32_t enable) {
   return TFETI_OK;
 }
 
+int tfeti_set_wait_limit(tfeti_ctx* c, int64_t cycles) {
+  if (!c || cycles < 0 || cycles > (1LL << 31)) return fail(c, TFETI_ERR_ARG, "wait limit must be in 0..2^31 cycles");
+  c->wait_limit = cycles;
+  c->g_inner_stale = true;   // a captured inner iteration holds the limit
+  return TFETI_OK;
+}
+
 int tfeti_set_recycling(tfeti_ctx* c, int32_t q) {
   if (!c || q < 0 || q > kRecMax) return fail(c, TFETI_ERR_ARG, "history size must be in 0..8");
   if (c->mlp_on && (q < 1 || q > kRecMax - 1))
@@ -3640,25 +3677,21 @@ int tfeti_set_state(tfeti_ctx* c, const double* u, const double* sigma, const do
 int tfeti_apply_F(tfeti_ctx* c, const double* x, double* y) {
   if (!c || !x || !y) return fail(c, TFETI_ERR_ARG, "null argument");
   op_F(c, x, y);
+  read_waits(c);
   sync(c);
   collect_events(c);
-  return cuda_check(c, "tfeti_apply_F");
+  const int cst = cuda_check(c, "tfeti_apply_F");
+  return cst != TFETI_OK ? cst : check_waits(c);
 }
 
 int tfeti_apply_F32(tfeti_ctx* c, const double* x, double* y) {
   if (!c || !x || !y) return fail(c, TFETI_ERR_ARG, "null argument");
   if (c->precision != TFETI_PRECISION_MIXED) return fail(c, TFETI_ERR_ARG, "FP32 F-apply needs the mixed mode");
   op_F32(c, x, y);
-  int herr = 0;
-  cudaMemcpyAsync(&herr, c->d_err, sizeof(int), cudaMemcpyDeviceToHost, c->st);
+  read_waits(c);
   sync(c);
   const int cst = cuda_check(c, "tfeti_apply_F32");
-  if (cst != TFETI_OK) return cst;
-  if (herr & 6) {
-    cudaMemsetAsync(c->d_err, 0, sizeof(int), c->st);
-    return fail(c, TFETI_ERR_TIMEOUT, "a bounded device wait gave up in the FP32 F-apply");
-  }
-  return TFETI_OK;
+  return cst != TFETI_OK ? cst : check_waits(c);
 }
 
 int tfeti_apply_projector(tfeti_ctx* c, const double* x, double* y) {
@@ -3671,8 +3704,10 @@ int tfeti_apply_projector(tfeti_ctx* c, const double* x, double* y) {
 int tfeti_apply_precond(tfeti_ctx* c, const double* x, double* y) {
   if (!c || !x || !y) return fail(c, TFETI_ERR_ARG, "null argument");
   op_precond(c, x, y);
+  read_waits(c);
   sync(c);
-  return cuda_check(c, "tfeti_apply_precond");
+  const int cst = cuda_check(c, "tfeti_apply_precond");
+  return cst != TFETI_OK ? cst : check_waits(c);
 }
 
 int tfeti_apply_N(tfeti_ctx* c, const double* x, double* y) {
@@ -3692,8 +3727,10 @@ int tfeti_apply_kdag(tfeti_ctx* c, const double* x, double* y) {
   a.out_mode = 1;
   fp64_pass(c, a);
   wood_correct_solve(c, a, c->st);
+  read_waits(c);
   sync(c);
-  return cuda_check(c, "tfeti_apply_kdag");
+  const int cst = cuda_check(c, "tfeti_apply_kdag");
+  return cst != TFETI_OK ? cst : check_waits(c);
 }
 
 int tfeti_apply_K(tfeti_ctx* c, const double* x, double* y) {

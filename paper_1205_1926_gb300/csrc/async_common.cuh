@@ -44,8 +44,12 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
   return ok != 0;
 }
 
-// Wait for phase `parity` of `bar`, giving up after `limit` SM cycles (default 2^31, ~1 s).
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = 1LL << 31) {
+constexpr long long kWaitLimit = 1LL << 31;   // SM cycles, ~1 s
+
+// Wait for phase `parity` of `bar`, giving up after `limit` SM cycles; limit 0 gives up without a look
+// (so that the way out of a kernel can be tested).
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = kWaitLimit) {
+  if (limit == 0) return false;
   if (mbar_test(bar, parity)) return true;
   const long long t0 = clock64();
   while (!mbar_test(bar, parity))
@@ -54,7 +58,8 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
 }
 
 // The same for a barrier on which stores of other CTAs of the cluster complete (cluster-scope acquire).
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, long long limit = 1LL << 31) {
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, long long limit = kWaitLimit) {
+  if (limit == 0) return false;
   auto test = [&]() {
     uint32_t ok;
     asm volatile(

@@ -32,6 +32,10 @@ __host__ __device__ inline int box_dof(const SubDev& S, int i) {
   return 3 * (a + S.nn[0] * (b + S.nn[1] * c)) + i % 3;
 }
 
+// Bits of a context's wait word (SolveArgs::err, DgArgs::err, ...): which bounded wait gave up.
+constexpr int kErrPanel = 2, kErrSchur = 4, kErrGrid = 32, kErrDigits = 64;
+constexpr int kErrWaits = kErrPanel | kErrSchur | kErrGrid | kErrDigits;
+
 constexpr int kMaxRHS = 4;     // right-hand sides one solve CTA carries
 constexpr int kSchurMinCount = 4;   // shapes with fewer subdomains never form their dual Schur block
 
@@ -190,7 +194,8 @@ struct SolveArgs {
   const SolveItem* items;
   int n_items;
   int in_mode, out_mode;
-  int* err;                    // bit 2 set if a bounded wait on a panel copy gives up
+  int* err;                    // kErrPanel set if a bounded wait gives up
+  long long wait_limit;        // of the bounded waits, in SM cycles
   int rec_max;                 // largest panel record of the launch (doubles, even)
   int npad;                    // vector stride in shared memory (largest n, even)
   int rcap;                    // vectors allocated per CTA (>= every item's count)
@@ -334,7 +339,8 @@ struct DgArgs {
   double* sA = nullptr;
   const double* sB = nullptr;
   long long* out = nullptr;
-  int* err = nullptr;                  // bit 4 set if a bounded wait gives up
+  int* err = nullptr;                  // kErrDigits set if a bounded wait gives up
+  long long wait_limit = 0;            // of those waits, in SM cycles
 };
 int dg_nk(int n);                      // stages of 16 columns
 int dg_chunk_stages();                 // K splits are multiples of this many stages

@@ -269,7 +269,7 @@ __device__ __forceinline__ void forward_rows32(const float* P, int bw, int jlo, 
 // complete.
 template <typename T, int R>
 __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __restrict__ dinv, const T* pan, int pstride,
-                     int NS, T* vec, int npad, uint64_t* bar, int* s_fail) {
+                     int NS, T* vec, int npad, uint64_t* bar, int* s_fail, long long limit) {
   const int n = S0.n_dof, bw = S0.bw, nb = S0.nb, nblk = S0.nblk, rec = S0.rec;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int nsteps = 2 * nblk;
@@ -302,7 +302,7 @@ __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __res
   int k_fail = -1, buf = 0;
   uint32_t phase = 0;
   for (int k = 0; k < nsteps; ++k) {
-    const bool ok = mbar_wait(&bar[buf], phase);
+    const bool ok = mbar_wait(&bar[buf], phase, limit);
     if (!ok) *s_fail = 1;
     const T* P = pan + buf * pstride;
     const int b = step_block(k);
@@ -444,15 +444,15 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? kThreads32 : kThreads, 1) k_s
   // the pipe also where its predicate is off (a single right-hand side took 1200 us of the four's
   // 1600 us for a 2187-dof box when all four were predicated)
   int k_fail;
-  if (R == 1) k_fail = sweep<T, 1>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
-  else if (R == 2) k_fail = sweep<T, 2>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
-  else if (R == 3) k_fail = sweep<T, 3>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
-  else k_fail = sweep<T, 4>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail);
+  if (R == 1) k_fail = sweep<T, 1>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail, a.wait_limit);
+  else if (R == 2) k_fail = sweep<T, 2>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail, a.wait_limit);
+  else if (R == 3) k_fail = sweep<T, 3>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail, a.wait_limit);
+  else k_fail = sweep<T, 4>(S0, fac, dinv, pan, a.rec_max, NS, vec, npad, bar, &s_fail, a.wait_limit);
   if (k_fail >= 0) {
     // a panel copy never completed: report, give the copies still in flight (steps k_fail ..
     // k_fail + NS - 1) a bounded time to land, and leave
     if (tid == 0) {
-      atomicOr(a.err, 2);
+      atomicOr(a.err, kErrPanel);
       for (int k = k_fail; k < k_fail + NS && k < nsteps; ++k) mbar_wait(&bar[k % NS], (uint32_t)((k / NS) & 1));
     }
     return;
@@ -589,10 +589,10 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
   // panels nor opens exchange phases any more (a phase may be opened once the one before it has completed)
   bool ok = true;
   auto wait_panel = [&](int k) {
-    if (ok) ok = mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1));
+    if (ok) ok = mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1), a.wait_limit);
   };
   auto wait_exchange = [&](int e) {
-    if (ok) ok = mbar_wait_cluster(&xbar[e % kClRing], (uint32_t)((e / kClRing) & 1));
+    if (ok) ok = mbar_wait_cluster(&xbar[e % kClRing], (uint32_t)((e / kClRing) & 1), a.wait_limit);
   };
   int issued = 0;
   if (tid == 0)
@@ -706,7 +706,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
       for (int r = 0; r < R; ++r) st_cluster(vec + r * npad + r0 + (int)q * rpc + lane, (unsigned)(b % C), zv[r]);
     if (tid == 0 && ok && issued < nsteps) fetch(issued++);
   }
-  if (!ok) atomicOr(a.err, 2);
+  if (!ok) atomicOr(a.err, kErrPanel);
   if (!ok && tid == 0)
     for (int k = max(0, issued - kClStages); k < issued; ++k)   // copies still in flight land first
       mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1));

@@ -304,7 +304,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
                                                              const DgCta* __restrict__ ctas, int full,
                                                              const unsigned char* __restrict__ A,
                                                              const unsigned char* __restrict__ B,
-                                                             long long* __restrict__ out, int* err) {
+                                                             long long* __restrict__ out, int* err,
+                                                             long long limit) {
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
   uint64_t* empty_bar = full_bar + kStages;
@@ -349,7 +350,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
       int issued = 0;
       for (int j = 0; j < n_ks; ++j) {
         const int st = j % kStages, u = j / kStages;
-        if (u > 0 && !mbar_wait(&empty_bar[st], (uint32_t)((u - 1) & 1))) {
+        if (u > 0 && !mbar_wait(&empty_bar[st], (uint32_t)((u - 1) & 1), limit)) {
           atomicOr(s_fail, 1);
           break;
         }
@@ -367,7 +368,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
     if (lane == 0) {
       bool ok = true;
       auto wait_full = [&](int j) {
-        if (!mbar_wait(&full_bar[j % kStages], (uint32_t)((j / kStages) & 1))) ok = false;
+        if (!mbar_wait(&full_bar[j % kStages], (uint32_t)((j / kStages) & 1), limit)) ok = false;
       };
       auto sa_of = [&](int j) { return smem_addr(smem + (j % kStages) * kStageBytes); };
       for (int j = 0; j < n_ks && ok; j += 2) {
@@ -388,7 +389,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
         const bool low_first = first && c > 0;
         if (low_first) {
           for (int s = j; s < j + m; ++s) issue_groups<kExact, kS>(tmem, sa_of(s), sa_of(s) + kS * kABytes, false);
-          if (!mbar_wait(drained_bar, (uint32_t)((c - 1) & 1))) {
+          if (!mbar_wait(drained_bar, (uint32_t)((c - 1) & 1), limit)) {
             ok = false;
             break;
           }
@@ -412,7 +413,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
     for (int k = 0; k < kN / 2; ++k) acc[k] = 0;
     bool ok = true;
     for (int c = 0; c < n_chunk && ok; ++c) {
-      ok = mbar_wait(exact_bar, (uint32_t)(c & 1));
+      ok = mbar_wait(exact_bar, (uint32_t)(c & 1), limit);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       fence_after();
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
   __syncwarp();
   fence_before();
   __syncthreads();
-  if (threadIdx.x == 0 && *s_fail) atomicOr(err, 4);
+  if (threadIdx.x == 0 && *s_fail) atomicOr(err, kErrDigits);
   if (warp == kEpiWarps) {
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem) : "memory");
@@ -535,7 +536,7 @@ int launch_dg_product(const DevMesh& M, const DgArgs& a, const double* src, cons
   cudaFuncSetAttribute(k_dg_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmem);
   k_dg_gemm<<<a.n_ctas, kGemmThreads, kGemmSmem, st>>>(a.blocks, a.ctas, full,
                                                        static_cast<const unsigned char*>(a.A),
-                                                       static_cast<const unsigned char*>(a.B), a.out, a.err);
+                                                       static_cast<const unsigned char*>(a.B), a.out, a.err, a.wait_limit);
   k_dg_scatter<<<a.n_rows, 256, xsm, st>>>(M, a.blocks, a.rows, full, a.out, a.sA, a.sB, cbuf, dst);
   return 3;
 }

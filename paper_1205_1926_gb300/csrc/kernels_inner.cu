@@ -41,7 +41,7 @@ __device__ __noinline__ void grid_sync(unsigned* bar, int* err) {
       unsigned long long spins = 0;
       while (*gen == g0) {
         if (++spins > kBarSpinLimit) {
-          atomicOr(err, 32);
+          atomicOr(err, kErrGrid);
           break;
         }
         __nanosleep(32);

@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(256, 1) k_schur_tc(int nk, const unsigned char
     for (int q = 0; q < 4; ++q)
       d4[q] = good ? make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
   }
-  if (threadIdx.x == 0 && s_flag[0] != 0) atomicOr(err, 4);
+  if (threadIdx.x == 0 && s_flag[0] != 0) atomicOr(err, kErrSchur);
   tc_fence_before();
   __syncthreads();
   if (warp == 0) {
