@@ -42,26 +42,39 @@ UNIT = "s/load_step"
 FP64_NOMINAL_TFLOPS = 1.25    # GB300 FP64 rate as published; the roofline uses the rate measured in the run
 
 
-def digit_product(w, boundary):
-    """Tensor-core work of one FP64 K^+ pass by the digit product (28 BF16 digit products of every box with
-    its shape's dense K^+, on all dofs or on the boundary dofs; shapes with at least 4 boxes and at most 3072
-    dofs), and whether every box takes it."""
-    count = {}
-    for k in range(len(w.cuts[2]) - 1):
-        for j in range(len(w.cuts[1]) - 1):
-            for i in range(len(w.cuts[0]) - 1):
-                a = tuple(w.cuts[d][q + 1] - w.cuts[d][q] for d, q in enumerate((i, j, k)))
-                count[a] = count.get(a, 0) + 1
-    flops, every = 0.0, True
-    for a, c in count.items():
-        n = 3 * (a[0] + 1) * (a[1] + 1) * (a[2] + 1)
-        inner = 3 * max(0, a[0] - 1) * max(0, a[1] - 1) * max(0, a[2] - 1)
-        if c < 4 or n > 3072:
-            every = False
-            continue
-        m = n - inner if boundary else n
-        flops += 28.0 * 2.0 * c * m * m
-    return flops, every
+def pass_roofline(tm, work, algo, pk, pk_kind, fp64_peak):
+    """Roofline object of the FP64 K^+ passes from the work they launched.  A pass is tensor-core work (the digit
+    product against the BF16 rate) where no box of any timed pass took the banded sweeps; else the sweeps' FP64
+    flops are set against the FP64 FMA rate, with the digit products that ran beside them given too."""
+    def rate(flops):
+        return flops / (tm["f_apply_ms_total"] * 1e-3) / 1e12 if tm["f_apply_ms_total"] > 0 else None
+
+    def frac(flops, peak):
+        return rate(flops) / peak if rate(flops) else None
+
+    n = max(work["passes"], 1)
+    fp64_kind = f"FP64 FMA rate measured in this run (tfeti_measure_fp64_fma); nominal {FP64_NOMINAL_TFLOPS}"
+    digit = {"achieved": rate(work["digit_flops"]), "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
+             "frac": frac(work["digit_flops"], pk["bf16_tflops"]), "peak_kind": f"{pk_kind} bf16_tflops"}
+    sweep = {"achieved": rate(work["banded_flops"]), "peak": fp64_peak, "unit": "TFLOP/s",
+             "frac": frac(work["banded_flops"], fp64_peak), "peak_kind": fp64_kind}
+    if work["digit_flops"] > 0 and work["banded_passes"] == 0:
+        roof = {"bound": "tensor"} | digit | {
+            "kernel": "k_dg_split_x + k_dg_gemm + k_dg_scatter (FP64 K^+ by BF16 digit products, tcgen05)"}
+    else:
+        roof = {"bound": "alu"} | sweep | {
+            "kernel": "k_solve_cl / k_sub_solve (banded sweeps, FP64)" + (
+                " beside the digit product" if work["digit_flops"] > 0 else ""),
+            "digit_product": digit if work["digit_flops"] > 0 else None}
+    return roof | {
+        "traffic": None,
+        "fp64_method": {"achieved": rate(algo["flops"] * work["passes"]), "peak": fp64_peak, "unit": "TFLOP/s",
+                        "peak_kind": fp64_kind},
+        "algorithmic": algo | {"note": "per pass: every subdomain's banded factor n (bw + 1) entries, "
+                                       "2 flops per entry and right-hand side, forward and backward sweep"},
+        "total_ms": tm["f_apply_ms_total"], "launches": tm["f_apply_launches"],
+        "avg_launch_ms": tm["f_apply_ms_total"] / n, "banded_passes": work["banded_passes"],
+        "executed_flops_per_launch": {"bf16_digit": work["digit_flops"] / n, "fp64_banded": work["banded_flops"] / n}}
 
 
 def algorithmic_fapply(w):
@@ -462,7 +475,8 @@ def run_gpu(args, rank, world, local_rank):
         barrier()
         clocks = sampler.stop() if sampler else None
         elapsed = max_over_ranks([e0.elapsed_time(e1) / 1e3], dev)[0]
-        return {"elapsed": elapsed, "infos": infos, "snaps": snaps, "tm": c.timing(), "clocks": clocks,
+        return {"elapsed": elapsed, "infos": infos, "snaps": snaps, "tm": c.timing(), "pass_work": c.pass_work(),
+                "clocks": clocks,
                 "tuning": c.tuning() if hasattr(c, "tuning") else None,
                 "deflation": c.deflation_stats() if arm == "mixed_learned_deflated" else None,
                 "woodbury": c.woodbury_stats() if arm != "fp64" else None}
@@ -520,39 +534,15 @@ def run_gpu(args, rank, world, local_rank):
     tm = main["tm"]
     # F-apply passes: K^+ of every box (the F-applies of the FP64 arm, the residual solves of the mixed
     # arms) and, with --fapply schur, the FP64 dual-Schur DGEMM.  The roofline object describes the one with
-    # the larger share of the headline arm's device time; the other sits beside it.  Where every box's shape
-    # takes the digit product (kernels_digits.cu) a pass is tensor-core work: its peak is the BF16 rate, and
-    # the method's FP64 flops over its time are given beside it.  Otherwise the banded sweeps set the time,
-    # bound by the FP64 FMA rate measured in this run.
-    algo = algorithmic_fapply(w)
-    avg_f_ms = tm["f_apply_ms_total"] / max(tm["f_apply_launches"], 1)
-    achieved_tf = algo["flops"] / (avg_f_ms * 1e-3) / 1e12 if avg_f_ms > 0 else None
-    peak_kind = (f"FP64 FMA rate measured in this run (tfeti_measure_fp64_fma); nominal {FP64_NOMINAL_TFLOPS}")
-    method = {"achieved": achieved_tf, "peak": fp64_peak, "unit": "TFLOP/s", "peak_kind": peak_kind}
-    digit_flops, all_digits = digit_product(w, boundary=main_arm == "fp64")
-    if all_digits:
-        d_tf = digit_flops / (avg_f_ms * 1e-3) / 1e12 if avg_f_ms > 0 else None
-        banded = {"bound": "tensor", "achieved": d_tf, "peak": pk["bf16_tflops"], "unit": "TFLOP/s",
-                  "frac": d_tf / pk["bf16_tflops"] if d_tf else None, "traffic": None,
-                  "kernel": "k_dg_split_x + k_dg_gemm + k_dg_scatter (FP64 K^+ by BF16 digit products, tcgen05)",
-                  "peak_kind": f"{pk_kind} bf16_tflops", "fp64_method": method}
-    else:
-        banded = {"bound": "alu", "achieved": achieved_tf, "peak": fp64_peak, "unit": "TFLOP/s",
-                  "frac": achieved_tf / fp64_peak if achieved_tf else None, "traffic": None,
-                  "kernel": "k_solve_cl / k_sub_solve (banded sweeps, FP64) beside the digit product of the shapes "
-                            "with at least 4 boxes",
-                  "peak_kind": peak_kind}
-    banded |= {"algorithmic": algo | {"note": "per pass: every subdomain's banded factor n (bw + 1) entries, "
-                                              "2 flops per entry and right-hand side, forward and backward sweep"},
-               "total_ms": tm["f_apply_ms_total"], "launches": tm["f_apply_launches"], "avg_launch_ms": avg_f_ms,
-               "executed_flops_per_launch": digit_flops if all_digits else tm["f_apply_flops"]}
+    # the larger share of the headline arm's device time; the other sits beside it.
+    banded = pass_roofline(tm, main["pass_work"], algorithmic_fapply(w), pk, pk_kind, fp64_peak)
     schur = None
     if tm["schur_launches"] > 0 and tm["schur_ms_total"] > 0:
         s_tf = tm["schur_flops_total"] / (tm["schur_ms_total"] * 1e-3) / 1e12
         schur = {"bound": "alu", "achieved": s_tf, "peak": fp64_peak, "unit": "TFLOP/s",
                  "frac": s_tf / fp64_peak, "traffic": None,
                  "kernel": "k_schur_dgemm (+ gather): Y = X S with the shape's FP64 dual Schur block",
-                 "peak_kind": peak_kind,
+                 "peak_kind": banded["fp64_method"]["peak_kind"],
                  "total_ms": tm["schur_ms_total"], "launches": tm["schur_launches"],
                  "flops_per_launch": tm["schur_flops_total"] / tm["schur_launches"],
                  "avg_launch_ms": tm["schur_ms_total"] / tm["schur_launches"]}

@@ -510,7 +510,7 @@ typedef struct tfeti_timing {
     double f_apply_ms_total;   /* summed device time of the F-apply kernel launches     */
     int64_t f_apply_launches;
     double f_apply_bytes;      /* algorithmic bytes of one F-apply                      */
-    double f_apply_flops;      /* FP64 flops of one F-apply                             */
+    double f_apply_flops;      /* FP64 flops of one F-apply with every box by banded sweeps */
     double factor_ms_total;
     int64_t factor_launches;
     int64_t kernel_launches;   /* library kernels launched since the last reset         */
@@ -527,6 +527,18 @@ typedef struct tfeti_timing {
     int64_t inner_body_runs;
 } tfeti_timing;
 int tfeti_timing_get(tfeti_ctx* ctx, tfeti_timing* out);
+
+/* Work that the passes counted in f_apply_launches launched since the last reset: the BF16 flops of
+ * the digit products (28 products of each box's row with its shape's dense K^+, on all dofs or on the
+ * boundary dofs as the pass needs), the FP64 flops of the banded sweeps of the boxes that did not take
+ * them, and the number of passes with any such box. */
+typedef struct tfeti_pass_work {
+    int64_t passes;
+    int64_t banded_passes;
+    double digit_flops;
+    double banded_flops;
+} tfeti_pass_work;
+int tfeti_timing_pass_work(tfeti_ctx* ctx, tfeti_pass_work* out);
 int tfeti_timing_reset(tfeti_ctx* ctx, int32_t enable_events);
 
 /* Failure detection of the bounded device waits (no context needed): one CTA waits on

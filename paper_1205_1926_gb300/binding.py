@@ -66,6 +66,11 @@ class Timing(C.Structure):
                 ("inner_iterations", C.c_int64), ("inner_body_runs", C.c_int64)]
 
 
+class PassWork(C.Structure):
+    _fields_ = [("passes", C.c_int64), ("banded_passes", C.c_int64), ("digit_flops", C.c_double),
+                ("banded_flops", C.c_double)]
+
+
 _P = C.c_void_p
 _D = C.c_double
 _I = C.c_int32
@@ -119,6 +124,7 @@ SIGNATURES = {
     "tfeti_apply_K": (C.c_int, [_P, _P, _P]),
     "tfeti_apply_projector_noalloc": (C.c_int, [_P, _P, _P]),
     "tfeti_timing_get": (C.c_int, [_P, C.POINTER(Timing)]),
+    "tfeti_timing_pass_work": (C.c_int, [_P, C.POINTER(PassWork)]),
     "tfeti_timing_reset": (C.c_int, [_P, _I]),
     "tfeti_check_bounded_wait": (C.c_int, [_P, C.c_int64, C.POINTER(_I)]),
     "tfeti_measure_fp64_fma": (C.c_int, [_P, _I, C.POINTER(C.c_double)]),
@@ -427,6 +433,12 @@ class Context:
         t = Timing()
         self.lib.tfeti_timing_get(self.h, C.byref(t))
         return {k: getattr(t, k) for k, _ in Timing._fields_}
+
+    def pass_work(self) -> dict:
+        """Work of the FP64 K^+ passes counted in ``f_apply_launches`` since the last reset."""
+        w = PassWork()
+        self.lib.tfeti_timing_pass_work(self.h, C.byref(w))
+        return {k: getattr(w, k) for k, _ in PassWork._fields_}
 
     def timing_reset(self, events: bool):
         self.lib.tfeti_timing_reset(self.h, 1 if events else 0)

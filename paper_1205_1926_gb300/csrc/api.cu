@@ -176,6 +176,11 @@ void sort_items_by_cost(const tfeti_ctx* c, std::vector<SolveItem>& items) {
                    [&cost](const SolveItem& a, const SolveItem& b) { return cost(a) > cost(b); });
 }
 
+// FP64 flops of a banded K^+ apply: two sweeps over the panels (nb x bw per block) and the inverted diagonal blocks.
+double banded_flops(const SubDev& s) {
+  return 4.0 * ((double)s.nblk * s.nb * s.bw + (double)s.nblk * s.nb * (s.nb + 1) / 2.0);
+}
+
 tfeti_ctx::ItemStat item_stat(const tfeti_ctx* c, const std::vector<SolveItem>& items) {
   tfeti_ctx::ItemStat s;
   double sum = 0.0, top = 0.0;
@@ -238,6 +243,7 @@ void build_item_list(tfeti_ctx* c, const std::vector<int>& plastic_count, int R,
 // results the scatter adds.  Wide shapes come first (the longest CTAs start first).
 void build_dg(tfeti_ctx* c, const std::vector<int>& plastic_count) {
   c->dg_rows = c->dg_ctas = c->dg_ctas_bd = c->dg_max_n = 0;
+  c->dg_flops = c->dg_flops_bd = 0.0;
   if (!c->dg_B) return;
   const Plan& P = c->plan;
   const int ns = (int)c->h_subs.size();
@@ -268,6 +274,8 @@ void build_dg(tfeti_ctx* c, const std::vector<int>& plastic_count) {
     tiles_bd += b.rows_pad / kDgM * (b.ld_bd / kDgN);
     for (size_t k = 0; k < by[sh].size(); ++k) rows.push_back({by[sh][k], (int)blocks.size(), (int)k, 0});
     c->dg_max_n = std::max(c->dg_max_n, b.n);
+    c->dg_flops += dg_flops((int)by[sh].size(), b.n);
+    c->dg_flops_bd += dg_flops((int)by[sh].size(), b.n_bd);
     blocks.push_back(b);
   }
   if (blocks.empty()) return;
@@ -379,6 +387,8 @@ void build_items(tfeti_ctx* c, const std::vector<int>& plastic_count) {
   build_item_list(c, plastic_count, R64_all, all);
   for (const SolveItem& it : all)
     if ((it.fac & kOwnFac) || !uses_schur(c->h_subs[it.sub[0]].shape)) pl64.push_back(it);
+  c->items_flops = 0.0;
+  for (const SolveItem& it : c->h_items) c->items_flops += it.count * banded_flops(c->h_subs[it.sub[0]]);
   c->is64 = item_stat(c, c->h_items);
   c->is32 = item_stat(c, c->h_items32);
   c->is_pl = item_stat(c, pl);
@@ -517,6 +527,8 @@ void wood_correct_end(tfeti_ctx* c, const SolveArgs& a) {
 // with digit tiles by one tensor-core product, the others (own factors, shapes without tiles) by the
 // banded sweeps, concurrently on the second stream; the items with own records wait for a deferred
 // refactorisation.  Both write their own subdomains' entries only.
+bool dg_full(const SolveArgs& a) { return a.in_mode != 0 || a.out_mode != 0; }   // else the boundary form
+
 void fp64_pass(tfeti_ctx* c, const SolveArgs& a) {
   const bool dg = c->dg_rows > 0, rest = a.n_items > 0;
   cudaStream_t sb = dg ? c->st2 : c->st;
@@ -545,7 +557,7 @@ void fp64_pass(tfeti_ctx* c, const SolveArgs& a) {
     d.blocks = c->d_dg_blocks;
     d.rows = c->d_dg_rows;
     d.n_rows = c->dg_rows;
-    d.full = a.in_mode != 0 || a.out_mode != 0;
+    d.full = dg_full(a);
     d.ctas = d.full ? c->d_dg_ctas : c->d_dg_ctas_bd;
     d.n_ctas = d.full ? c->dg_ctas : c->dg_ctas_bd;
     d.max_n = c->dg_max_n;
@@ -572,6 +584,9 @@ void timed_sub_solve(tfeti_ctx* c, const SolveArgs& a) {
   if (e1) cudaEventRecord(e1, c->st);
   if (corr) wood_correct_end(c, a);
   c->f_launches += 1;
+  c->f_digit_flops += dg_full(a) ? c->dg_flops : c->dg_flops_bd;
+  c->f_band_flops += c->items_flops;
+  c->f_band_passes += c->n_items > 0 ? 1 : 0;
 }
 
 void op_F(tfeti_ctx* c, const double* x, double* yv) {
@@ -3748,10 +3763,8 @@ int tfeti_timing_get(tfeti_ctx* c, tfeti_timing* out) {
   out->f_apply_launches = c->f_launches;
   double bytes = 0.0, flops = 0.0;
   for (const SubDev& s : c->h_subs) {
-    // two sweeps over the panels (nb x bw per block) and the inverted diagonal blocks
-    const double panel = (double)s.nblk * s.nb * s.bw, diag = (double)s.nblk * s.nb * (s.nb + 1) / 2.0;
-    bytes += 2.0 * 8.0 * (panel + (double)s.nblk * s.nb * s.nb);
-    flops += 2.0 * 2.0 * (panel + diag);
+    bytes += 2.0 * 8.0 * ((double)s.nblk * s.nb * s.bw + (double)s.nblk * s.nb * s.nb);
+    flops += banded_flops(s);
   }
   out->f_apply_bytes = bytes;
   out->f_apply_flops = flops;
@@ -3768,12 +3781,23 @@ int tfeti_timing_get(tfeti_ctx* c, tfeti_timing* out) {
   return TFETI_OK;
 }
 
+int tfeti_timing_pass_work(tfeti_ctx* c, tfeti_pass_work* out) {
+  if (!c || !out) return TFETI_ERR_ARG;
+  out->passes = c->f_launches;
+  out->banded_passes = c->f_band_passes;
+  out->digit_flops = c->f_digit_flops;
+  out->banded_flops = c->f_band_flops;
+  return TFETI_OK;
+}
+
 int tfeti_timing_reset(tfeti_ctx* c, int32_t enable_events) {
   if (!c) return TFETI_ERR_ARG;
   collect_events(c);
   c->events = enable_events != 0;
   c->f_ms = c->factor_ms = 0.0;
   c->f_launches = c->factor_launches = c->launches = 0;
+  c->f_digit_flops = c->f_band_flops = 0.0;
+  c->f_band_passes = 0;
   c->g_ms = c->g_flops = c->g_bytes = 0.0;
   c->g_launches = 0;
   c->inner_ms = 0.0;

@@ -108,6 +108,7 @@ struct tfeti_ctx {
   tfeti::DgRow* d_dg_rows = nullptr;
   tfeti::DgCta *d_dg_ctas = nullptr, *d_dg_ctas_bd = nullptr;
   int dg_rows = 0, dg_ctas = 0, dg_ctas_bd = 0, dg_max_n = 0;
+  double dg_flops = 0.0, dg_flops_bd = 0.0;  // digit products of the rows, full and boundary form
   std::vector<char> h_wood;                  // per subdomain: on the Woodbury correction
   std::vector<int> h_np_all;                 // plastic points per subdomain at the last assembly
   tfeti::WoodArgs wood;
@@ -297,5 +298,8 @@ struct tfeti_ctx {
   long long inner_its = 0, inner_runs = 0;         // their PCGP iterations and body runs
   double f_ms = 0.0, factor_ms = 0.0;
   long long f_launches = 0, factor_launches = 0, launches = 0;
+  // work of the counted FP64 passes: digit products, banded sweeps, passes with any of the latter
+  double f_digit_flops = 0.0, f_band_flops = 0.0, items_flops = 0.0;
+  long long f_band_passes = 0;
   std::vector<int> last_refactored;
 };

@@ -344,6 +344,7 @@ struct DgArgs {
 };
 int dg_nk(int n);                      // stages of 16 columns
 int dg_chunk_stages();                 // K splits are multiples of this many stages
+double dg_flops(int rows, int n);      // of the digit products of rows x n with n x n
 long long dg_a_elems(int rows_pad, int n);
 long long dg_b_elems(int n);
 // Digit tiles and row scales of one shape's K^+ (full) or S, from its dense kinv (set-up).

@@ -516,6 +516,7 @@ __global__ void __launch_bounds__(256) k_dg_scatter(DevMesh M, const DgBlock* __
 
 int dg_nk(int n) { return (n + kK - 1) / kK; }
 int dg_chunk_stages() { return kChunk; }
+double dg_flops(int rows, int n) { return 2.0 * (kS * (kS + 1) / 2) * (double)rows * n * n; }
 long long dg_a_elems(int rows_pad, int n) { return (long long)rows_pad * dg_nk(n) * kK * kS; }
 long long dg_b_elems(int n) { return (long long)((n + kN - 1) / kN) * kN * dg_nk(n) * kK * kS; }
 
