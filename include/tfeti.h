@@ -108,8 +108,8 @@ typedef struct tfeti_problem {
  * doubles, 4.8 GB at 4096 subdomains) applied by one GEMV.  PLANES: G G^T is block
  * tridiagonal over the planes of subdomains with equal z index (a subdomain couples
  * only to the boxes around it); its block LDL^T with explicit inverses of the pivot
- * blocks, eliminated from both ends, is applied by nz + 1 dependent GEMVs of (6 nx ny)^2, nz planes of nx x ny
- * subdomains (3 x 16 x 1536^2 doubles = 0.9 GB at 16^3 subdomains).  Both give H g to
+ * blocks, eliminated from both ends, is applied by nz (odd) or nz + 1 (even) dependent
+ * GEMVs of (6 nx ny)^2, nz planes of nx x ny subdomains (3 x 16 x 1536^2 doubles = 0.9 GB at 16^3 subdomains).  Both give H g to
  * rounding. */
 #define TFETI_COARSE_AUTO   0
 #define TFETI_COARSE_DENSE  1
@@ -393,9 +393,11 @@ int tfeti_mlp_train(tfeti_ctx* ctx, const double* la, const double* lb, const do
  * shape's elastic tangent (Sec. 4.2 leaves the K^+ apply open).  BANDED (default):
  * forward and backward substitution with the shape's factor or, for shapes with at least four
  * subdomains and at most 3072 dofs, the product with the shape's dense K^+ (formed at set-up from
- * the same factor) on the tensor cores, both operands split into integer digits so that the
- * product has FP64 accuracy; the other FP64 K^+ applies (residuals, recovery, tfeti_apply_kdag)
- * take the same path in either mode.  SCHUR: one DGEMM per
+ * the same factor) on the tensor cores, both operands split into integer digits of 55 bits
+ * below the largest entry of each subdomain's vector and of each row of K^+: the error of entry i
+ * of a subdomain of n dofs is of the order of n 2^-54 max|x| max_j |K^+_ij| (norm-wise, as the banded
+ * solve's; entries of x below 2^-56 of the subdomain's largest do not count).  The other FP64 K^+ applies
+ * (residuals, recovery, tfeti_apply_kdag) take the same path in either mode.  SCHUR: one DGEMM per
  * shape with the shape's dual Schur block S = (K^+)_{boundary,boundary} (formed once
  * in FP64 from the same factor, 1158^2 doubles for an 8^3 box), which has the same
  * flop count but keeps all SMs busy; subdomains with plastic points keep their
@@ -494,8 +496,8 @@ int tfeti_apply_K(tfeti_ctx* ctx, const double* x, double* y);
  *   it makes that device current for its duration and then restores the
  *   caller's current device.
  * - The first call for a device resolves the array's device address on that
- *   device with cudaGetSymbolAddress; make that first call before any stream
- *   capture.
+ *   device with cudaGetSymbolAddress.  No call can be part of a stream capture:
+ *   each one synchronises its stream.
  * - All calls on a device share the array: calls whose kernels overlap on the
  *   GPU race.  Both work vectors are overwritten before they are read, so no
  *   clearing is needed between calls.

@@ -377,9 +377,9 @@ void launch_lumped(const DevMesh& M, const double* w, const double* kbb, const l
 // inverse H (l x l, and its FP32 copy H32 with rows padded to h32_ld(l)), one GEMV.  Planes:
 // G G^T is block tridiagonal over the planes of subdomains with equal z index (a subdomain
 // couples only to the 26 boxes around it), n_planes blocks of n_pl = 6 x (subdomains per
-// plane); a block LDL^T with explicit inverses W_k of the pivots and the products V_k, U_k
-// eliminating from both ends at once, turns the solve into n_planes + 1 dependent launches of n_pl x n_pl
-// GEMVs (coarse_planes_factor).
+// plane); a block LDL^T with explicit inverses W_k of the pivots and the products V_k, U_k,
+// eliminating from both ends at once, turns the solve into n_planes (odd) or n_planes + 1 (even) dependent
+// launches of n_pl x n_pl GEMVs (coarse_planes_factor).
 constexpr int kCoarseDense = 0, kCoarsePlanes = 1;
 constexpr long long kCoarseDenseMax = 6144;   // TFETI_COARSE_AUTO: dense H up to this n_coarse
 struct CoarseOp {

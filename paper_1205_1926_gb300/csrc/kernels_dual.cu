@@ -856,8 +856,8 @@ __global__ void k_coarse_assemble_planes(DevMesh M, const int* __restrict__ pair
 }
 
 // Apply of the plane solver (H = (G G^T)^-1 by a block LDL^T over the planes that eliminates from both
-// ends towards the middle plane m, so that the two ends' steps run side by side: n_planes + 1 dependent
-// launches instead of 2 n_planes - 1 from one end): first y_k = alpha W_k x_k for every plane (blockIdx.y =
+// ends towards the middle plane m, so that the two ends' steps run side by side: n_planes (odd) or n_planes + 1 (even)
+// dependent launches instead of 2 n_planes - 1 from one end): first y_k = alpha W_k x_k for every plane (blockIdx.y =
 // k), then y_k -= V_k y_{k-1} for k = 1..m-1 beside y_k -= U_k y_{k+1} for k = n_planes-2..m+1, the middle
 // plane y_m -= V_m y_{m-1} + U_m y_{m+1}, and back out, y_k -= U_k y_{k+1} for k = m-1..0 beside y_k -=
 // V_k y_{k-1} for k = m+1..n_planes-1.
