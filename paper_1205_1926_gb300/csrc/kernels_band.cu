@@ -801,7 +801,9 @@ bool launch_cl(const DevMesh& M, const SolveArgs& a, int C, cudaStream_t st) {
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_solve_cl<R>, M, a) == cudaSuccess;
+  if (cudaLaunchKernelEx(&cfg, k_solve_cl<R>, M, a) == cudaSuccess) return true;
+  cudaGetLastError();   // this launch's error, not one of an earlier call
+  return false;
 }
 
 }  // namespace
@@ -847,7 +849,7 @@ void launch_band_chol(const DevMesh& M, const int* sub_list, int n_list, const l
   cudaFuncSetAttribute(k_band_chol, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   const bool big = cudaFuncSetAttribute(k_band_chol, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
                    cudaSuccess;
-  cudaGetLastError();
+  if (!big) cudaGetLastError();
   // cluster size: the largest power of two with n_list * C <= 2 * n_sm (at most 16, or 8 if
   // non-portable cluster sizes are unavailable); 54 boxes of 8^3 elements take 17.4 ms with 4 CTAs each,
   // 19.8 ms with 8
@@ -900,7 +902,6 @@ void launch_sub_solve(const DevMesh& M, const SolveArgs& args, cudaStream_t st) 
     while (C > 1 && a.n_eff * C > 2 * n_sm) C /= 2;
     if (C > 1) {
       if (a.max_count == 1 ? launch_cl<1>(M, a, C, st) : launch_cl<2>(M, a, C, st)) return;
-      cudaGetLastError();
     }
   }
   // One CTA per item.  A step's panel (35 KB in FP32 for an 8^3 box) takes about a microsecond from

@@ -1348,8 +1348,10 @@ static void plane_apply(const T* W, const T* V, const T* U, int n, int np, const
   const size_t smem = sizeof(T) * (size_t)n;
   const long long blk = (long long)n * n;
   if (smem > 48 * 1024) {
-    cudaFuncSetAttribute(k_plane_first<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_plane_step<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static const int lim_first = dyn_smem_limit((const void*)k_plane_first<T>);
+    static const int lim_step = dyn_smem_limit((const void*)k_plane_step<T>);
+    cudaFuncSetAttribute(k_plane_first<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim_first);
+    cudaFuncSetAttribute(k_plane_step<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim_step);
   }
   k_plane_first<T><<<dim3(rb, (unsigned)np), 256, smem, st>>>(W, n, x, alpha, y, y8, np == 1 ? 1 : 0);
   const int m = np / 2;

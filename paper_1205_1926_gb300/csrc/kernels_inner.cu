@@ -432,7 +432,9 @@ size_t inner_smem(const InnerArgs& a) {
 }
 
 int inner_grid(int n_sm, size_t smem) {
-  if (cudaFuncSetAttribute(k_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+  static const int lim = dyn_smem_limit((const void*)k_inner);
+  if (smem > (size_t)lim) return 0;
+  if (cudaFuncSetAttribute(k_inner, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }

@@ -566,7 +566,8 @@ void launch_wood_setup(const DevMesh& M, const WoodArgs& a, cudaStream_t st) {
   k_wood_Zb32<<<dim3((unsigned)a.n, (unsigned)((rmax + 7) / 8)), 256, 0, st>>>(M, a);
   cudaMemcpyAsync(a.y_pool, a.z_pool, sizeof(float) * (size_t)a.z_total, cudaMemcpyDeviceToDevice, st);
   const size_t smem = sizeof(float) * (size_t)rmax * kBlk;
-  cudaFuncSetAttribute(k_wood_subst, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  static const int lim = dyn_smem_limit((const void*)k_wood_subst);
+  cudaFuncSetAttribute(k_wood_subst, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   k_wood_subst<<<dim3((unsigned)a.n, (unsigned)((a.max_bd + kBlk - 1) / kBlk)), 256, smem, st>>>(M.subs, a);
 }
 
