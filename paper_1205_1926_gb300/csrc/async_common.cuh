@@ -46,10 +46,8 @@ __device__ __forceinline__ bool mbar_test(uint64_t* bar, uint32_t parity) {
 
 constexpr long long kWaitLimit = 1LL << 31;   // SM cycles, ~1 s
 
-// Wait for phase `parity` of `bar`, giving up after `limit` SM cycles; limit 0 gives up without a look
-// (so that the way out of a kernel can be tested).
+// Wait for phase `parity` of `bar`, giving up after `limit` SM cycles.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long long limit = kWaitLimit) {
-  if (limit == 0) return false;
   if (mbar_test(bar, parity)) return true;
   const long long t0 = clock64();
   while (!mbar_test(bar, parity))
@@ -59,7 +57,6 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
 
 // The same for a barrier on which stores of other CTAs of the cluster complete (cluster-scope acquire).
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, long long limit = kWaitLimit) {
-  if (limit == 0) return false;
   auto test = [&]() {
     uint32_t ok;
     asm volatile(

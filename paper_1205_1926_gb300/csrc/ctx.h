@@ -282,8 +282,9 @@ struct tfeti_ctx {
   double *partial = nullptr, *sc = nullptr, *h_sc = nullptr;
   int* d_ctr = nullptr;                      // arrival counters of the fused inner-iteration kernels
   int* d_dot_ctr = nullptr;                  // and of the dot products
-  int* d_err = nullptr;                      // wait word: which bounded waits gave up (kErr..., zero between calls)
-  int* h_err = nullptr;                      // its pinned copy
+  // wait word: which bounded waits gave up (kErr..., zero between calls), in mapped host memory, and its
+  // device address
+  int *h_err = nullptr, *d_err = nullptr;
   int* d_piv = nullptr;                      // pivots of the factorisations on the context stream
   long long wait_limit = 1LL << 31;          // of the bounded waits of the banded solves and the digit product, SM cycles
   int max_copy = 0;

@@ -302,7 +302,7 @@ __device__ int sweep(const SubDev& S0, const T* __restrict__ fac, const T* __res
   int k_fail = -1, buf = 0;
   uint32_t phase = 0;
   for (int k = 0; k < nsteps; ++k) {
-    const bool ok = mbar_wait(&bar[buf], phase, limit);
+    const bool ok = limit != 0 && mbar_wait(&bar[buf], phase, limit);
     if (!ok) *s_fail = 1;
     const T* P = pan + buf * pstride;
     const int b = step_block(k);
@@ -587,7 +587,7 @@ __device__ void cl_solve(const DevMesh& M, const SolveArgs& a, const SolveItem& 
   };
   // after a wait that gave up, the remaining steps run through without waiting; thread 0 then neither fetches
   // panels nor opens exchange phases any more (a phase may be opened once the one before it has completed)
-  bool ok = true;
+  bool ok = a.wait_limit != 0;
   auto wait_panel = [&](int k) {
     if (ok) ok = mbar_wait(&bar[k % kClStages], (uint32_t)((k / kClStages) & 1), a.wait_limit);
   };

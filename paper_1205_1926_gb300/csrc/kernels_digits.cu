@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
   const int nk = full ? blk.nk : blk.nk_bd;
   const int n_ks = cta.ks1 - cta.ks0;
   const int n_chunk = (n_ks + kChunk - 1) / kChunk;
+  auto wait = [limit](uint64_t* bar, uint32_t parity) { return limit != 0 && mbar_wait(bar, parity, limit); };
 
   if (threadIdx.x == 0) {
     for (int q = 0; q < kStages; ++q) {
@@ -350,7 +351,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
       int issued = 0;
       for (int j = 0; j < n_ks; ++j) {
         const int st = j % kStages, u = j / kStages;
-        if (u > 0 && !mbar_wait(&empty_bar[st], (uint32_t)((u - 1) & 1), limit)) {
+        if (u > 0 && !wait(&empty_bar[st], (uint32_t)((u - 1) & 1))) {
           atomicOr(s_fail, 1);
           break;
         }
@@ -368,7 +369,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
     if (lane == 0) {
       bool ok = true;
       auto wait_full = [&](int j) {
-        if (!mbar_wait(&full_bar[j % kStages], (uint32_t)((j / kStages) & 1), limit)) ok = false;
+        if (!wait(&full_bar[j % kStages], (uint32_t)((j / kStages) & 1))) ok = false;
       };
       auto sa_of = [&](int j) { return smem_addr(smem + (j % kStages) * kStageBytes); };
       for (int j = 0; j < n_ks && ok; j += 2) {
@@ -389,7 +390,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
         const bool low_first = first && c > 0;
         if (low_first) {
           for (int s = j; s < j + m; ++s) issue_groups<kExact, kS>(tmem, sa_of(s), sa_of(s) + kS * kABytes, false);
-          if (!mbar_wait(drained_bar, (uint32_t)((c - 1) & 1), limit)) {
+          if (!wait(drained_bar, (uint32_t)((c - 1) & 1))) {
             ok = false;
             break;
           }
@@ -413,7 +414,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) k_dg_gemm(const DgBlock* __re
     for (int k = 0; k < kN / 2; ++k) acc[k] = 0;
     bool ok = true;
     for (int c = 0; c < n_chunk && ok; ++c) {
-      ok = mbar_wait(exact_bar, (uint32_t)(c & 1), limit);
+      ok = wait(exact_bar, (uint32_t)(c & 1));
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       fence_after();
