@@ -64,7 +64,7 @@ static_assert(sizeof(GroupDev) % 16 == 0 && offsetof(GroupDev, dirichlet) == 12,
 // row).  Almost every slot has one entry (copies shared by two subdomains, Dirichlet rows), so (B^T x) costs one
 // coalesced 16-byte load and one gather of x instead of the chain slot -> group number -> header of an 80-byte group
 // record -> x and the Helmert table.  Latency and load sectors bound these gathers: 1728 boxes of 8^3, splitting of
-// B^T lambda 59 -> 45 us; 512 boxes, FP32 lumped preconditioner 29.4 -> 26.7 us, operand gather 13.2 -> 10.1 us.
+// B^T lambda 61 -> 49 us; 512 boxes, FP32 lumped preconditioner 37.5 -> 34.2 us, operand gather 12.5 -> 10.2 us.
 struct alignas(16) SlotRow {
   int row, rest;
   double c;
@@ -72,7 +72,7 @@ struct alignas(16) SlotRow {
 
 // Row of B: its first two copy slots (s1 = -1: a Dirichlet row, one slot), its Helmert number r and its group, whose
 // record holds the further slots of a row with r > 1.  (B v)[row] of the usual two-slot row is one coalesced load and
-// two gathers: B v over 1728 boxes of 8^3 22.1 -> 14.0 us, over 512 boxes 8.0 -> 6.8 us.
+// two gathers: B v over 1728 boxes of 8^3 22.2 -> 13.5 us, over 512 boxes 8.1 -> 6.9 us.
 struct alignas(16) RowSlots {
   int s0, s1, r, group;
 };
