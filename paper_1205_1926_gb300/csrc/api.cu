@@ -1280,7 +1280,8 @@ int tune_schur_threshold(tfeti_ctx* c) {
   c->schur_threshold = best_t;
   for (size_t sh = 0; sh < nsh; ++sh) c->schur_use[sh] = c->schur_formed[sh] && count[sh] >= best_t;
   build_items(c, np);
-  return cuda_check(c, "tuning the inner F-apply");
+  const int cst = cuda_check(c, "tuning the inner F-apply");
+  return cst != TFETI_OK ? cst : check_waits(c);   // of the timed applies, synchronised above
 }
 
 void op_project(tfeti_ctx* c, const double* x, double* out) {

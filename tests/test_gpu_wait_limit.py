@@ -100,6 +100,33 @@ def test_load_step_reports_and_recovers():
     assert torch.equal(u0, u1)
 
 
+def test_precision_change_reports_and_recovers():
+    w = cube(2, 4)
+    ctx, other = T.Context(w), T.Context(w)
+    n = ctx.sizes["n_dof"]
+    f, u0, u1 = new(n), new(n), new(n)
+    ctx.traction_load((1.0, 0.2, 0.3), f)
+    ctx.set_wait_limit(0)
+    with pytest.raises(T.TfetiError) as e:
+        ctx.set_precision(True, 1e-4)
+    assert e.value.status == TIMEOUT
+    ctx.set_wait_limit()
+    for c, u in ((ctx, u0), (other, u1)):
+        c.set_precision(True, 1e-4)
+        c.set_schur_threshold(4)
+        c.assemble_tangent(new(n), f)
+        c.dual_pcg(f, u, rtol=1e-10)
+    assert torch.equal(u0, u1)
+    ctx.set_wait_limit(0)
+    with pytest.raises(T.TfetiError) as e:
+        ctx.set_schur_threshold(0)        # times the applies, banded ones among them
+    assert e.value.status == TIMEOUT
+    ctx.set_wait_limit()
+    ctx.set_schur_threshold(4)
+    ctx.dual_pcg(f, u1, rtol=1e-10)
+    assert torch.equal(u0, u1)
+
+
 def test_limits_refused():
     ctx = T.Context(cube(2, 2))
     for cycles in (-1, (1 << 31) + 1):
